@@ -49,6 +49,8 @@ struct lbm_ctx {
     int fused_threads = 256;  // threads per CTA of that kernel (32 x 8 or 32 x 16)
     int sms = 0;
     int* status = nullptr;  // device status word written by bounded waits
+    cudaGraphExec_t step_graph[2] = {nullptr, nullptr};  // STEP_GRAPH steps starting from buf[0] / buf[1]
+    int step_graph_shape[6] = {-1, -1, -1, -1, -1, -1};  // launch shape the graphs were captured with
     std::string err;
     bool owns = true;            // false for the per-domain views of a batch
     lbm_ctx* parent = nullptr;   // the batch a view belongs to
