@@ -549,7 +549,7 @@ lbm_status lbm_batch_create(lbm_ctx** out, int ndomains, const lbm_grid* grids, 
     // rest state for every domain
     for (int d = 0; d < ndomains && e == cudaSuccess; ++d) {
         lbm_ctx* v = B->views[d];
-        for (int z0 = 0; z0 < v->box.nz && e == cudaSuccess; ++z0) e = lbm_internal_init_slab(v, z0, 1, true);
+        e = lbm_internal_init_rest(v);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {

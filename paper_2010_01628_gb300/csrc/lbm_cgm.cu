@@ -76,24 +76,23 @@ __global__ void __launch_bounds__(256) cgm_collide_kernel(const S* __restrict__ 
 }
 
 template <typename S, typename C>
-__global__ void cgm_init_kernel(S* __restrict__ dst, const double* __restrict__ slab, CgmArgs p, int z0, int nzs,
+__global__ void cgm_init_kernel(S* __restrict__ dst, FieldsIn in, CgmArgs p, int z0, int nzs,
                                 bool uniform) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, zs = blockIdx.z;
     const Box& b = p.box;
     if (x >= b.nx || zs >= nzs) return;
-    const size_t m = (size_t)b.nx * b.ny * nzs;
     const size_t k = ((size_t)zs * b.ny + y) * b.nx + x;
     const uint32_t self = ((uint32_t)(z0 + zs) * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     double rho = 1.0, ph = -1.0;
     CgmNode<C> s;
     s.ux = s.uy = s.uz = (C)0;
     if (!uniform) {
-        rho = slab[k];
-        ph = slab[4 * m + k];
-        s.ux = (C)slab[m + k];
-        s.uy = (C)slab[2 * m + k];
-        s.uz = (C)slab[3 * m + k];
+        rho = in.rho[k];
+        ph = in.phase[k];
+        s.ux = (C)in.value(in.u[0], k);
+        s.uy = (C)in.value(in.u[1], k);
+        s.uz = (C)in.value(in.u[2], k);
     }
     const double rr = rho * (1.0 + ph) * 0.5, rb = rho * (1.0 - ph) * 0.5;
     s.rho_r = (C)rr;
@@ -134,13 +133,12 @@ __global__ void cgm_init_kernel(S* __restrict__ dst, const double* __restrict__ 
 }
 
 template <typename S, typename C, bool WALLS>
-__global__ void cgm_fields_kernel(const S* __restrict__ src, double* __restrict__ slab, CgmArgs p, int z0, int nzs) {
+__global__ void cgm_fields_kernel(const S* __restrict__ src, FieldsOut out, CgmArgs p, int z0, int nzs) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, zs = blockIdx.z;
     const Box& b = p.box;
     if (x >= b.nx || zs >= nzs) return;
     const int z = z0 + zs;
-    const size_t m = (size_t)b.nx * b.ny * nzs;
     const size_t k = ((size_t)zs * b.ny + y) * b.nx + x;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
@@ -148,11 +146,11 @@ __global__ void cgm_fields_kernel(const S* __restrict__ src, double* __restrict_
     cgm_pull_all<S, C, WALLS>(src, b, q, x, y, z, self, f, r);
     const Moments<C> mo = moments19(f);
     const CgmNode<C> s = cgm_macro<C>(f, mo, colour_sum(r), p);
-    slab[k] = (double)s.rho;
-    slab[m + k] = (double)s.ux;
-    slab[2 * m + k] = (double)s.uy;
-    slab[3 * m + k] = (double)s.uz;
-    slab[4 * m + k] = (double)((s.rho_r - s.rho_b) / s.rho);
+    if (out.rho) out.rho[k] = (double)s.rho;
+    if (out.u[0]) out.u[0][k] = (double)s.ux;
+    if (out.u[1]) out.u[1][k] = (double)s.uy;
+    if (out.u[2]) out.u[2][k] = (double)s.uz;
+    if (out.phase) out.phase[k] = (double)((s.rho_r - s.rho_b) / s.rho);
 }
 
 template <typename S, typename C, bool WALLS>
@@ -223,22 +221,22 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
 }
 
 template <typename S, typename C>
-static cudaError_t init_t(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform) {
+static cudaError_t init_t(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform) {
     const int bx = c->block_x;
     dim3 grid((unsigned)((c->box.nx + bx - 1) / bx), (unsigned)c->box.ny, (unsigned)nzs);
-    cgm_init_kernel<S, C><<<grid, bx, 0, c->stream>>>((S*)c->buf[c->cur], slab, cgm_args(c), z0, nzs, uniform);
+    cgm_init_kernel<S, C><<<grid, bx, 0, c->stream>>>((S*)c->buf[c->cur], in, cgm_args(c), z0, nzs, uniform);
     return cudaGetLastError();
 }
 
 template <typename S, typename C>
-static cudaError_t fields_t(lbm_ctx* c, double* slab, int z0, int nzs) {
+static cudaError_t fields_t(lbm_ctx* c, const FieldsOut& out, int z0, int nzs) {
     const CgmArgs p = cgm_args(c);
     const int bx = c->block_x;
     dim3 grid((unsigned)((c->box.nx + bx - 1) / bx), (unsigned)c->box.ny, (unsigned)nzs);
     if ((c->box.periodic & 7u) != 7u)
-        cgm_fields_kernel<S, C, true><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], slab, p, z0, nzs);
+        cgm_fields_kernel<S, C, true><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], out, p, z0, nzs);
     else
-        cgm_fields_kernel<S, C, false><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], slab, p, z0, nzs);
+        cgm_fields_kernel<S, C, false><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], out, p, z0, nzs);
     return cudaGetLastError();
 }
 
@@ -259,12 +257,12 @@ static cudaError_t reduce_t(lbm_ctx* c, bool record) {
 cudaError_t cgm_step(lbm_ctx* c, long n, bool dry) {
     return c->prec == LBM_FP64 ? step_t<double, double>(c, n, dry) : step_t<float, float>(c, n, dry);
 }
-cudaError_t cgm_init(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform) {
-    return c->prec == LBM_FP64 ? init_t<double, double>(c, slab, z0, nzs, uniform)
-                               : init_t<float, float>(c, slab, z0, nzs, uniform);
+cudaError_t cgm_init(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform) {
+    return c->prec == LBM_FP64 ? init_t<double, double>(c, in, z0, nzs, uniform)
+                               : init_t<float, float>(c, in, z0, nzs, uniform);
 }
-cudaError_t cgm_fields(lbm_ctx* c, double* slab, int z0, int nzs) {
-    return c->prec == LBM_FP64 ? fields_t<double, double>(c, slab, z0, nzs) : fields_t<float, float>(c, slab, z0, nzs);
+cudaError_t cgm_fields(lbm_ctx* c, const FieldsOut& out, int z0, int nzs) {
+    return c->prec == LBM_FP64 ? fields_t<double, double>(c, out, z0, nzs) : fields_t<float, float>(c, out, z0, nzs);
 }
 cudaError_t cgm_reduce(lbm_ctx* c, bool record) {
     return c->prec == LBM_FP64 ? reduce_t<double, double>(c, record) : reduce_t<float, float>(c, record);

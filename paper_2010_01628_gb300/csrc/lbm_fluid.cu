@@ -410,24 +410,23 @@ __global__ void __launch_bounds__(256, 4) fluid_step_tma_kernel(const S* __restr
     }
 }
 
-// Equilibrium initialisation of a z-slab from FP64 fields (rho, ux, uy, uz
-// planes of nx*ny*nzs values), or of the uniform rest state.
+// Equilibrium initialisation of nzs z-planes from FP64 fields, or of the
+// uniform rest state.
 template <typename S, typename C>
-__global__ void fluid_init_kernel(S* __restrict__ dst, const double* __restrict__ slab, Box b, int z0, int nzs,
+__global__ void fluid_init_kernel(S* __restrict__ dst, FieldsIn in, Box b, int z0, int nzs,
                                   bool uniform) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, zs = blockIdx.z;
     if (x >= b.nx || zs >= nzs) return;
-    const size_t m = (size_t)b.nx * b.ny * nzs;
     const size_t k = ((size_t)zs * b.ny + y) * b.nx + x;
     const uint32_t self = ((uint32_t)(z0 + zs) * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     C rho = (C)1, drho = (C)0, ux = (C)0, uy = (C)0, uz = (C)0;
     if (!uniform) {
-        drho = (C)(slab[k] - 1.0);  // the shift is taken in FP64
-        rho = (C)slab[k];
-        ux = (C)slab[m + k];
-        uy = (C)slab[2 * m + k];
-        uz = (C)slab[3 * m + k];
+        drho = (C)(in.rho[k] - 1.0);  // the shift is taken in FP64
+        rho = (C)in.rho[k];
+        ux = (C)in.value(in.u[0], k);
+        uy = (C)in.value(in.u[1], k);
+        uz = (C)in.value(in.u[2], k);
     }
     C f[Q];
     equilibrium_shifted<C>(rho, drho, ux, uy, uz, f);
@@ -438,14 +437,13 @@ __global__ void fluid_init_kernel(S* __restrict__ dst, const double* __restrict_
 // Moments of the gathered state for a z-slab: rho, u (with +F/2).  REG: the
 // regularized walls' rebuilt populations on the wall rows.
 template <typename S, typename C, bool WALLS, bool REG = false>
-__global__ void fluid_fields_kernel(const S* __restrict__ src, double* __restrict__ slab, FluidArgs p, int z0,
+__global__ void fluid_fields_kernel(const S* __restrict__ src, FieldsOut out, FluidArgs p, int z0,
                                     int nzs) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, zs = blockIdx.z;
     const Box& b = p.box;
     if (x >= b.nx || zs >= nzs) return;
     const int z = z0 + zs;
-    const size_t m = (size_t)b.nx * b.ny * nzs;
     const size_t k = ((size_t)zs * b.ny + y) * b.nx + x;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
@@ -456,10 +454,10 @@ __global__ void fluid_fields_kernel(const S* __restrict__ src, double* __restric
         gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
     const Moments<C> mo = moments19(f);
     const Macro<C> a = fluid_macro(mo, (C)p.g[0], (C)p.g[1], (C)p.g[2]);
-    slab[k] = (double)a.rho;
-    slab[m + k] = (double)a.ux;
-    slab[2 * m + k] = (double)a.uy;
-    slab[3 * m + k] = (double)a.uz;
+    if (out.rho) out.rho[k] = (double)a.rho;
+    if (out.u[0]) out.u[0][k] = (double)a.ux;
+    if (out.u[1]) out.u[1][k] = (double)a.uy;
+    if (out.u[2]) out.u[2][k] = (double)a.uz;
 }
 
 template <typename S, typename C, bool WALLS, bool REG = false>
@@ -553,6 +551,7 @@ static cudaError_t launch_tma(lbm_ctx* c, const S* src, S* dst, const FluidArgs&
     if (grid > rows) grid = rows;
     int block = ((c->box.nx + 31) / 32) * 32;
     if (block > 256) block = 256;
+    c->bounded_waits = true;
     fluid_step_tma_kernel<S, C, WALLS><<<(unsigned)grid, block, smem, c->stream>>>(src, dst, p, stages, c->status);
     return cudaSuccess;
 }
@@ -638,24 +637,24 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
 }
 
 template <typename S, typename C>
-static cudaError_t init_t(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform) {
+static cudaError_t init_t(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform) {
     const int bx = c->block_x;
     dim3 grid((unsigned)((c->box.nx + bx - 1) / bx), (unsigned)c->box.ny, (unsigned)nzs);
-    fluid_init_kernel<S, C><<<grid, bx, 0, c->stream>>>((S*)c->buf[c->cur], slab, c->box, z0, nzs, uniform);
+    fluid_init_kernel<S, C><<<grid, bx, 0, c->stream>>>((S*)c->buf[c->cur], in, c->box, z0, nzs, uniform);
     return cudaGetLastError();
 }
 
 template <typename S, typename C>
-static cudaError_t fields_t(lbm_ctx* c, double* slab, int z0, int nzs) {
+static cudaError_t fields_t(lbm_ctx* c, const FieldsOut& out, int z0, int nzs) {
     const FluidArgs p = fluid_args(c);
     const int bx = c->block_x;
     dim3 grid((unsigned)((c->box.nx + bx - 1) / bx), (unsigned)c->box.ny, (unsigned)nzs);
     if (c->grid.wall_model == LBM_WALL_REGULARIZED)
-        fluid_fields_kernel<S, C, true, true><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], slab, p, z0, nzs);
+        fluid_fields_kernel<S, C, true, true><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], out, p, z0, nzs);
     else if ((c->box.periodic & 7u) != 7u)
-        fluid_fields_kernel<S, C, true><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], slab, p, z0, nzs);
+        fluid_fields_kernel<S, C, true><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], out, p, z0, nzs);
     else
-        fluid_fields_kernel<S, C, false><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], slab, p, z0, nzs);
+        fluid_fields_kernel<S, C, false><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], out, p, z0, nzs);
     return cudaGetLastError();
 }
 
@@ -685,21 +684,21 @@ cudaError_t fluid_step(lbm_ctx* c, long n, bool dry) {
     }
     return cudaErrorInvalidValue;
 }
-cudaError_t fluid_init(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform) {
+cudaError_t fluid_init(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform) {
     switch (c->prec) {
-        case LBM_FP64: return init_t<double, double>(c, slab, z0, nzs, uniform);
-        case LBM_FP32: return init_t<float, float>(c, slab, z0, nzs, uniform);
-        case LBM_FP16_SHIFTED: return init_t<__half, float>(c, slab, z0, nzs, uniform);
-        case LBM_BF16_SHIFTED: return init_t<__nv_bfloat16, float>(c, slab, z0, nzs, uniform);
+        case LBM_FP64: return init_t<double, double>(c, in, z0, nzs, uniform);
+        case LBM_FP32: return init_t<float, float>(c, in, z0, nzs, uniform);
+        case LBM_FP16_SHIFTED: return init_t<__half, float>(c, in, z0, nzs, uniform);
+        case LBM_BF16_SHIFTED: return init_t<__nv_bfloat16, float>(c, in, z0, nzs, uniform);
     }
     return cudaErrorInvalidValue;
 }
-cudaError_t fluid_fields(lbm_ctx* c, double* slab, int z0, int nzs) {
+cudaError_t fluid_fields(lbm_ctx* c, const FieldsOut& out, int z0, int nzs) {
     switch (c->prec) {
-        case LBM_FP64: return fields_t<double, double>(c, slab, z0, nzs);
-        case LBM_FP32: return fields_t<float, float>(c, slab, z0, nzs);
-        case LBM_FP16_SHIFTED: return fields_t<__half, float>(c, slab, z0, nzs);
-        case LBM_BF16_SHIFTED: return fields_t<__nv_bfloat16, float>(c, slab, z0, nzs);
+        case LBM_FP64: return fields_t<double, double>(c, out, z0, nzs);
+        case LBM_FP32: return fields_t<float, float>(c, out, z0, nzs);
+        case LBM_FP16_SHIFTED: return fields_t<__half, float>(c, out, z0, nzs);
+        case LBM_BF16_SHIFTED: return fields_t<__nv_bfloat16, float>(c, out, z0, nzs);
     }
     return cudaErrorInvalidValue;
 }

@@ -49,6 +49,7 @@ struct lbm_ctx {
     int fused_threads = 256;  // threads per CTA of that kernel (32 x 8 or 32 x 16)
     int sms = 0;
     int* status = nullptr;  // device status word written by bounded waits
+    bool bounded_waits = false;  // a kernel that may write `status` has been launched
     cudaGraphExec_t step_graph[2] = {nullptr, nullptr};  // STEP_GRAPH steps starting from buf[0] / buf[1]
     int step_graph_shape[6] = {-1, -1, -1, -1, -1, -1};  // launch shape the graphs were captured with
     std::string err;
@@ -63,7 +64,7 @@ void lbm_internal_get_allocator(lbm_alloc_fn* a, lbm_free_fn* r, void** user);
 void lbm_internal_dev_free(lbm_ctx* c, void* p);
 lbm_status lbm_internal_alloc_batch(lbm_ctx* c, size_t state_elems, size_t cells, size_t max_plane);
 void lbm_internal_release(lbm_ctx* c);
-cudaError_t lbm_internal_init_slab(lbm_ctx* c, int z0, int nzs, bool uniform);
+cudaError_t lbm_internal_init_rest(lbm_ctx* c);
 cudaError_t lbm_internal_step(lbm_ctx* c, long n, bool dry);
 lbm_status lbm_internal_batch_status(lbm_ctx* c);
 lbm_status lbm_internal_alloc_batch_tables(lbm_ctx* c);
@@ -76,6 +77,23 @@ namespace lbm {
 constexpr int RED_WIDTH = 8;  // mass, mom x/y/z, |du|^2, |u|^2, bad-node count, spare
 constexpr int RED_BLOCKS = 1216;  // 152 SMs x 8
 constexpr int RED_THREADS = 256;
+
+// Fields of a run of whole z-planes, node 0 the first of them: the staging slab's
+// planes, or the caller's own device arrays.  A null u or B is zero on the way
+// in; a null output is not wanted.
+struct FieldsIn {
+    const double* rho = nullptr;
+    const double* u[3] = {nullptr, nullptr, nullptr};
+    const double* phase = nullptr;
+    const double* B[3] = {nullptr, nullptr, nullptr};
+    __device__ static __forceinline__ double value(const double* p, size_t k) { return p ? p[k] : 0.0; }
+};
+struct FieldsOut {
+    double* rho = nullptr;
+    double* u[3] = {nullptr, nullptr, nullptr};
+    double* phase = nullptr;
+    double* B[3] = {nullptr, nullptr, nullptr};
+};
 
 // Kernel launchers, one per physics module; each returns cudaGetLastError().
 // A "dry" step reads the current state and writes the other buffer without
@@ -92,29 +110,29 @@ inline bool packed16_ok(const lbm_ctx* c) {
     return c->physics == LBM_PHYS_FLUID && (c->prec == LBM_FP16_SHIFTED || c->prec == LBM_BF16_SHIFTED) &&
            c->grid.wall_model == LBM_WALL_BOUNCE_BACK && c->relax.moment_space == LBM_MOMENTS_CENTRAL && c->q == 19;
 }
-cudaError_t fluid_init(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform);
-cudaError_t fluid_fields(lbm_ctx* c, double* slab, int z0, int nzs);
+cudaError_t fluid_init(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform);
+cudaError_t fluid_fields(lbm_ctx* c, const FieldsOut& out, int z0, int nzs);
 cudaError_t fluid_reduce(lbm_ctx* c, bool record);
 
 cudaError_t mhd_step(lbm_ctx* c, long n, bool dry = false);
-cudaError_t mhd_init(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform);
-cudaError_t mhd_fields(lbm_ctx* c, double* slab, int z0, int nzs);
+cudaError_t mhd_init(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform);
+cudaError_t mhd_fields(lbm_ctx* c, const FieldsOut& out, int z0, int nzs);
 cudaError_t mhd_reduce(lbm_ctx* c, bool record);
 
 cudaError_t cgm_step(lbm_ctx* c, long n, bool dry = false);
-cudaError_t cgm_init(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform);
-cudaError_t cgm_fields(lbm_ctx* c, double* slab, int z0, int nzs);
+cudaError_t cgm_init(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform);
+cudaError_t cgm_fields(lbm_ctx* c, const FieldsOut& out, int z0, int nzs);
 cudaError_t cgm_reduce(lbm_ctx* c, bool record);
 
 // D3Q27 single phase (lbm_q27.cu).
 cudaError_t q27_step(lbm_ctx* c, long n, bool dry = false);
-cudaError_t q27_init(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform);
-cudaError_t q27_fields(lbm_ctx* c, double* slab, int z0, int nzs);
+cudaError_t q27_init(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform);
+cudaError_t q27_fields(lbm_ctx* c, const FieldsOut& out, int z0, int nzs);
 cudaError_t q27_reduce(lbm_ctx* c, bool record);
 
 // Shan-Chen (lbm_sc.cu); initialisation is the single-phase one.
 cudaError_t sc_step(lbm_ctx* c, long n, bool dry = false);
-cudaError_t sc_fields(lbm_ctx* c, double* slab, int z0, int nzs);
+cudaError_t sc_fields(lbm_ctx* c, const FieldsOut& out, int z0, int nzs);
 cudaError_t sc_reduce(lbm_ctx* c, bool record);
 
 // Sum RED_BLOCKS partials into c->result (deterministic order).

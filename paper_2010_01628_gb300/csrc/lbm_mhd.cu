@@ -15,25 +15,24 @@ __global__ void __launch_bounds__(256) mhd_step_kernel(const S* __restrict__ src
 }
 
 template <typename S, typename C>
-__global__ void mhd_init_kernel(S* __restrict__ dst, const double* __restrict__ slab, Box b, int z0, int nzs,
+__global__ void mhd_init_kernel(S* __restrict__ dst, FieldsIn in, Box b, int z0, int nzs,
                                 bool uniform) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, zs = blockIdx.z;
     if (x >= b.nx || zs >= nzs) return;
-    const size_t m = (size_t)b.nx * b.ny * nzs;
     const size_t k = ((size_t)zs * b.ny + y) * b.nx + x;
     const uint32_t self = ((uint32_t)(z0 + zs) * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     C rho = (C)1, drho = (C)0, ux = (C)0, uy = (C)0, uz = (C)0;
     C bb[3] = {(C)0, (C)0, (C)0};
     if (!uniform) {
-        drho = (C)(slab[k] - 1.0);
-        rho = (C)slab[k];
-        ux = (C)slab[m + k];
-        uy = (C)slab[2 * m + k];
-        uz = (C)slab[3 * m + k];
-        bb[0] = (C)slab[5 * m + k];
-        bb[1] = (C)slab[6 * m + k];
-        bb[2] = (C)slab[7 * m + k];
+        drho = (C)(in.rho[k] - 1.0);
+        rho = (C)in.rho[k];
+        ux = (C)in.value(in.u[0], k);
+        uy = (C)in.value(in.u[1], k);
+        uz = (C)in.value(in.u[2], k);
+        bb[0] = (C)in.value(in.B[0], k);
+        bb[1] = (C)in.value(in.B[1], k);
+        bb[2] = (C)in.value(in.B[2], k);
     }
     C f[Q];
     equilibrium_shifted<C>(rho, drho, ux, uy, uz, f);
@@ -49,13 +48,12 @@ __global__ void mhd_init_kernel(S* __restrict__ dst, const double* __restrict__ 
 }
 
 template <typename S, typename C, bool WALLS>
-__global__ void mhd_fields_kernel(const S* __restrict__ src, double* __restrict__ slab, MhdArgs p, int z0, int nzs) {
+__global__ void mhd_fields_kernel(const S* __restrict__ src, FieldsOut out, MhdArgs p, int z0, int nzs) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, zs = blockIdx.z;
     const Box& b = p.box;
     if (x >= b.nx || zs >= nzs) return;
     const int z = z0 + zs;
-    const size_t m = (size_t)b.nx * b.ny * nzs;
     const size_t k = ((size_t)zs * b.ny + y) * b.nx + x;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
@@ -67,13 +65,13 @@ __global__ void mhd_fields_kernel(const S* __restrict__ src, double* __restrict_
     const Moments<C> mo = moments19(f);
     C bb[3];
     const Macro<C> a = mhd_macro<C>(mo, g, p, bb);
-    slab[k] = (double)a.rho;
-    slab[m + k] = (double)a.ux;
-    slab[2 * m + k] = (double)a.uy;
-    slab[3 * m + k] = (double)a.uz;
-    slab[5 * m + k] = (double)bb[0];
-    slab[6 * m + k] = (double)bb[1];
-    slab[7 * m + k] = (double)bb[2];
+    if (out.rho) out.rho[k] = (double)a.rho;
+    if (out.u[0]) out.u[0][k] = (double)a.ux;
+    if (out.u[1]) out.u[1][k] = (double)a.uy;
+    if (out.u[2]) out.u[2][k] = (double)a.uz;
+    if (out.B[0]) out.B[0][k] = (double)bb[0];
+    if (out.B[1]) out.B[1][k] = (double)bb[1];
+    if (out.B[2]) out.B[2][k] = (double)bb[2];
 }
 
 template <typename S, typename C, bool WALLS>
@@ -141,22 +139,22 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
 }
 
 template <typename S, typename C>
-static cudaError_t init_t(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform) {
+static cudaError_t init_t(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform) {
     const int bx = c->block_x;
     dim3 grid((unsigned)((c->box.nx + bx - 1) / bx), (unsigned)c->box.ny, (unsigned)nzs);
-    mhd_init_kernel<S, C><<<grid, bx, 0, c->stream>>>((S*)c->buf[c->cur], slab, c->box, z0, nzs, uniform);
+    mhd_init_kernel<S, C><<<grid, bx, 0, c->stream>>>((S*)c->buf[c->cur], in, c->box, z0, nzs, uniform);
     return cudaGetLastError();
 }
 
 template <typename S, typename C>
-static cudaError_t fields_t(lbm_ctx* c, double* slab, int z0, int nzs) {
+static cudaError_t fields_t(lbm_ctx* c, const FieldsOut& out, int z0, int nzs) {
     const MhdArgs p = mhd_args(c);
     const int bx = c->block_x;
     dim3 grid((unsigned)((c->box.nx + bx - 1) / bx), (unsigned)c->box.ny, (unsigned)nzs);
     if ((c->box.periodic & 7u) != 7u)
-        mhd_fields_kernel<S, C, true><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], slab, p, z0, nzs);
+        mhd_fields_kernel<S, C, true><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], out, p, z0, nzs);
     else
-        mhd_fields_kernel<S, C, false><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], slab, p, z0, nzs);
+        mhd_fields_kernel<S, C, false><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], out, p, z0, nzs);
     return cudaGetLastError();
 }
 
@@ -177,12 +175,12 @@ static cudaError_t reduce_t(lbm_ctx* c, bool record) {
 cudaError_t mhd_step(lbm_ctx* c, long n, bool dry) {
     return c->prec == LBM_FP64 ? step_t<double, double>(c, n, dry) : step_t<float, float>(c, n, dry);
 }
-cudaError_t mhd_init(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform) {
-    return c->prec == LBM_FP64 ? init_t<double, double>(c, slab, z0, nzs, uniform)
-                               : init_t<float, float>(c, slab, z0, nzs, uniform);
+cudaError_t mhd_init(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform) {
+    return c->prec == LBM_FP64 ? init_t<double, double>(c, in, z0, nzs, uniform)
+                               : init_t<float, float>(c, in, z0, nzs, uniform);
 }
-cudaError_t mhd_fields(lbm_ctx* c, double* slab, int z0, int nzs) {
-    return c->prec == LBM_FP64 ? fields_t<double, double>(c, slab, z0, nzs) : fields_t<float, float>(c, slab, z0, nzs);
+cudaError_t mhd_fields(lbm_ctx* c, const FieldsOut& out, int z0, int nzs) {
+    return c->prec == LBM_FP64 ? fields_t<double, double>(c, out, z0, nzs) : fields_t<float, float>(c, out, z0, nzs);
 }
 cudaError_t mhd_reduce(lbm_ctx* c, bool record) {
     return c->prec == LBM_FP64 ? reduce_t<double, double>(c, record) : reduce_t<float, float>(c, record);

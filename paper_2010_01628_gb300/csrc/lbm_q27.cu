@@ -364,21 +364,20 @@ __global__ void __launch_bounds__(256) step_kernel(const S* __restrict__ src, S*
 
 // f - w = rho (prod phi(u) - prod w) + (rho - 1) w.
 template <typename S, typename C>
-__global__ void init_kernel(S* __restrict__ dst, const double* __restrict__ slab, Box b, int z0, int nzs, bool uniform) {
+__global__ void init_kernel(S* __restrict__ dst, FieldsIn in, Box b, int z0, int nzs, bool uniform) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, zs = blockIdx.z;
     if (x >= b.nx || zs >= nzs) return;
-    const size_t m = (size_t)b.nx * b.ny * nzs;
     const size_t k = ((size_t)zs * b.ny + y) * b.nx + x;
     const uint32_t self = ((uint32_t)(z0 + zs) * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     double rho = 1.0, u[3] = {0.0, 0.0, 0.0};
     if (!uniform) {
-        rho = slab[k];
-        u[0] = slab[m + k];
-        u[1] = slab[2 * m + k];
-        u[2] = slab[3 * m + k];
+        rho = in.rho[k];
+        u[0] = in.value(in.u[0], k);
+        u[1] = in.value(in.u[1], k);
+        u[2] = in.value(in.u[2], k);
     }
-    const double drho = uniform ? 0.0 : slab[k] - 1.0;
+    const double drho = uniform ? 0.0 : in.rho[k] - 1.0;
     double ph[3][3], dl[3][3];
     for (int ax = 0; ax < 3; ++ax) {
         const double v = u[ax], v2 = v * v;
@@ -404,23 +403,22 @@ __global__ void init_kernel(S* __restrict__ dst, const double* __restrict__ slab
 }
 
 template <typename S, typename C, bool WALLS>
-__global__ void fields_kernel(const S* __restrict__ src, double* __restrict__ slab, Args p, int z0, int nzs) {
+__global__ void fields_kernel(const S* __restrict__ src, FieldsOut out, Args p, int z0, int nzs) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, zs = blockIdx.z;
     const Box& b = p.box;
     if (x >= b.nx || zs >= nzs) return;
     const int z = z0 + zs;
-    const size_t m = (size_t)b.nx * b.ny * nzs;
     const size_t k = ((size_t)zs * b.ny + y) * b.nx + x;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
     C g[3][3][3];
     gather<S, C, WALLS>(src, b, q, x, y, z, self, p, g);
     const Node<C> s = macro<C>(moments<C>(g), p);
-    slab[k] = (double)s.rho;
-    slab[m + k] = (double)s.ux;
-    slab[2 * m + k] = (double)s.uy;
-    slab[3 * m + k] = (double)s.uz;
+    if (out.rho) out.rho[k] = (double)s.rho;
+    if (out.u[0]) out.u[0][k] = (double)s.ux;
+    if (out.u[1]) out.u[1][k] = (double)s.uy;
+    if (out.u[2]) out.u[2][k] = (double)s.uz;
 }
 
 template <typename S, typename C, bool WALLS>
@@ -480,22 +478,22 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
 }
 
 template <typename S, typename C>
-static cudaError_t init_t(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform) {
+static cudaError_t init_t(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform) {
     const int bx = c->block_x;
     dim3 grid((unsigned)((c->box.nx + bx - 1) / bx), (unsigned)c->box.ny, (unsigned)nzs);
-    init_kernel<S, C><<<grid, bx, 0, c->stream>>>((S*)c->buf[c->cur], slab, c->box, z0, nzs, uniform);
+    init_kernel<S, C><<<grid, bx, 0, c->stream>>>((S*)c->buf[c->cur], in, c->box, z0, nzs, uniform);
     return cudaGetLastError();
 }
 
 template <typename S, typename C>
-static cudaError_t fields_t(lbm_ctx* c, double* slab, int z0, int nzs) {
+static cudaError_t fields_t(lbm_ctx* c, const FieldsOut& out, int z0, int nzs) {
     const Args p = args_of(c);
     const int bx = c->block_x;
     dim3 grid((unsigned)((c->box.nx + bx - 1) / bx), (unsigned)c->box.ny, (unsigned)nzs);
     if ((c->box.periodic & 7u) != 7u)
-        fields_kernel<S, C, true><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], slab, p, z0, nzs);
+        fields_kernel<S, C, true><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], out, p, z0, nzs);
     else
-        fields_kernel<S, C, false><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], slab, p, z0, nzs);
+        fields_kernel<S, C, false><<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], out, p, z0, nzs);
     return cudaGetLastError();
 }
 
@@ -518,13 +516,13 @@ static cudaError_t reduce_t(lbm_ctx* c, bool record) {
 cudaError_t q27_step(lbm_ctx* c, long n, bool dry) {
     return c->prec == LBM_FP64 ? q27::step_t<double, double>(c, n, dry) : q27::step_t<float, float>(c, n, dry);
 }
-cudaError_t q27_init(lbm_ctx* c, const double* slab, int z0, int nzs, bool uniform) {
-    return c->prec == LBM_FP64 ? q27::init_t<double, double>(c, slab, z0, nzs, uniform)
-                               : q27::init_t<float, float>(c, slab, z0, nzs, uniform);
+cudaError_t q27_init(lbm_ctx* c, const FieldsIn& in, int z0, int nzs, bool uniform) {
+    return c->prec == LBM_FP64 ? q27::init_t<double, double>(c, in, z0, nzs, uniform)
+                               : q27::init_t<float, float>(c, in, z0, nzs, uniform);
 }
-cudaError_t q27_fields(lbm_ctx* c, double* slab, int z0, int nzs) {
-    return c->prec == LBM_FP64 ? q27::fields_t<double, double>(c, slab, z0, nzs)
-                               : q27::fields_t<float, float>(c, slab, z0, nzs);
+cudaError_t q27_fields(lbm_ctx* c, const FieldsOut& out, int z0, int nzs) {
+    return c->prec == LBM_FP64 ? q27::fields_t<double, double>(c, out, z0, nzs)
+                               : q27::fields_t<float, float>(c, out, z0, nzs);
 }
 cudaError_t q27_reduce(lbm_ctx* c, bool record) {
     return c->prec == LBM_FP64 ? q27::reduce_t<double, double>(c, record) : q27::reduce_t<float, float>(c, record);

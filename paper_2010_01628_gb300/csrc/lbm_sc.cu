@@ -168,14 +168,13 @@ __global__ void __launch_bounds__(32 * BY) sc_fused_kernel(const S* __restrict__
 
 // rho, u (with +F/2) and psi of a z-slab; psi of the whole box is current.
 template <typename S, typename C, bool WALLS>
-__global__ void sc_fields_kernel(const S* __restrict__ src, const C* __restrict__ psi, double* __restrict__ slab,
+__global__ void sc_fields_kernel(const S* __restrict__ src, const C* __restrict__ psi, FieldsOut out,
                                  ScArgs p, int z0, int nzs) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, zs = blockIdx.z;
     const Box& b = p.box;
     if (x >= b.nx || zs >= nzs) return;
     const int z = z0 + zs;
-    const size_t m = (size_t)b.nx * b.ny * nzs;
     const size_t k = ((size_t)zs * b.ny + y) * b.nx + x;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
@@ -183,11 +182,11 @@ __global__ void sc_fields_kernel(const S* __restrict__ src, const C* __restrict_
     gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
     const Moments<C> mo = moments19(f);
     const Macro<C> a = sc_macro<C>(mo, psi, b, q, x, y, z, self, p);
-    slab[k] = (double)a.rho;
-    slab[m + k] = (double)a.ux;
-    slab[2 * m + k] = (double)a.uy;
-    slab[3 * m + k] = (double)a.uz;
-    slab[4 * m + k] = (double)psi[self];
+    if (out.rho) out.rho[k] = (double)a.rho;
+    if (out.u[0]) out.u[0][k] = (double)a.ux;
+    if (out.u[1]) out.u[1][k] = (double)a.uy;
+    if (out.u[2]) out.u[2][k] = (double)a.uz;
+    if (out.phase) out.phase[k] = (double)psi[self];
 }
 
 template <typename S, typename C, bool WALLS>
@@ -282,16 +281,16 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
 }
 
 template <typename S, typename C>
-static cudaError_t fields_t(lbm_ctx* c, double* slab, int z0, int nzs) {
+static cudaError_t fields_t(lbm_ctx* c, const FieldsOut& out, int z0, int nzs) {
     const ScArgs p = sc_args(c);
     const S* src = (const S*)c->buf[c->cur];
     if (z0 == 0) launch_psi<S, C>(c, src, p);  // slabs are read in order from z0 = 0
     const int bx = c->block_x;
     dim3 grid((unsigned)((c->box.nx + bx - 1) / bx), (unsigned)c->box.ny, (unsigned)nzs);
     if ((c->box.periodic & 7u) != 7u)
-        sc_fields_kernel<S, C, true><<<grid, bx, 0, c->stream>>>(src, (const C*)c->phi, slab, p, z0, nzs);
+        sc_fields_kernel<S, C, true><<<grid, bx, 0, c->stream>>>(src, (const C*)c->phi, out, p, z0, nzs);
     else
-        sc_fields_kernel<S, C, false><<<grid, bx, 0, c->stream>>>(src, (const C*)c->phi, slab, p, z0, nzs);
+        sc_fields_kernel<S, C, false><<<grid, bx, 0, c->stream>>>(src, (const C*)c->phi, out, p, z0, nzs);
     return cudaGetLastError();
 }
 
@@ -314,8 +313,8 @@ static cudaError_t reduce_t(lbm_ctx* c, bool record) {
 cudaError_t sc_step(lbm_ctx* c, long n, bool dry) {
     return c->prec == LBM_FP64 ? step_t<double, double>(c, n, dry) : step_t<float, float>(c, n, dry);
 }
-cudaError_t sc_fields(lbm_ctx* c, double* slab, int z0, int nzs) {
-    return c->prec == LBM_FP64 ? fields_t<double, double>(c, slab, z0, nzs) : fields_t<float, float>(c, slab, z0, nzs);
+cudaError_t sc_fields(lbm_ctx* c, const FieldsOut& out, int z0, int nzs) {
+    return c->prec == LBM_FP64 ? fields_t<double, double>(c, out, z0, nzs) : fields_t<float, float>(c, out, z0, nzs);
 }
 cudaError_t sc_reduce(lbm_ctx* c, bool record) {
     return c->prec == LBM_FP64 ? reduce_t<double, double>(c, record) : reduce_t<float, float>(c, record);
