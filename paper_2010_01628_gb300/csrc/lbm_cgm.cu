@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(256) cgm_collide_kernel(const S* __restrict__ 
     const CgmNode<C> s = cgm_macro<C>(f, m, rho_red[self], p);
     cgm_collide<C>(f, m, s, (C)p.omega);
     C gr[3];
-    grad_phi<C>(phi, b, q, x, y, z, self, gr);
+    grad_phi<C, WALLS>(phi, b, q, x, y, z, self, gr);
     const C n2 = gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2];
     const C nrm = sqrt(n2);
     // each colour's operator carries A_k/2 = A/2; together they perturb the total by

@@ -202,7 +202,7 @@ __device__ __forceinline__ void cgm_phi_node(const S* __restrict__ src, C* __res
 
 // grad phi = (1/c_s^2) sum_i w_i c_i phi(x + c_i): the axis and the diagonal
 // neighbours are summed apart and scaled once (3/18 and 3/36).
-template <typename C, bool NC = true>
+template <typename C, bool WALLS, bool NC = true>
 __device__ __forceinline__ void grad_phi(const C* __restrict__ phi, const Box& b, const Nbr& q, int x, int y, int z,
                                          uint32_t self, C (&gr)[3]) {
     const C own = NC ? phi[self] : ld_coherent(phi + self);
@@ -211,7 +211,7 @@ __device__ __forceinline__ void grad_phi(const C* __restrict__ phi, const Box& b
     {                                                                                       \
         constexpr int ex = cx_of(I), ey = cy_of(I), ez = cz_of(I);                          \
         constexpr bool axis = ex * ex + ey * ey + ez * ez == 1;                             \
-        const C t = field_nbr<C, I, NC>(phi, b, q, x, y, z, own);                           \
+        const C t = field_nbr<C, WALLS, I, NC>(phi, b, q, x, y, z, own);                           \
         if (ex) { if (axis) ax += ex > 0 ? t : -t; else dx += ex > 0 ? t : -t; }            \
         if (ey) { if (axis) ay += ey > 0 ? t : -t; else dy += ey > 0 ? t : -t; }            \
         if (ez) { if (axis) az += ez > 0 ? t : -t; else dz += ez > 0 ? t : -t; }            \
@@ -264,7 +264,7 @@ __device__ __forceinline__ void cgm_collide_node(const S* __restrict__ src, S* _
     const CgmNode<C> s = cgm_macro<C>(f, m, NC ? rho_red[self] : ld_coherent(rho_red + self), p);
     cgm_collide<C>(f, m, s, (C)p.omega);
     C gr[3];
-    grad_phi<C, NC>(phi, b, q, x, y, z, self, gr);
+    grad_phi<C, WALLS, NC>(phi, b, q, x, y, z, self, gr);
     const C n2 = gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2];
     const C nrm = sqrt(n2);
     // each colour's operator carries A_k/2 = A/2; together they perturb the total by

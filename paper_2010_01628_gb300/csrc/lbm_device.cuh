@@ -201,18 +201,20 @@ __device__ __forceinline__ void gather19(const S* __restrict__ src, const Box& b
 }
 
 // Value of a node field v at x + c_I; a neighbour behind a wall contributes
-// the node's own value `own`.  NC: read-only path (the field is not written
+// the node's own value `own`.  WALLS = false (every axis periodic) carries none
+// of the wall predicates, which cost the issue-bound collide passes about 90 of
+// their 760 (Shan-Chen) and 1004 (colour gradient) instructions.  NC: read-only path (the field is not written
 // during the kernel); else a plain load (persistent kernels that rewrite the
 // field between grid-wide barriers; see Store::load_coherent).
-template <typename C, int I, bool NC = true>
+template <typename C, bool WALLS, int I, bool NC = true>
 __device__ __forceinline__ C field_nbr(const C* __restrict__ v, const Box& b, const Nbr& q, int x, int y, int z,
                                        C own) {
     constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
     const int sx = cx == 0 ? x : (cx > 0 ? q.xp : q.xm);
     const int sy = cy == 0 ? y : (cy > 0 ? q.yp : q.ym);
     const int sz = cz == 0 ? z : (cz > 0 ? q.zp : q.zm);
-    const bool wall = (cx > 0 && q.wxp) || (cx < 0 && q.wxm) || (cy > 0 && q.wyp) || (cy < 0 && q.wym) ||
-                      (cz > 0 && q.wzp) || (cz < 0 && q.wzm);
+    const bool wall = WALLS && ((cx > 0 && q.wxp) || (cx < 0 && q.wxm) || (cy > 0 && q.wyp) || (cy < 0 && q.wym) ||
+                                (cz > 0 && q.wzp) || (cz < 0 && q.wzm));
     if (wall) return own;
     const C* a = v + ((uint32_t)sz * (uint32_t)b.ny + (uint32_t)sy) * (uint32_t)b.nx + (uint32_t)sx;
     return NC ? __ldg(a) : ld_coherent(a);
@@ -221,13 +223,13 @@ __device__ __forceinline__ C field_nbr(const C* __restrict__ v, const Box& b, co
 // s = sum_i w_i c_i v(x + c_i) over the 18 moving directions: the lattice
 // first moment of a node field (times 1/c_s^2 the isotropic gradient of the
 // colour-gradient model; times -G psi(x) the Shan-Chen force).
-template <typename C, bool NC = true>
+template <typename C, bool WALLS, bool NC = true>
 __device__ __forceinline__ void lattice_first_moment(const C* __restrict__ v, const Box& b, const Nbr& q, int x,
                                                      int y, int z, C own, C (&s)[3]) {
     C gx = (C)0, gy = (C)0, gz = (C)0;
 #define LBM_FM(I)                                                           \
     {                                                                       \
-        const C t = field_nbr<C, I, NC>(v, b, q, x, y, z, own) * (C)w_of(I); \
+        const C t = field_nbr<C, WALLS, I, NC>(v, b, q, x, y, z, own) * (C)w_of(I); \
         if (cx_of(I)) gx += (C)cx_of(I) * t;                                \
         if (cy_of(I)) gy += (C)cy_of(I) * t;                                \
         if (cz_of(I)) gz += (C)cz_of(I) * t;                                \

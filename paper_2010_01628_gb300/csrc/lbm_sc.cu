@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(256) sc_collide_kernel(const S* __restrict__ s
     C f[Q];
     gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
     const Moments<C> m = moments19(f);
-    const Macro<C> a = sc_macro<C>(m, psi, b, q, x, y, z, self, p);
+    const Macro<C> a = sc_macro<C, WALLS>(m, psi, b, q, x, y, z, self, p);
     collide_fluid<C>(f, m, a, (C)p.omega);
     conserve_mass<C>(f, m.drho);
     scatter19<S, C>(dst, b.n, self, f);
@@ -181,7 +181,7 @@ __global__ void sc_fields_kernel(const S* __restrict__ src, const C* __restrict_
     C f[Q];
     gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
     const Moments<C> mo = moments19(f);
-    const Macro<C> a = sc_macro<C>(mo, psi, b, q, x, y, z, self, p);
+    const Macro<C> a = sc_macro<C, WALLS>(mo, psi, b, q, x, y, z, self, p);
     if (out.rho) out.rho[k] = (double)a.rho;
     if (out.u[0]) out.u[0][k] = (double)a.ux;
     if (out.u[1]) out.u[1][k] = (double)a.uy;
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(RED_THREADS) sc_reduce_kernel(const S* __restr
             C f[Q];
             gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
             const Moments<C> mo = moments19(f);
-            const Macro<C> a = sc_macro<C>(mo, psi, b, q, x, y, z, self, p);
+            const Macro<C> a = sc_macro<C, WALLS>(mo, psi, b, q, x, y, z, self, p);
             reduce_node<C>(acc, a.rho, a.ux, a.uy, a.uz, uprev, b.n, self, have_prev, record);
         }
     }

@@ -25,14 +25,14 @@ __device__ __forceinline__ C pseudopotential(C rho) {
 // rho, F = rho g + F_sc and u = (j + F/2)/rho of a pulled node.
 // NC: read-only loads of psi (it is not written during the kernel); else
 // plain loads (the batched persistent kernel rewrites psi between barriers).
-template <typename C, bool NC = true>
+template <typename C, bool WALLS, bool NC = true>
 __device__ __forceinline__ Macro<C> sc_macro(const Moments<C>& m, const C* __restrict__ psi, const Box& b,
                                              const Nbr& q, int x, int y, int z, uint32_t self, const ScArgs& p) {
     Macro<C> a;
     a.rho = (C)1 + m.drho;
     const C own = NC ? psi[self] : ld_coherent(psi + self);
     C s[3];
-    lattice_first_moment<C, NC>(psi, b, q, x, y, z, own, s);
+    lattice_first_moment<C, WALLS, NC>(psi, b, q, x, y, z, own, s);
     const C mg = -(C)p.G * own;
     a.Fx = (a.rho * (C)p.g[0] - (C)p.rg[0]) + mg * s[0];
     a.Fy = (a.rho * (C)p.g[1] - (C)p.rg[1]) + mg * s[1];
@@ -66,7 +66,7 @@ __device__ __forceinline__ void sc_collide_node(const S* __restrict__ src, S* __
     C f[Q];
     gather19<S, C, WALLS, NC>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
     const Moments<C> m = moments19(f);
-    const Macro<C> a = sc_macro<C, NC>(m, psi, b, q, x, y, z, self, p);
+    const Macro<C> a = sc_macro<C, WALLS, NC>(m, psi, b, q, x, y, z, self, p);
     collide_fluid<C>(f, m, a, (C)p.omega);
     conserve_mass<C>(f, m.drho);
     scatter19<S, C>(dst, b.n, self, f);
