@@ -313,7 +313,7 @@ def _mhd_batch(L, timed, steps, peak, domains, tune_cache="tmp", ranks=None):
     out = {}
 
     # C3: Hartmann channels (64 by default), sizes {32,48,64,96}^3, Ha in [1,20], FP32 MHD,
-    # one persistent cooperative launch per call, captured in a CUDA graph.  With several ranks the sweep's
+    # one launch per step over all domains, replayed from captured graphs.  With several ranks the sweep's
     # domains are partitioned by node count (no exchange between ranks): strong scaling of the fixed sweep.
     full = inputs.hartmann_batch(domains, seed=2)
     world = ranks.world if ranks else 1
@@ -345,7 +345,7 @@ def _mhd_batch(L, timed, steps, peak, domains, tune_cache="tmp", ranks=None):
     ach = 320 * cells * n_b / t / 1e9
     out[f"mhd_batch_{domains}"] = {"MLUPS": cells * n_b / t / 1e6, "cells": cells, "steps": n_b, "bytes_per_lup": 320,
                            "achieved_GBps": ach, "frac_of_hbm_peak": ach / peak, "launch": info,
-                           "autotune_MLUPS": tuned, "launches_per_call": 1, "ranks": world,
+                           "autotune_MLUPS": tuned, "launches_per_step": 1, "ranks": world,
                            "domains_on_rank0": len(mine)}
     return out
 
@@ -357,8 +357,8 @@ CGM_BYTES = 24 * 2 * 4 + 2 * 2 * 4
 
 def _cgm_batch(L, timed, steps, peak, domains=64, tune_cache="tmp"):
     """Density-ratio sweep: `domains` periodic droplet boxes, sizes {32,48,64,96}^3, density ratio U[2, 10]
-    (seed 5), sigma = 1e-4, tau = 0.8, beta = 0.7, FP32, in one persistent cooperative launch per call (two
-    passes per step with a grid barrier after each), captured in a CUDA graph."""
+    (seed 5), sigma = 1e-4, tau = 0.8, beta = 0.7, FP32, as one batch (two launches per step over all domains,
+    replayed from captured graphs)."""
     import tempfile
     sweep = inputs.droplet_sweep(domains, seed=5)
     shapes = [(n, n, n) for n, _ in sweep]
@@ -383,8 +383,8 @@ def _cgm_batch(L, timed, steps, peak, domains=64, tune_cache="tmp"):
     return {f"cgm_batch_{domains}": {
         "MLUPS": cells * n_b / t / 1e6, "cells": cells, "steps": n_b, "bytes_per_lup": CGM_BYTES,
         "moved_bytes_per_lup": 284, "achieved_GBps": ach, "frac_of_hbm_peak": ach / peak, "launch": info,
-        "autotune_MLUPS": tuned, "launches_per_call": 1,
-        "note": "colour-gradient density-ratio sweep (ratio U[2,10]) in one persistent launch; "
+        "autotune_MLUPS": tuned, "launches_per_step": 2,
+        "note": "colour-gradient density-ratio sweep (ratio U[2,10]) stepped as one batch; "
                 + CGM_NOTE}}
 CGM_NOTE = ("two passes per step (phi and rho_r, then collide); 24 stored values per node (total populations, red "
             "fraction, recolouring vector, red rest), 208 B/LUP algorithmic; pass 1 and pass 2 both read the totals "
@@ -418,8 +418,8 @@ def _cgm(L, timed, steps, peak, n, launch="auto"):
 
 def _sc_batch(L, timed, steps, peak, domains=64, tune_cache="tmp"):
     """Interaction-strength sweep: `domains` periodic static-bubble boxes, sizes {32,48,64,96}^3, G U[-5.5, -4.5]
-    (seed 6; the coexistence densities, hence the density ratio, follow G), radius n/4, nu = 0.0333, FP32, in one
-    persistent cooperative launch per call (pseudopotential pass, barrier, collision pass, barrier)."""
+    (seed 6; the coexistence densities, hence the density ratio, follow G), radius n/4, nu = 0.0333, FP32, as one
+    batch (two launches per step over all domains: pseudopotential, collision)."""
     import tempfile
     sweep = inputs.bubble_sweep(domains, seed=6)
     shapes = [(n, n, n) for n, _ in sweep]
@@ -441,8 +441,8 @@ def _sc_batch(L, timed, steps, peak, domains=64, tune_cache="tmp"):
     return {f"sc_batch_{domains}": {
         "MLUPS": cells * n_b / t / 1e6, "cells": cells, "steps": n_b, "bytes_per_lup": 160,
         "moved_bytes_per_lup": 236, "achieved_GBps": ach, "frac_of_hbm_peak": ach / peak, "launch": info,
-        "autotune_MLUPS": tuned, "launches_per_call": 1,
-        "note": "Shan-Chen interaction-strength sweep in one persistent launch: two passes per step "
+        "autotune_MLUPS": tuned, "launches_per_step": 2,
+        "note": "Shan-Chen interaction-strength sweep stepped as one batch: two passes per step "
                 "(pseudopotential, then forced collision); 160 B/LUP algorithmic (populations read and written, psi "
                 "written and read once); the two passes move 236 B"}}
 

@@ -49,7 +49,7 @@ typedef enum {
     LBM_ERR_OOM = 2,         /* device allocation failed */
     LBM_ERR_CUDA = 3,        /* a CUDA call failed */
     LBM_ERR_DIVERGED = 4,    /* NaN/Inf or rho <= 0 found by a reduction */
-    LBM_ERR_TIMEOUT = 5,     /* a bounded device wait (batch grid barrier) ran out */
+    LBM_ERR_TIMEOUT = 5,     /* a bounded device wait ran out */
     LBM_ERR_UNSUPPORTED = 6  /* valid request this build does not implement */
 } lbm_status;
 
@@ -199,32 +199,28 @@ lbm_status lbm_set_populations(lbm_ctx *ctx, const void *src, size_t bytes);
 
 /* ---- Batched parameter sweeps ---------------------------------------------
  * Many independent domains (uneven sizes, per-domain omega, force, wall field,
- * density ratio, surface tension) advanced together: each lbm_batch_step runs
- * ONE persistent cooperative kernel that performs all n steps with a
- * bounded-wait grid barrier between steps, replayed from a CUDA graph captured
- * on first use (per step count and buffer parity).  Physics: LBM_PHYS_FLUID,
- * LBM_PHYS_MHD, LBM_PHYS_CGM (App. E colour gradient) or LBM_PHYS_SC (Sec.
- * III.G Shan-Chen); the two-phase steps take two passes per step (order
- * parameter or pseudopotential, then collision) separated by a second grid
- * barrier, and the batch holds their phi and rho_r (psi) planes for all
- * domains; FP64 or FP32.  grids/relax/forcing/phys are arrays of ndomains
- * entries (forcing may be NULL; rho_ref must be 0 except for CGM and SC; phys
- * is required for MHD, CGM and SC, whose tau_m and b_wall, alpha_r, alpha_b,
- * A, beta, or G are taken per domain; the colour gradient and MHD have no
- * moving lid).  Domain d is initialised, read back, reduced and
+ * density ratio, surface tension) advanced together: a step is one launch over
+ * the nodes of all domains (two for the two-phase modules: order parameter or
+ * pseudopotential, then collision; more launches beyond 128 domains), and 16
+ * steps at a time are replayed from a captured CUDA graph.  Physics:
+ * LBM_PHYS_FLUID, LBM_PHYS_MHD, LBM_PHYS_CGM (App. E colour gradient) or
+ * LBM_PHYS_SC (Sec. III.G Shan-Chen), whose batch holds the phi and rho_r (psi)
+ * planes for all domains; FP64 or FP32.  grids/relax/forcing/phys are arrays of
+ * ndomains entries (forcing may be NULL; rho_ref must be 0 except for CGM and
+ * SC; phys is required for MHD, CGM and SC, whose tau_m and b_wall, alpha_r,
+ * alpha_b, A, beta, or G are taken per domain; the colour gradient and MHD have
+ * no moving lid).  Domain d is initialised, read back, reduced and
  * checkpointed through its view (lbm_batch_domain), which accepts
  * lbm_init_fields, lbm_fields, lbm_reduce and lbm_get/set_populations; the view
  * is owned by the batch (lbm_destroy on it does nothing, lbm_step on it is
- * LBM_ERR_UNSUPPORTED).  lbm_step on the batch context equals lbm_batch_step.
- * A barrier wait longer than 2 s ends the kernel; lbm_sync then returns
- * LBM_ERR_TIMEOUT. */
+ * LBM_ERR_UNSUPPORTED).  lbm_step on the batch context equals lbm_batch_step. */
 lbm_status lbm_batch_create(lbm_ctx **out, int ndomains, const lbm_grid *grids, const lbm_relax *relax,
                             const lbm_forcing *forcing, lbm_physics physics, const lbm_physparams *phys,
                             lbm_precision precision, void *cuda_stream);
 lbm_status lbm_batch_domain(lbm_ctx *batch, int domain, lbm_ctx **view);
 lbm_status lbm_batch_step(lbm_ctx *batch, long n);
-/* Launch shape of the persistent kernel: threads per CTA, CTAs, whether the
- * launch is replayed from a captured graph, number of tiles per step. */
+/* Launch shape of a step: threads per CTA, CTAs, whether steps are replayed
+ * from captured graphs, number of tiles (one CTA each). */
 lbm_status lbm_batch_info(const lbm_ctx *batch, int *threads, int *grid, int *graph, long *tiles);
 
 /* Diagnostic of the bounded device waits: runs a grid barrier that can never
@@ -241,8 +237,7 @@ lbm_status lbm_mbarrier_selftest(double timeout_s, int arrive, int *observed);
 
 /* ---- Autotuner ---------------------------------------------------------------
  * Chooses the launch shape of a context by timed trials that leave its state
- * unchanged: threads per block of the single-domain step kernels, or threads
- * per CTA and CTAs per SM of the batched persistent kernel.  Results are cached
+ * unchanged: threads per block of the single-domain or batched step kernels.  Results are cached
  * in a JSON file (cache_path, may be NULL = no cache) keyed by device, physics,
  * precision and geometry; a cached entry is applied without timing unless
  * force != 0.  Reports the chosen throughput in MLUPS (may be NULL). */

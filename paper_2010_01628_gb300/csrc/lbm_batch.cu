@@ -1,23 +1,25 @@
 // lbm_batch.cu -- batched parameter sweeps: many independent domains of
-// uneven sizes advanced by ONE persistent cooperative kernel per call to
-// lbm_batch_step (n steps inside the kernel, a grid-wide barrier between
-// steps), replayed from a captured CUDA graph.
+// uneven sizes advanced together, one launch per pass of a step over the nodes
+// of all of them (lbm_step replays 16 steps per captured graph).
 //
 // Work decomposition: every domain is cut into tiles of `threads` consecutive
-// nodes (x fastest); tiles of all domains form one global index space that the
-// resident CTAs walk with a grid stride.  A CTA finds its tile's domain by a
-// binary search over the per-domain first-tile table (uniform across the CTA).
-// Per-domain parameters (size, boundaries, omega, g, Hartmann field, colour
-// densities and surface tension, Shan-Chen interaction strength...) come from
-// a small device table.  The colour-gradient and Shan-Chen steps take two
-// passes (order parameter or pseudopotential, then collision), so their
-// kernels run a grid-wide barrier after each pass.
+// nodes (x fastest), one CTA per tile.  The first tiles and the parameters (size,
+// boundaries, omega, g, Hartmann field, colour densities and surface tension,
+// Shan-Chen interaction strength...) of up to BATCH_TAB domains are kernel
+// parameters: a CTA finds its domain by a binary search in the constant bank and
+// starts its pulls at once (the same tables in global memory put two dependent
+// loads before them: 64-domain Shan-Chen sweep 18.6 GLUPS instead of 27.4).
+// More domains take more launches.  The colour-gradient and Shan-Chen steps take two passes
+// (order parameter or pseudopotential, then collision).
 //
-// The barrier waits are bounded: a CTA that waits longer than the timeout
-// records LBM_ERR_TIMEOUT and every CTA returns; the host reads the status at
-// the next lbm_sync.  The buffers are rewritten between barriers, so the
-// read-only (.nc) path is not valid here: the kernel uses plain cached loads,
-// which the barrier's GPU-scope fences order after the other CTAs' stores.
+// A launch per pass beats a persistent kernel that holds both passes and
+// synchronises the grid between them: each pass keeps its own register count
+// (32-48 instead of the joint 64), may use the read-only load path, and the
+// launch boundary as a graph node costs less than a grid barrier did.
+// Persistent -> per pass, FP32, GB300, GLUPS: 64 domains of 32..96^3: MHD 19.8
+// -> 21.9 (7.0 TB/s at 320 B per update: HBM-bound), Shan-Chen 20.8 -> 27.4,
+// colour gradient 14.1 -> 16.0, fluid 41.1 -> 46.4 (HBM-bound); 4 domains of
+// 32^3 (latency-bound): 11.4 -> 18.8, 9.8 -> 15.9, 8.0 -> 10.8, 20 -> 30.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,6 +36,22 @@
 
 namespace lbm {
 
+// Quotient by a constant for dividends below 2^31: q = umulhi(n, mul) >> shift
+// (mul = ceil(2^p / d), p = 31 + ceil(log2 d)); mul = 0 stands for d = 1.
+struct FastDiv {
+    uint32_t mul, shift;
+};
+inline FastDiv make_fast_div(uint32_t d) {
+    if (d == 1) return {0u, 0u};
+    uint32_t l = 0;
+    while ((1ull << l) < d) ++l;
+    const uint32_t p = 31 + l;
+    return {(uint32_t)(((1ull << p) + d - 1) / d), p - 32};
+}
+__device__ __forceinline__ uint32_t fast_div(uint32_t n, FastDiv f) {
+    return f.mul ? __umulhi(n, f.mul) >> f.shift : n;
+}
+
 struct BatchDomain {
     FluidArgs fl;     // box, omega, g, lid
     MhdArgs mh;       // box, omega, tau_m, g, b_wall
@@ -41,7 +59,7 @@ struct BatchDomain {
     ScArgs sc;        // box, omega, G, g, rho_ref g, lid
     size_t off;       // element offset of the domain's plane 0 in a state copy
     size_t soff;      // offset of the domain's node 0 in each scratch plane (colour gradient)
-    uint32_t tile0;   // first global tile of the domain
+    FastDiv div_nx, div_ny;
     uint32_t ntiles;
 };
 
@@ -51,8 +69,6 @@ struct BarrierState {
     int err;
     int pad;
 };
-
-constexpr unsigned long long BARRIER_TIMEOUT_NS = 2000000000ull;  // 2 s per wait
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
@@ -99,102 +115,76 @@ __device__ bool grid_barrier(BarrierState* bs, unsigned expected, unsigned long 
     return ok != 0;
 }
 
-// Domain of global tile t (binary search over the first-tile table; uniform
-// across the CTA) and the node's coordinates; false past the domain's end.
-__device__ __forceinline__ bool tile_node(const BatchDomain* __restrict__ doms, int nd, uint32_t t, int& d, int& x,
-                                          int& y, int& z) {
-    int lo = 0, hi = nd - 1;
+// Domains [first, first + nd) of the batch, as a kernel parameter.
+constexpr int BATCH_TAB = 128;
+template <class Args>
+struct BatchRec {
+    Args a;          // starts with its Box
+    size_t off;      // element offset of the domain's plane 0 in a state copy
+    size_t soff;     // offset of its node 0 in each scratch plane
+    FastDiv div_nx, div_ny;  // node -> row -> plane
+};
+template <class Args>
+struct BatchTab {
+    int nd;
+    uint32_t tile0[BATCH_TAB];
+    BatchRec<Args> rec[BATCH_TAB];
+};
+
+template <int PHYS> struct BatchArgs;
+template <> struct BatchArgs<LBM_PHYS_FLUID> { using T = FluidArgs; };
+template <> struct BatchArgs<LBM_PHYS_MHD> { using T = MhdArgs; };
+template <> struct BatchArgs<LBM_PHYS_CGM> { using T = CgmArgs; };
+template <> struct BatchArgs<LBM_PHYS_SC> { using T = ScArgs; };
+
+// One pass of one step.  scratch (colour gradient, Shan-Chen): phi (psi) of
+// every domain's nodes, then rho_r, each `scratch_n` values long.  WALLS: false
+// when every domain is periodic in all three directions (the node code then
+// carries no bounce-back).
+// CTAs of 256 threads per SM the FP32 passes are held to.  Unbounded, the
+// parameters picked from the constant bank at a run-time index fill up to 128
+// registers (Shan-Chen sweep 19.7 GLUPS, 27.4 at these bounds; colour gradient
+// 14.4, 15.2 at 4 and 16.0 at 5 CTAs).
+constexpr int batch_ctas(int phys, int pass, size_t elem) {
+    if (elem != 4) return 1;
+    if (phys == LBM_PHYS_MHD) return 4;
+    if (phys == LBM_PHYS_SC) return pass == 0 ? 6 : 5;
+    if (phys == LBM_PHYS_CGM) return 5;
+    return 6;
+}
+template <int PHYS, int PASS, typename S, typename C, bool WALLS>
+__global__ void __launch_bounds__(256, batch_ctas(PHYS, PASS, sizeof(S)))
+    batch_pass_kernel(const S* __restrict__ src, S* __restrict__ dst, C* __restrict__ scratch, size_t scratch_n,
+                      const __grid_constant__ BatchTab<typename BatchArgs<PHYS>::T> tab) {
+    int lo = 0, hi = tab.nd - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (doms[mid].tile0 <= t)
+        if (tab.tile0[mid] <= blockIdx.x)
             lo = mid;
         else
             hi = mid - 1;
     }
-    d = lo;
-    const Box& b = doms[lo].fl.box;
-    const uint32_t cell = (t - doms[lo].tile0) * blockDim.x + threadIdx.x;
-    if (cell >= (uint32_t)b.n) return false;
-    const uint32_t plane = (uint32_t)b.nx * (uint32_t)b.ny;
-    const uint32_t zz = cell / plane;
-    const uint32_t r = cell - zz * plane;
-    const uint32_t yy = r / (uint32_t)b.nx;
-    x = (int)(r - yy * (uint32_t)b.nx);
-    y = (int)yy;
-    z = (int)zz;
-    return true;
-}
-
-// scratch (colour gradient only): phi of every domain's nodes, then rho_r,
-// each `scratch_n` values long; a domain's nodes start at its soff.  WALLS:
-// false when every domain is periodic in all three directions (the node code
-// then carries no bounce-back).  The FP32 colour-gradient and Shan-Chen
-// variants are held to 64 registers (4 CTAs of 256 or 8 of 128 per SM): their
-// first passes wait on the neighbours' loads and need the warps.  Measured on
-// the 64-domain sweeps: Shan-Chen 20.6 GLUPS at 64 registers, 19.0 at 96 and
-// 18.9 at 48; colour gradient 14.0 at 64, 13.7 at 80 and 12.3 at 48.
-template <int PHYS, typename S, typename C, bool WALLS>
-__global__ void __launch_bounds__(256, ((PHYS == LBM_PHYS_CGM || PHYS == LBM_PHYS_SC) && sizeof(S) == 4) ? 4 : 1)
-    batch_kernel(S* bufA, S* bufB, const BatchDomain* __restrict__ doms, int nd,
-                                                    uint32_t ntiles, long nsteps, int parity0, int dry,
-                                                    BarrierState* bs, unsigned long long timeout_ns, C* scratch,
-                                                    size_t scratch_n) {
-    for (long s = 0; s < nsteps; ++s) {
-        const int par = dry ? parity0 : (int)((parity0 + s) & 1);
-        const S* src = par ? bufB : bufA;
-        S* dst = par ? bufA : bufB;
-        if (PHYS == LBM_PHYS_SC) {
-            // pass 1: pseudopotential psi = 1 - exp(-rho) of every node
-            for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-                int d, x, y, z;
-                if (tile_node(doms, nd, t, d, x, y, z)) {
-                    const BatchDomain& D = doms[d];
-                    sc_psi_node<S, C, WALLS, false>(src + D.off, scratch + D.soff, D.sc, x, y, z);
-                }
-            }
-            if (!grid_barrier(bs, gridDim.x, timeout_ns)) return;
-            // pass 2: force, forced collision
-            for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-                int d, x, y, z;
-                if (tile_node(doms, nd, t, d, x, y, z)) {
-                    const BatchDomain& D = doms[d];
-                    sc_collide_node<S, C, WALLS, false>(src + D.off, dst + D.off, scratch + D.soff, D.sc, x, y, z);
-                }
-            }
-        } else if (PHYS == LBM_PHYS_CGM) {
-            // pass 1: order parameter and red density of every node
-            for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-                int d, x, y, z;
-                if (tile_node(doms, nd, t, d, x, y, z)) {
-                    const BatchDomain& D = doms[d];
-                    cgm_phi_node<S, C, WALLS, false>(src + D.off, scratch + D.soff, scratch + scratch_n + D.soff, D.cg,
-                                                    x, y, z);
-                }
-            }
-            if (!grid_barrier(bs, gridDim.x, timeout_ns)) return;
-            // pass 2: collision, perturbation, recolouring
-            for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-                int d, x, y, z;
-                if (tile_node(doms, nd, t, d, x, y, z)) {
-                    const BatchDomain& D = doms[d];
-                    cgm_collide_node<S, C, WALLS, false>(src + D.off, dst + D.off, scratch + D.soff,
-                                                        scratch + scratch_n + D.soff, D.cg, x, y, z);
-                }
-            }
-        } else {
-            for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-                int d, x, y, z;
-                if (tile_node(doms, nd, t, d, x, y, z)) {
-                    const BatchDomain& D = doms[d];
-                    if (PHYS == LBM_PHYS_MHD)
-                        mhd_node<S, C, WALLS, false>(src + D.off, dst + D.off, D.mh, x, y, z);
-                    else
-                        fluid_node<S, C, WALLS, false>(src + D.off, dst + D.off, D.fl, x, y, z);
-                }
-            }
-        }
-        if (s + 1 < nsteps && !grid_barrier(bs, gridDim.x, timeout_ns)) return;
-    }
+    const auto& D = tab.rec[lo];
+    const Box& b = D.a.box;
+    const uint32_t cell = (blockIdx.x - tab.tile0[lo]) * blockDim.x + threadIdx.x;
+    if (cell >= (uint32_t)b.n) return;
+    const uint32_t row = fast_div(cell, D.div_nx);
+    const int x = (int)(cell - row * (uint32_t)b.nx);
+    const int z = (int)fast_div(row, D.div_ny);
+    const int y = (int)(row - (uint32_t)z * (uint32_t)b.ny);
+    if constexpr (PHYS == LBM_PHYS_SC && PASS == 0)
+        sc_psi_node<S, C, WALLS>(src + D.off, scratch + D.soff, D.a, x, y, z);
+    else if constexpr (PHYS == LBM_PHYS_SC)
+        sc_collide_node<S, C, WALLS>(src + D.off, dst + D.off, scratch + D.soff, D.a, x, y, z);
+    else if constexpr (PHYS == LBM_PHYS_CGM && PASS == 0)
+        cgm_phi_node<S, C, WALLS>(src + D.off, scratch + D.soff, scratch + scratch_n + D.soff, D.a, x, y, z);
+    else if constexpr (PHYS == LBM_PHYS_CGM)
+        cgm_collide_node<S, C, WALLS>(src + D.off, dst + D.off, scratch + D.soff, scratch + scratch_n + D.soff,
+                                           D.a, x, y, z);
+    else if constexpr (PHYS == LBM_PHYS_MHD)
+        mhd_node<S, C, WALLS>(src + D.off, dst + D.off, D.a, x, y, z);
+    else
+        fluid_node<S, C, WALLS>(src + D.off, dst + D.off, D.a, x, y, z);
 }
 
 // Diagnostic: a barrier that waits for one CTA more than the grid has, so
@@ -213,155 +203,101 @@ struct BatchState {
     int nd = 0;
     std::vector<lbm_ctx*> views;
     std::vector<BatchDomain> doms;
-    BatchDomain* d_doms = nullptr;
-    BarrierState* d_bar = nullptr;
     uint32_t ntiles = 0;
     int threads = 256;
-    int ctas_per_sm = 0;  // 0 = as many as fit
-    int grid = 0;
-    int sms = 0;
-    cudaStream_t cap = nullptr;
-    cudaEvent_t ev_in = nullptr, ev_out = nullptr;
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};
-    long graph_n[2] = {-1, -1};
-    bool graph_ok = true;
     size_t state_elems = 0;
     size_t scratch_n = 0;  // values per scratch plane (colour gradient: all domains' nodes)
     bool walls = true;     // false: every domain periodic in x, y and z
-    unsigned long long timeout_ns = lbm::BARRIER_TIMEOUT_NS;
 };
 
 namespace {
 
-template <int PHYS, typename S, typename C>
-void* kernel_ptr(bool walls) {
-    return walls ? (void*)lbm::batch_kernel<PHYS, S, C, true> : (void*)lbm::batch_kernel<PHYS, S, C, false>;
-}
-
-void* batch_kernel_for(const lbm_ctx* c) {
-    const bool f64 = c->prec == LBM_FP64, w = c->batch->walls;
-    switch (c->physics) {
-        case LBM_PHYS_MHD:
-            return f64 ? kernel_ptr<LBM_PHYS_MHD, double, double>(w) : kernel_ptr<LBM_PHYS_MHD, float, float>(w);
-        case LBM_PHYS_CGM:
-            return f64 ? kernel_ptr<LBM_PHYS_CGM, double, double>(w) : kernel_ptr<LBM_PHYS_CGM, float, float>(w);
-        case LBM_PHYS_SC:
-            return f64 ? kernel_ptr<LBM_PHYS_SC, double, double>(w) : kernel_ptr<LBM_PHYS_SC, float, float>(w);
-        default:
-            return f64 ? kernel_ptr<0, double, double>(w) : kernel_ptr<0, float, float>(w);
-    }
-}
-
-void build_tiles(BatchState* B) {
-    uint32_t t = 0;
+// Tiles of the current CTA size.
+void configure(lbm_ctx* c) {
+    BatchState* B = c->batch;
+    B->ntiles = 0;
     for (auto& d : B->doms) {
-        d.tile0 = t;
         d.ntiles = (uint32_t)((d.fl.box.n + B->threads - 1) / B->threads);
-        t += d.ntiles;
+        B->ntiles += d.ntiles;
     }
-    B->ntiles = t;
+    c->block_x = B->threads;  // part of the launch shape that captured graphs are kept for
 }
 
-cudaError_t configure(lbm_ctx* c) {
+const lbm::FluidArgs& args_of(const BatchDomain& d, lbm::FluidArgs*) { return d.fl; }
+const lbm::MhdArgs& args_of(const BatchDomain& d, lbm::MhdArgs*) { return d.mh; }
+const lbm::CgmArgs& args_of(const BatchDomain& d, lbm::CgmArgs*) { return d.cg; }
+const lbm::ScArgs& args_of(const BatchDomain& d, lbm::ScArgs*) { return d.sc; }
+
+template <int PHYS, typename S, typename C, bool WALLS>
+cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
+    using Args = typename lbm::BatchArgs<PHYS>::T;
+    using Tab = lbm::BatchTab<Args>;
+    static_assert(sizeof(Tab) <= 32000, "kernel parameters are limited to 32,764 bytes");
     BatchState* B = c->batch;
-    build_tiles(B);
-    cudaError_t e = cudaMemcpyAsync(B->d_doms, B->doms.data(), sizeof(BatchDomain) * B->nd, cudaMemcpyHostToDevice,
-                                    c->stream);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_for(c), B->threads, 0);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    const int want = B->ctas_per_sm > 0 ? std::min(B->ctas_per_sm, per_sm) : per_sm;
-    long grid = (long)want * B->sms;
-    if (grid > (long)B->ntiles) grid = B->ntiles;
-    B->grid = (int)std::max(1L, grid);
-    for (int k = 0; k < 2; ++k) {
-        if (B->graph[k]) cudaGraphExecDestroy(B->graph[k]);
-        B->graph[k] = nullptr;
-        B->graph_n[k] = -1;
+    const int chunks = (B->nd + lbm::BATCH_TAB - 1) / lbm::BATCH_TAB;
+    std::vector<Tab> tabs((size_t)chunks);
+    std::vector<uint32_t> tiles((size_t)chunks, 0u);
+    for (int d = 0; d < B->nd; ++d) {
+        Tab& t = tabs[d / lbm::BATCH_TAB];
+        uint32_t& next = tiles[d / lbm::BATCH_TAB];
+        const int k = d % lbm::BATCH_TAB;
+        const BatchDomain& D = B->doms[d];
+        t.nd = k + 1;
+        t.tile0[k] = next;
+        t.rec[k].a = args_of(D, (Args*)nullptr);
+        t.rec[k].off = D.off;
+        t.rec[k].soff = D.soff;
+        t.rec[k].div_nx = D.div_nx;
+        t.rec[k].div_ny = D.div_ny;
+        next += D.ntiles;
     }
-    return cudaStreamSynchronize(c->stream);
-}
-
-cudaError_t launch_direct(lbm_ctx* c, cudaStream_t st, long n, int parity, int dry) {
-    BatchState* B = c->batch;
-    cudaError_t e = cudaMemsetAsync(B->d_bar, 0, sizeof(BarrierState), st);
-    if (e != cudaSuccess) return e;
-    void* a = c->buf[0];
-    void* b = c->buf[1];
-    BatchDomain* doms = B->d_doms;
-    int nd = B->nd;
-    uint32_t nt = B->ntiles;
-    BarrierState* bar = B->d_bar;
-    unsigned long long to = B->timeout_ns;
-    void* scratch = c->phi;  // colour gradient: phi and rho_r planes of all domains (else unused)
-    size_t scratch_n = B->scratch_n;
-    void* args[] = {&a, &b, &doms, &nd, &nt, &n, &parity, &dry, &bar, &to, &scratch, &scratch_n};
-    return cudaLaunchCooperativeKernel(batch_kernel_for(c), dim3(B->grid), dim3(B->threads), args, 0, st);
-}
-
-// Capture (once per starting parity and step count) and replay.
-cudaError_t run_batch(lbm_ctx* c, long n, int dry) {
-    BatchState* B = c->batch;
-    const int parity = c->cur;
-    cudaError_t e = cudaEventRecord(B->ev_in, c->stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(B->cap, B->ev_in, 0);
-    if (e != cudaSuccess) return e;
-    if (dry || !B->graph_ok) {
-        e = launch_direct(c, B->cap, n, parity, dry);
-    } else {
-        if (!B->graph[parity] || B->graph_n[parity] != n) {
-            if (B->graph[parity]) cudaGraphExecDestroy(B->graph[parity]);
-            B->graph[parity] = nullptr;
-            cudaGraph_t g = nullptr;
-            e = cudaStreamBeginCapture(B->cap, cudaStreamCaptureModeThreadLocal);
-            if (e == cudaSuccess) {
-                cudaError_t el = launch_direct(c, B->cap, n, parity, 0);
-                e = cudaStreamEndCapture(B->cap, &g);
-                if (e == cudaSuccess) e = el;
-            }
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&B->graph[parity], g, 0);
-            if (g) cudaGraphDestroy(g);
-            if (e != cudaSuccess) {
-                // capture of cooperative launches unavailable: launch directly from now on
-                cudaGetLastError();
-                B->graph_ok = false;
-                B->graph[parity] = nullptr;
-                e = launch_direct(c, B->cap, n, parity, 0);
-            } else {
-                B->graph_n[parity] = n;
-            }
+    for (long s = 0; s < n; ++s) {
+        const S* src = (const S*)c->buf[c->cur];
+        S* dst = (S*)c->buf[c->cur ^ 1];
+        for (int k = 0; k < chunks; ++k) {
+            if constexpr (PHYS == LBM_PHYS_SC || PHYS == LBM_PHYS_CGM)
+                lbm::batch_pass_kernel<PHYS, 0, S, C, WALLS><<<tiles[k], B->threads, 0, c->stream>>>(
+                    src, dst, (C*)c->phi, B->scratch_n, tabs[k]);
+            lbm::batch_pass_kernel<PHYS, 1, S, C, WALLS><<<tiles[k], B->threads, 0, c->stream>>>(
+                src, dst, (C*)c->phi, B->scratch_n, tabs[k]);
         }
-        if (B->graph_ok && B->graph[parity]) e = cudaGraphLaunch(B->graph[parity], B->cap);
+        if (!dry) c->cur ^= 1;
     }
-    if (e != cudaSuccess) return e;
-    e = cudaEventRecord(B->ev_out, B->cap);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, B->ev_out, 0);
-    if (e == cudaSuccess && !dry && (n & 1)) {
-        c->cur ^= 1;
-        for (lbm_ctx* v : B->views) v->cur = c->cur;
-    }
-    return e;
+    return cudaGetLastError();
+}
+
+template <int PHYS>
+cudaError_t steps_phys(lbm_ctx* c, long n, bool dry) {
+    if (c->prec == LBM_FP64)
+        return c->batch->walls ? steps_t<PHYS, double, double, true>(c, n, dry)
+                               : steps_t<PHYS, double, double, false>(c, n, dry);
+    return c->batch->walls ? steps_t<PHYS, float, float, true>(c, n, dry)
+                           : steps_t<PHYS, float, float, false>(c, n, dry);
 }
 
 }  // namespace
 
 namespace lbm {
 
-// Timed dry run of the persistent kernel (state unchanged) for the autotuner.
-cudaError_t batch_time_config(lbm_ctx* c, int threads, int ctas_per_sm, long steps, float* ms) {
-    BatchState* B = c->batch;
-    B->threads = threads;
-    B->ctas_per_sm = ctas_per_sm;
-    cudaError_t e = configure(c);
+cudaError_t batch_step(lbm_ctx* c, long n, bool dry) {
+    switch (c->physics) {
+        case LBM_PHYS_MHD: return steps_phys<LBM_PHYS_MHD>(c, n, dry);
+        case LBM_PHYS_CGM: return steps_phys<LBM_PHYS_CGM>(c, n, dry);
+        case LBM_PHYS_SC: return steps_phys<LBM_PHYS_SC>(c, n, dry);
+        default: return steps_phys<LBM_PHYS_FLUID>(c, n, dry);
+    }
+}
+
+// Timed dry run (state unchanged) for the autotuner.
+cudaError_t batch_time_config(lbm_ctx* c, int threads, long steps, float* ms) {
+    cudaError_t e = batch_apply_config(c, threads);
     if (e != cudaSuccess) return e;
     cudaEvent_t a, b;
     cudaEventCreate(&a);
     cudaEventCreate(&b);
-    e = run_batch(c, 2, 1);  // warm-up
+    e = batch_step(c, 2, true);  // warm-up
     if (e == cudaSuccess) e = cudaEventRecord(a, c->stream);
-    if (e == cudaSuccess) e = run_batch(c, steps, 1);
+    if (e == cudaSuccess) e = batch_step(c, steps, true);
     if (e == cudaSuccess) e = cudaEventRecord(b, c->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(b);
     if (e == cudaSuccess) e = cudaEventElapsedTime(ms, a, b);
@@ -370,20 +306,16 @@ cudaError_t batch_time_config(lbm_ctx* c, int threads, int ctas_per_sm, long ste
     return e;
 }
 
-cudaError_t batch_apply_config(lbm_ctx* c, int threads, int ctas_per_sm) {
+cudaError_t batch_apply_config(lbm_ctx* c, int threads) {
+    if (threads < BATCH_MIN_THREADS || threads > 256 || threads % 32 != 0) return cudaErrorInvalidValue;
     c->batch->threads = threads;
-    c->batch->ctas_per_sm = ctas_per_sm;
-    return configure(c);
+    configure(c);
+    return cudaSuccess;
 }
 
 void batch_destroy(lbm_ctx* c) {
     BatchState* B = c->batch;
     if (!B) return;
-    for (int k = 0; k < 2; ++k)
-        if (B->graph[k]) cudaGraphExecDestroy(B->graph[k]);
-    if (B->ev_in) cudaEventDestroy(B->ev_in);
-    if (B->ev_out) cudaEventDestroy(B->ev_out);
-    if (B->cap) cudaStreamDestroy(B->cap);
     for (lbm_ctx* v : B->views) delete v;
     delete B;
     c->batch = nullptr;
@@ -464,10 +396,7 @@ lbm_status lbm_batch_create(lbm_ctx** out, int ndomains, const lbm_grid* grids, 
     B->scratch_n = cells;
     B->walls = false;
     for (int d = 0; d < ndomains; ++d) B->walls = B->walls || (grids[d].periodic_mask & 7u) != 7u;
-    cudaDeviceGetAttribute(&B->sms, cudaDevAttrMultiProcessorCount, c->device);
-    cudaError_t e = cudaStreamCreateWithFlags(&B->cap, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&B->ev_in, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&B->ev_out, cudaEventDisableTiming);
+    cudaError_t e = cudaSuccess;
     size_t off = 0, uoff = 0, soff = 0;
     for (int d = 0; d < ndomains && e == cudaSuccess; ++d) {
         const lbm_grid& g = grids[d];
@@ -478,6 +407,8 @@ lbm_status lbm_batch_create(lbm_ctx** out, int ndomains, const lbm_grid* grids, 
         D.fl.box.nz = g.nz;
         D.fl.box.periodic = g.periodic_mask & 7u;
         D.fl.box.n = (size_t)g.nx * g.ny * g.nz;
+        D.div_nx = lbm::make_fast_div((uint32_t)g.nx);
+        D.div_ny = lbm::make_fast_div((uint32_t)g.ny);
         D.fl.omega = relax[d].omega;
         for (int a = 0; a < 3; ++a) {
             D.fl.g[a] = forcing ? forcing[d].g[a] : 0.0;
@@ -545,7 +476,7 @@ lbm_status lbm_batch_create(lbm_ctx** out, int ndomains, const lbm_grid* grids, 
         uoff += 3 * D.fl.box.n;
         soff += D.fl.box.n;
     }
-    if (e == cudaSuccess) e = configure(c);
+    if (e == cudaSuccess) configure(c);
     // rest state for every domain
     for (int d = 0; d < ndomains && e == cudaSuccess; ++d) {
         lbm_ctx* v = B->views[d];
@@ -573,7 +504,8 @@ lbm_status lbm_batch_domain(lbm_ctx* c, int d, lbm_ctx** view) {
 lbm_status lbm_batch_step(lbm_ctx* c, long n) {
     if (!c || !c->batch || n < 0) return LBM_ERR_ARG;
     if (n == 0) return LBM_OK;
-    cudaError_t e = run_batch(c, n, 0);
+    const cudaError_t e = lbm_internal_run_steps(c, n);
+    for (lbm_ctx* v : c->batch->views) v->cur = c->cur;
     if (e != cudaSuccess) {
         c->err = std::string("lbm_batch_step: ") + cudaGetErrorString(e);
         return LBM_ERR_CUDA;
@@ -584,8 +516,8 @@ lbm_status lbm_batch_step(lbm_ctx* c, long n) {
 lbm_status lbm_batch_info(const lbm_ctx* c, int* threads, int* grid, int* graph, long* tiles) {
     if (!c || !c->batch) return LBM_ERR_ARG;
     if (threads) *threads = c->batch->threads;
-    if (grid) *grid = c->batch->grid;
-    if (graph) *graph = c->batch->graph_ok ? 1 : 0;
+    if (grid) *grid = (int)c->batch->ntiles;
+    if (graph) *graph = c->graph_failed ? 0 : 1;
     if (tiles) *tiles = (long)c->batch->ntiles;
     return LBM_OK;
 }
@@ -613,33 +545,4 @@ lbm_status lbm_barrier_selftest(double timeout_s, int* observed) {
 
 }  // extern "C"
 
-lbm_status lbm_internal_batch_status(lbm_ctx* c) {
-    if (!c || !c->batch) return LBM_OK;
-    BarrierState h;
-    cudaError_t e = cudaMemcpy(&h, c->batch->d_bar, sizeof(h), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return LBM_ERR_CUDA;
-    if (h.err == (int)LBM_ERR_TIMEOUT) {
-        c->err = "batch grid barrier wait exceeded its limit";
-        return LBM_ERR_TIMEOUT;
-    }
-    return LBM_OK;
-}
-
 size_t lbm_internal_batch_state_elems(const lbm_ctx* c) { return c->batch ? c->batch->state_elems : 0; }
-
-lbm_status lbm_internal_alloc_batch_tables(lbm_ctx* c) {
-    BatchState* B = c->batch;
-    B->d_doms = (BatchDomain*)lbm_internal_dev_alloc(c, sizeof(BatchDomain) * (size_t)B->nd);
-    B->d_bar = (BarrierState*)lbm_internal_dev_alloc(c, sizeof(BarrierState));
-    if (!B->d_doms || !B->d_bar) return LBM_ERR_OOM;
-    return LBM_OK;
-}
-
-void lbm_internal_free_batch_tables(lbm_ctx* c) {
-    BatchState* B = c->batch;
-    if (!B) return;
-    lbm_internal_dev_free(c, B->d_doms);
-    lbm_internal_dev_free(c, B->d_bar);
-    B->d_doms = nullptr;
-    B->d_bar = nullptr;
-}

@@ -67,6 +67,7 @@ int slab_planes(const lbm_ctx* c) {
 }
 
 cudaError_t phys_step(lbm_ctx* c, long n, bool dry = false) {
+    if (c->batch) return lbm::batch_step(c, n, dry);
     if (c->q == 27) return lbm::q27_step(c, n, dry);
     switch (c->physics) {
         case LBM_PHYS_FLUID: return lbm::fluid_step(c, n, dry);
@@ -157,6 +158,7 @@ cudaGraphExec_t step_graph(lbm_ctx* c) {
         cudaGetLastError();
         c->step_graph[k] = nullptr;
     }
+    c->graph_failed = e != cudaSuccess;
     cudaThreadExchangeStreamCaptureMode(&mode);
     return c->step_graph[k];
 }
@@ -305,16 +307,14 @@ void lbm_internal_get_allocator(lbm_alloc_fn* a, lbm_free_fn* r, void** user) {
     *user = g_user;
 }
 void lbm_internal_dev_free(lbm_ctx* c, void* p) { dev_free(c, p); }
-void lbm_internal_release(lbm_ctx* c) {
-    if (c->batch) lbm_internal_free_batch_tables(c);
-    release_all(c);
-}
+void lbm_internal_release(lbm_ctx* c) { release_all(c); }
 cudaError_t lbm_internal_init_rest(lbm_ctx* c) { return init_in_place(c, lbm::FieldsIn(), true); }
 cudaError_t lbm_internal_step(lbm_ctx* c, long n, bool dry) { return phys_step(c, n, dry); }
+cudaError_t lbm_internal_run_steps(lbm_ctx* c, long n) { return run_steps(c, n); }
 
 // Buffers of a batch: two state copies of `state_elems` values, the residual
 // velocity of every node, reduction scratch, a staging slab sized for the
-// largest domain plane, and the device tables of the persistent kernel.
+// largest domain plane.
 lbm_status lbm_internal_alloc_batch(lbm_ctx* c, size_t state_elems, size_t cells, size_t max_plane) {
     c->alloc = g_alloc;
     c->release = g_release;
@@ -342,7 +342,7 @@ lbm_status lbm_internal_alloc_batch(lbm_ctx* c, size_t state_elems, size_t cells
         c->result_host = nullptr;
         return LBM_ERR_OOM;
     }
-    return lbm_internal_alloc_batch_tables(c);
+    return LBM_OK;
 }
 
 extern "C" {
@@ -451,7 +451,6 @@ lbm_status lbm_create(lbm_ctx** out, const lbm_grid* grid, lbm_lattice lattice, 
     size_t kz = SLAB_TARGET_CELLS / plane;
     if (kz < 1) kz = 1;
     if (kz > (size_t)grid->nz) kz = (size_t)grid->nz;
-    const int nzs = (int)kz;
     c->staging_cells = plane * kz;
     c->buf[0] = dev_alloc(c, state);
     c->buf[1] = dev_alloc(c, state);
@@ -498,10 +497,7 @@ lbm_status lbm_create(lbm_ctx** out, const lbm_grid* grid, lbm_lattice lattice, 
 void lbm_destroy(lbm_ctx* c) {
     if (!c || !c->owns) return;  // views of a batch are owned by the batch
     cudaStreamSynchronize(c->stream);
-    if (c->batch) {
-        lbm_internal_free_batch_tables(c);
-        lbm::batch_destroy(c);
-    }
+    if (c->batch) lbm::batch_destroy(c);
     release_all(c);
     delete c;
 }
@@ -585,9 +581,7 @@ lbm_status lbm_sync(lbm_ctx* c) {
     if (!c) return LBM_ERR_ARG;
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "lbm_sync");
-    const lbm_status st = device_status(c);
-    if (st != LBM_OK) return st;
-    return lbm_internal_batch_status(c);
+    return device_status(c);
 }
 
 lbm_status lbm_fields(lbm_ctx* c, double* rho, double* u, double* phase, double* B) {

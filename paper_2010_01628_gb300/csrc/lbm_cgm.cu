@@ -1,7 +1,7 @@
 // lbm_cgm.cu -- colour-gradient two-phase step (App. E of arXiv:2010.01628):
 // the single-domain kernels (two passes per step), initialisation, fields and
 // reductions.  The two passes take the same steps as cgm_phi_node and
-// cgm_collide_node of lbm_cgm.cuh (which the batched persistent kernel uses),
+// cgm_collide_node of lbm_cgm.cuh (which the batched kernels uses),
 // written out in the kernels: built on those node functions, the
 // single-domain step compiled to code 8 % slower (16.9 against 18.5 GLUPS on
 // the 256^3 droplets, GB300).

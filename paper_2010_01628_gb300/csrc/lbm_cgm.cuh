@@ -1,7 +1,7 @@
 // lbm_cgm.cuh -- device side of the colour-gradient two-phase step (App. E of
 // arXiv:2010.01628): the pull, moments, collision, gradient, perturbation and
 // recolouring shared by the single-domain kernels (lbm_cgm.cu) and the
-// batched persistent kernel (lbm_batch.cu), and the node functions of the two
+// batched kernels (lbm_batch.cu), and the node functions of the two
 // passes that the batch runs.
 //
 // Two passes per step.  Pass 1 pulls the populations of every node and writes
@@ -76,12 +76,9 @@ __device__ __forceinline__ C red_pop(C a, C vx, C vy, C vz, C f) {
     return fma_rn(a, f, (C)kappa * cv);
 }
 
-// NC: read-only path; else a plain cached load (persistent kernels whose
-// sources are rewritten between grid-wide barriers).
-template <typename S, typename C, bool NC = true>
+template <typename S, typename C>
 __device__ __forceinline__ C cgm_ld(const S* __restrict__ src, size_t n, int plane, uint32_t cell) {
-    if (NC) return (C)Store<S>::load(src + (size_t)plane * n + cell);
-    return (C)Store<S>::load_coherent(src + (size_t)plane * n + cell);
+    return (C)Store<S>::load(src + (size_t)plane * n + cell);
 }
 
 // All 19 pulled populations of a node, f_I(x) = f*_I(x - c_I), and their red
@@ -94,7 +91,7 @@ template <typename C>
 struct RedSrc {
     C a, vx, vy, vz;
 };
-template <typename S, typename C, bool WALLS, int I, bool NC = true>
+template <typename S, typename C, bool WALLS, int I>
 __device__ __forceinline__ void cgm_load(const S* __restrict__ src, const Box& b, const Nbr& q, int x, int y, int z,
                                          uint32_t self, C& f, RedSrc<C>& g) {
     uint32_t cell;
@@ -102,19 +99,19 @@ __device__ __forceinline__ void cgm_load(const S* __restrict__ src, const Box& b
     constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
     const bool bb = WALLS && wall;
     const uint32_t at = bb ? self : cell;
-    f = cgm_ld<S, C, NC>(src, b.n, bb ? opp_of(I) : I, at);
-    g.a = cgm_ld<S, C, NC>(src, b.n, CGM_FRAC, at);
-    g.vx = cx ? cgm_ld<S, C, NC>(src, b.n, CGM_VX, at) : (C)0;
-    g.vy = cy ? cgm_ld<S, C, NC>(src, b.n, CGM_VY, at) : (C)0;
-    g.vz = cz ? cgm_ld<S, C, NC>(src, b.n, CGM_VZ, at) : (C)0;
+    f = cgm_ld<S, C>(src, b.n, bb ? opp_of(I) : I, at);
+    g.a = cgm_ld<S, C>(src, b.n, CGM_FRAC, at);
+    g.vx = cx ? cgm_ld<S, C>(src, b.n, CGM_VX, at) : (C)0;
+    g.vy = cy ? cgm_ld<S, C>(src, b.n, CGM_VY, at) : (C)0;
+    g.vz = cz ? cgm_ld<S, C>(src, b.n, CGM_VZ, at) : (C)0;
 }
-template <typename S, typename C, bool WALLS, bool NC = true>
+template <typename S, typename C, bool WALLS>
 __device__ __forceinline__ void cgm_pull_all(const S* __restrict__ src, const Box& b, const Nbr& q, int x, int y,
                                              int z, uint32_t self, C (&f)[Q], C (&r)[Q]) {
     RedSrc<C> g[Q];
-    f[0] = cgm_ld<S, C, NC>(src, b.n, 0, self);
-    r[0] = cgm_ld<S, C, NC>(src, b.n, CGM_RED0, self);
-#define LBM_CL(I) cgm_load<S, C, WALLS, I, NC>(src, b, q, x, y, z, self, f[I], g[I]);
+    f[0] = cgm_ld<S, C>(src, b.n, 0, self);
+    r[0] = cgm_ld<S, C>(src, b.n, CGM_RED0, self);
+#define LBM_CL(I) cgm_load<S, C, WALLS, I>(src, b, q, x, y, z, self, f[I], g[I]);
     LBM_CL(1) LBM_CL(2) LBM_CL(3) LBM_CL(4) LBM_CL(5) LBM_CL(6) LBM_CL(7) LBM_CL(8) LBM_CL(9) LBM_CL(10)
     LBM_CL(11) LBM_CL(12) LBM_CL(13) LBM_CL(14) LBM_CL(15) LBM_CL(16) LBM_CL(17) LBM_CL(18)
 #undef LBM_CL
@@ -187,14 +184,14 @@ __device__ __forceinline__ void cgm_collide(C (&f)[Q], const Moments<C>& m, cons
 }
 
 // Pass 1 at one node: phi and rho_r from its pulled populations.
-template <typename S, typename C, bool WALLS, bool NC>
+template <typename S, typename C, bool WALLS>
 __device__ __forceinline__ void cgm_phi_node(const S* __restrict__ src, C* __restrict__ phi, C* __restrict__ rho_red,
                                              const CgmArgs& p, int x, int y, int z) {
     const Box& b = p.box;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
     C f[Q], r[Q];
-    cgm_pull_all<S, C, WALLS, NC>(src, b, q, x, y, z, self, f, r);
+    cgm_pull_all<S, C, WALLS>(src, b, q, x, y, z, self, f, r);
     const C sr = colour_sum(r), st = colour_sum(f);
     phi[self] = (sr - (st - sr)) / st;
     rho_red[self] = sr;
@@ -202,16 +199,16 @@ __device__ __forceinline__ void cgm_phi_node(const S* __restrict__ src, C* __res
 
 // grad phi = (1/c_s^2) sum_i w_i c_i phi(x + c_i): the axis and the diagonal
 // neighbours are summed apart and scaled once (3/18 and 3/36).
-template <typename C, bool WALLS, bool NC = true>
+template <typename C, bool WALLS>
 __device__ __forceinline__ void grad_phi(const C* __restrict__ phi, const Box& b, const Nbr& q, int x, int y, int z,
                                          uint32_t self, C (&gr)[3]) {
-    const C own = NC ? phi[self] : ld_coherent(phi + self);
+    const C own = phi[self];
     C ax = (C)0, ay = (C)0, az = (C)0, dx = (C)0, dy = (C)0, dz = (C)0;
 #define LBM_GP(I)                                                                           \
     {                                                                                       \
         constexpr int ex = cx_of(I), ey = cy_of(I), ez = cz_of(I);                          \
         constexpr bool axis = ex * ex + ey * ey + ez * ez == 1;                             \
-        const C t = field_nbr<C, WALLS, I, NC>(phi, b, q, x, y, z, own);                           \
+        const C t = field_nbr<C, WALLS, I>(phi, b, q, x, y, z, own);                           \
         if (ex) { if (axis) ax += ex > 0 ? t : -t; else dx += ex > 0 ? t : -t; }            \
         if (ey) { if (axis) ay += ey > 0 ? t : -t; else dy += ey > 0 ? t : -t; }            \
         if (ez) { if (axis) az += ez > 0 ? t : -t; else dz += ez > 0 ? t : -t; }            \
@@ -251,7 +248,7 @@ __device__ __forceinline__ void perturb_store(S* __restrict__ dst, size_t n, uin
 }
 
 // Pass 2 at one node: pull, collide the totals, perturb, recolour.
-template <typename S, typename C, bool WALLS, bool NC>
+template <typename S, typename C, bool WALLS>
 __device__ __forceinline__ void cgm_collide_node(const S* __restrict__ src, S* __restrict__ dst,
                                                  const C* __restrict__ phi, const C* __restrict__ rho_red,
                                                  const CgmArgs& p, int x, int y, int z) {
@@ -259,12 +256,12 @@ __device__ __forceinline__ void cgm_collide_node(const S* __restrict__ src, S* _
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
     C f[Q];
-    gather19<S, C, WALLS, NC>(src, b, q, x, y, z, self, (C)0, (C)0, (C)0, f);
+    gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)0, (C)0, (C)0, f);
     const Moments<C> m = moments19(f);
-    const CgmNode<C> s = cgm_macro<C>(f, m, NC ? rho_red[self] : ld_coherent(rho_red + self), p);
+    const CgmNode<C> s = cgm_macro<C>(f, m, rho_red[self], p);
     cgm_collide<C>(f, m, s, (C)p.omega);
     C gr[3];
-    grad_phi<C, WALLS, NC>(phi, b, q, x, y, z, self, gr);
+    grad_phi<C, WALLS>(phi, b, q, x, y, z, self, gr);
     const C n2 = gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2];
     const C nrm = sqrt(n2);
     // each colour's operator carries A_k/2 = A/2; together they perturb the total by

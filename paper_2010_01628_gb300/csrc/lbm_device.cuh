@@ -52,34 +52,11 @@ struct Box {
 // Storage formats.  FP64/FP32 hold f - w (shift by the rest state of rho0 = 1);
 // the 16-bit formats hold (f - w)/w so every direction uses the same range.
 template <typename S> struct Store;
-// Plain (weak, L1-cached) global loads in inline PTX, so that a const
-// __restrict__ source cannot be turned into a read-only (.nc) load.
-__device__ __forceinline__ double ld_coherent(const double* p) {
-    double v;
-    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ float ld_coherent(const float* p) {
-    float v;
-    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ unsigned short ld_coherent(const unsigned short* p) {
-    unsigned short v;
-    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
-    return v;
-}
-// load(): read-only path (ld.global.nc), valid when the source buffer is not
-// written during the kernel.  load_coherent(): a plain cached load for
-// persistent kernels that rewrite their sources between grid-wide barriers:
-// the barrier's GPU-scope fences order it after the other CTAs' stores (the
-// read-only path has no such guarantee), and it still caches in L1, which the
-// neighbours' shared source values of the colour-gradient pull need.
+// load(): read-only path (ld.global.nc): no kernel writes the copy it reads.
 template <> struct Store<double> {
     static constexpr bool scaled = false;
     __device__ static __forceinline__ double to_float(double v) { return v; }
     __device__ static __forceinline__ double load(const double* p) { return __ldg(p); }
-    __device__ static __forceinline__ double load_coherent(const double* p) { return ld_coherent(p); }
     __device__ static __forceinline__ void store(double* p, double v) { __stcs(p, v); }
 };
 template <> struct Store<float> {
@@ -92,37 +69,25 @@ template <> struct Store<float> {
         asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
         return v;
     }
-    // cached, with the same prefetch size
-    __device__ static __forceinline__ float load_coherent(const float* p) {
-        float v;
-        asm volatile("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
-        return v;
-    }
     __device__ static __forceinline__ void store(float* p, float v) { __stcs(p, v); }
 };
 template <> struct Store<__half> {
     static constexpr bool scaled = true;
     __device__ static __forceinline__ float to_float(__half v) { return __half2float(v); }
     __device__ static __forceinline__ float load(const __half* p) { return __half2float(__ldg(p)); }
-    __device__ static __forceinline__ float load_coherent(const __half* p) {
-        return __half2float(__ushort_as_half(ld_coherent(reinterpret_cast<const unsigned short*>(p))));
-    }
     __device__ static __forceinline__ void store(__half* p, float v) { *p = __float2half_rn(v); }
 };
 template <> struct Store<__nv_bfloat16> {
     static constexpr bool scaled = true;
     __device__ static __forceinline__ float to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
     __device__ static __forceinline__ float load(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
-    __device__ static __forceinline__ float load_coherent(const __nv_bfloat16* p) {
-        return __uint_as_float((uint32_t)ld_coherent(reinterpret_cast<const unsigned short*>(p)) << 16);
-    }
     __device__ static __forceinline__ void store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 };
 
 // Read the shifted population f - w of direction I from storage.
-template <typename S, typename C, int I, bool NC = true>
+template <typename S, typename C, int I>
 __device__ __forceinline__ C load_shifted(const S* p) {
-    C v = NC ? (C)Store<S>::load(p) : (C)Store<S>::load_coherent(p);
+    C v = (C)Store<S>::load(p);
     if (Store<S>::scaled) v *= (C)w_of(I);
     return v;
 }
@@ -173,15 +138,15 @@ __device__ __forceinline__ bool pull_source(const Box& b, const Nbr& q, int x, i
 }
 
 // One pulled population f_I(x) = f*_I(x - c_I) (shifted).
-template <typename S, typename C, bool WALLS, int I, bool NC>
+template <typename S, typename C, bool WALLS, int I>
 __device__ __forceinline__ C gather_one(const S* __restrict__ src, const Box& b, const Nbr& q, int x, int y, int z,
                                         uint32_t self, C lx, C ly, C lz) {
     uint32_t cell;
     const bool wall = pull_source<I>(b, q, x, y, z, cell);
-    if (!WALLS) return load_shifted<S, C, I, NC>(src + (size_t)I * b.n + cell);
+    if (!WALLS) return load_shifted<S, C, I>(src + (size_t)I * b.n + cell);
     // behind a wall: the node's own opposite population (same weight), chosen by
     // address rather than by a branch (+9% on the walled batch, +10% Rayleigh-Taylor)
-    C v = load_shifted<S, C, I, NC>(src + (size_t)(wall ? opp_of(I) : I) * b.n + (wall ? self : cell));
+    C v = load_shifted<S, C, I>(src + (size_t)(wall ? opp_of(I) : I) * b.n + (wall ? self : cell));
     if (cy_of(I) < 0 && q.wyp)  // source beyond the +y face: the moving lid
         v += (C)(6.0 * w_of(I)) * ((C)cx_of(I) * lx + (C)cy_of(I) * ly + (C)cz_of(I) * lz);
     return v;
@@ -191,10 +156,10 @@ __device__ __forceinline__ C gather_one(const S* __restrict__ src, const Box& b,
 // selects the variant with bounce-back; a pull from behind a wall reads the
 // node's own post-collision population of the opposite direction, plus
 // 6 w_i c_i . u_lid when the wall crossed is the moving +y lid.
-template <typename S, typename C, bool WALLS, bool NC = true>
+template <typename S, typename C, bool WALLS>
 __device__ __forceinline__ void gather19(const S* __restrict__ src, const Box& b, const Nbr& q, int x, int y, int z,
                                          uint32_t self, C lx, C ly, C lz, C (&f)[Q]) {
-#define LBM_G(I) f[I] = gather_one<S, C, WALLS, I, NC>(src, b, q, x, y, z, self, lx, ly, lz);
+#define LBM_G(I) f[I] = gather_one<S, C, WALLS, I>(src, b, q, x, y, z, self, lx, ly, lz);
     LBM_G(0) LBM_G(1) LBM_G(2) LBM_G(3) LBM_G(4) LBM_G(5) LBM_G(6) LBM_G(7) LBM_G(8) LBM_G(9) LBM_G(10)
     LBM_G(11) LBM_G(12) LBM_G(13) LBM_G(14) LBM_G(15) LBM_G(16) LBM_G(17) LBM_G(18)
 #undef LBM_G
@@ -203,10 +168,8 @@ __device__ __forceinline__ void gather19(const S* __restrict__ src, const Box& b
 // Value of a node field v at x + c_I; a neighbour behind a wall contributes
 // the node's own value `own`.  WALLS = false (every axis periodic) carries none
 // of the wall predicates, which cost the issue-bound collide passes about 90 of
-// their 760 (Shan-Chen) and 1004 (colour gradient) instructions.  NC: read-only path (the field is not written
-// during the kernel); else a plain load (persistent kernels that rewrite the
-// field between grid-wide barriers; see Store::load_coherent).
-template <typename C, bool WALLS, int I, bool NC = true>
+// their 760 (Shan-Chen) and 1004 (colour gradient) instructions.
+template <typename C, bool WALLS, int I>
 __device__ __forceinline__ C field_nbr(const C* __restrict__ v, const Box& b, const Nbr& q, int x, int y, int z,
                                        C own) {
     constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
@@ -217,19 +180,19 @@ __device__ __forceinline__ C field_nbr(const C* __restrict__ v, const Box& b, co
                                 (cz > 0 && q.wzp) || (cz < 0 && q.wzm));
     if (wall) return own;
     const C* a = v + ((uint32_t)sz * (uint32_t)b.ny + (uint32_t)sy) * (uint32_t)b.nx + (uint32_t)sx;
-    return NC ? __ldg(a) : ld_coherent(a);
+    return __ldg(a);
 }
 
 // s = sum_i w_i c_i v(x + c_i) over the 18 moving directions: the lattice
 // first moment of a node field (times 1/c_s^2 the isotropic gradient of the
 // colour-gradient model; times -G psi(x) the Shan-Chen force).
-template <typename C, bool WALLS, bool NC = true>
+template <typename C, bool WALLS>
 __device__ __forceinline__ void lattice_first_moment(const C* __restrict__ v, const Box& b, const Nbr& q, int x,
                                                      int y, int z, C own, C (&s)[3]) {
     C gx = (C)0, gy = (C)0, gz = (C)0;
 #define LBM_FM(I)                                                           \
     {                                                                       \
-        const C t = field_nbr<C, WALLS, I, NC>(v, b, q, x, y, z, own) * (C)w_of(I); \
+        const C t = field_nbr<C, WALLS, I>(v, b, q, x, y, z, own) * (C)w_of(I); \
         if (cx_of(I)) gx += (C)cx_of(I) * t;                                \
         if (cy_of(I)) gy += (C)cy_of(I) * t;                                \
         if (cz_of(I)) gz += (C)cz_of(I) * t;                                \

@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(256) fluid_step_kernel(const S* __restrict__ s
                                                          FluidArgs p) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.box.nx) return;
-    fluid_node<S, C, WALLS, true, RM>(src, dst, p, x, blockIdx.y, blockIdx.z);
+    fluid_node<S, C, WALLS, RM>(src, dst, p, x, blockIdx.y, blockIdx.z);
 }
 
 // Channels (x and z periodic, walls on y, ny >= 3) step in two launches: the
@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(256) fluid_step_interior_kernel(const S* __res
                                                                   FluidArgs p) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.box.nx) return;
-    fluid_node<S, C, false, true>(src, dst, p, x, blockIdx.y + 1, blockIdx.z);
+    fluid_node<S, C, false>(src, dst, p, x, blockIdx.y + 1, blockIdx.z);
 }
 
 // The wall rows y = 0 (blockIdx.y = 0) and y = ny - 1 (blockIdx.y = 1) of a
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(256) fluid_step_wallrows_kernel(const S* __res
     const int y = blockIdx.y == 0 ? 0 : b.ny - 1, z = blockIdx.z;
     if (x >= b.nx) return;
     if (!REG) {
-        fluid_node<S, C, true, true>(src, dst, p, x, y, z);
+        fluid_node<S, C, true>(src, dst, p, x, y, z);
         return;
     }
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;

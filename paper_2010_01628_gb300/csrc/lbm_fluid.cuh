@@ -1,5 +1,5 @@
 // lbm_fluid.cuh -- per-node single-phase update (Sec. II of arXiv:2010.01628),
-// shared by the single-domain kernels and the batched persistent kernel.
+// shared by the single-domain and the batched kernels.
 #pragma once
 
 #include "lbm_device.cuh"
@@ -93,16 +93,15 @@ __device__ __forceinline__ void gather_regularized(const S* __restrict__ src, co
 }
 
 // One node: pull (stream + boundaries), moments, forced CM collision, store.
-// NC selects the read-only load path (sources not written during the kernel);
-// RM the raw-moment variant of App. C.
-template <typename S, typename C, bool WALLS, bool NC, bool RM = false>
+// RM: the raw-moment variant of App. C.
+template <typename S, typename C, bool WALLS, bool RM = false>
 __device__ __forceinline__ void fluid_node(const S* __restrict__ src, S* __restrict__ dst, const FluidArgs& p, int x,
                                            int y, int z) {
     const Box& b = p.box;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
     C f[Q];
-    gather19<S, C, WALLS, NC>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
+    gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
     const Moments<C> m = moments19(f);
     const Macro<C> a = fluid_macro(m, (C)p.g[0], (C)p.g[1], (C)p.g[2]);
     if (RM)

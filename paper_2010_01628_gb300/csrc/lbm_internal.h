@@ -51,6 +51,7 @@ struct lbm_ctx {
     int* status = nullptr;  // device status word written by bounded waits
     bool bounded_waits = false;  // a kernel that may write `status` has been launched
     cudaGraphExec_t step_graph[2] = {nullptr, nullptr};  // STEP_GRAPH steps starting from buf[0] / buf[1]
+    bool graph_failed = false;  // a capture did not succeed: steps are launched one by one
     int step_graph_shape[6] = {-1, -1, -1, -1, -1, -1};  // launch shape the graphs were captured with
     std::string err;
     bool owns = true;            // false for the per-domain views of a batch
@@ -66,10 +67,8 @@ lbm_status lbm_internal_alloc_batch(lbm_ctx* c, size_t state_elems, size_t cells
 void lbm_internal_release(lbm_ctx* c);
 cudaError_t lbm_internal_init_rest(lbm_ctx* c);
 cudaError_t lbm_internal_step(lbm_ctx* c, long n, bool dry);
-lbm_status lbm_internal_batch_status(lbm_ctx* c);
-lbm_status lbm_internal_alloc_batch_tables(lbm_ctx* c);
+cudaError_t lbm_internal_run_steps(lbm_ctx* c, long n);
 size_t lbm_internal_batch_state_elems(const lbm_ctx* c);
-void lbm_internal_free_batch_tables(lbm_ctx* c);
 
 namespace lbm {
 
@@ -138,9 +137,11 @@ cudaError_t sc_reduce(lbm_ctx* c, bool record);
 // Sum RED_BLOCKS partials into c->result (deterministic order).
 cudaError_t reduce_finalize(lbm_ctx* c);
 
-// Batched persistent kernel (lbm_batch.cu).
-cudaError_t batch_time_config(lbm_ctx* c, int threads, int ctas_per_sm, long steps, float* ms);
-cudaError_t batch_apply_config(lbm_ctx* c, int threads, int ctas_per_sm);
+// Batched step (lbm_batch.cu): CTAs of BATCH_MIN_THREADS to 256 threads.
+constexpr int BATCH_MIN_THREADS = 128;
+cudaError_t batch_step(lbm_ctx* c, long n, bool dry = false);
+cudaError_t batch_time_config(lbm_ctx* c, int threads, long steps, float* ms);
+cudaError_t batch_apply_config(lbm_ctx* c, int threads);
 void batch_destroy(lbm_ctx* c);
 
 inline dim3 step_grid(const Box& b, int bx) { return dim3((unsigned)((b.nx + bx - 1) / bx), (unsigned)b.ny, (unsigned)b.nz); }

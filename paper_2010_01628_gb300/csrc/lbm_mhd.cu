@@ -11,7 +11,7 @@ template <typename S, typename C, bool WALLS>
 __global__ void __launch_bounds__(256) mhd_step_kernel(const S* __restrict__ src, S* __restrict__ dst, MhdArgs p) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.box.nx) return;
-    mhd_node<S, C, WALLS, true>(src, dst, p, x, blockIdx.y, blockIdx.z);
+    mhd_node<S, C, WALLS>(src, dst, p, x, blockIdx.y, blockIdx.z);
 }
 
 template <typename S, typename C>

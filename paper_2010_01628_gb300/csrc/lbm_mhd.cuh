@@ -33,7 +33,7 @@ __host__ __device__ constexpr int mopp(int m) { return m == 0 ? 0 : ((m & 1) ? m
 __host__ __device__ constexpr double mw(int m) { return m == 0 ? 0.25 : 0.125; }
 constexpr double CSM2 = 0.25;
 
-template <typename S, typename C, bool WALLS, int M, bool NC>
+template <typename S, typename C, bool WALLS, int M>
 __device__ __forceinline__ void gather_mag_dir(const S* __restrict__ gsrc, const Box& b, const Nbr& q, int x, int y,
                                                int z, uint32_t self, const C (&bw)[3], C (&g)[7][3]) {
     constexpr int cx = mcx(M), cy = mcy(M), cz = mcz(M);
@@ -47,21 +47,21 @@ __device__ __forceinline__ void gather_mag_dir(const S* __restrict__ gsrc, const
     for (int a = 0; a < 3; ++a) {
         const S* p = (!WALLS || !wall) ? gsrc + (size_t)(3 * M + a) * b.n + cell
                                        : gsrc + (size_t)(3 * mopp(M) + a) * b.n + self;
-        const C v = NC ? (C)Store<S>::load(p) : (C)Store<S>::load_coherent(p);
+        const C v = (C)Store<S>::load(p);
         g[M][a] = (!WALLS || !wall) ? v : -v + (C)(2.0 * mw(M)) * bw[a];
     }
 }
 
-template <typename S, typename C, bool WALLS, bool NC = true>
+template <typename S, typename C, bool WALLS>
 __device__ __forceinline__ void gather_mag(const S* __restrict__ gsrc, const Box& b, const Nbr& q, int x, int y,
                                            int z, uint32_t self, const C (&bw)[3], C (&g)[7][3]) {
-    gather_mag_dir<S, C, WALLS, 0, NC>(gsrc, b, q, x, y, z, self, bw, g);
-    gather_mag_dir<S, C, WALLS, 1, NC>(gsrc, b, q, x, y, z, self, bw, g);
-    gather_mag_dir<S, C, WALLS, 2, NC>(gsrc, b, q, x, y, z, self, bw, g);
-    gather_mag_dir<S, C, WALLS, 3, NC>(gsrc, b, q, x, y, z, self, bw, g);
-    gather_mag_dir<S, C, WALLS, 4, NC>(gsrc, b, q, x, y, z, self, bw, g);
-    gather_mag_dir<S, C, WALLS, 5, NC>(gsrc, b, q, x, y, z, self, bw, g);
-    gather_mag_dir<S, C, WALLS, 6, NC>(gsrc, b, q, x, y, z, self, bw, g);
+    gather_mag_dir<S, C, WALLS, 0>(gsrc, b, q, x, y, z, self, bw, g);
+    gather_mag_dir<S, C, WALLS, 1>(gsrc, b, q, x, y, z, self, bw, g);
+    gather_mag_dir<S, C, WALLS, 2>(gsrc, b, q, x, y, z, self, bw, g);
+    gather_mag_dir<S, C, WALLS, 3>(gsrc, b, q, x, y, z, self, bw, g);
+    gather_mag_dir<S, C, WALLS, 4>(gsrc, b, q, x, y, z, self, bw, g);
+    gather_mag_dir<S, C, WALLS, 5>(gsrc, b, q, x, y, z, self, bw, g);
+    gather_mag_dir<S, C, WALLS, 6>(gsrc, b, q, x, y, z, self, bw, g);
 }
 
 // b, the Lorentz force and the corrected velocity of one node.
@@ -123,17 +123,17 @@ __device__ __forceinline__ void store_geq(S* __restrict__ gdst, size_t n, uint32
 
 // One node: fluid and magnetic pulls, Lorentz force, CM collision, magnetic
 // BGK, stores.
-template <typename S, typename C, bool WALLS, bool NC>
+template <typename S, typename C, bool WALLS>
 __device__ __forceinline__ void mhd_node(const S* __restrict__ src, S* __restrict__ dst, const MhdArgs& p, int x,
                                          int y, int z) {
     const Box& b = p.box;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
     C f[Q];
-    gather19<S, C, WALLS, NC>(src, b, q, x, y, z, self, (C)0, (C)0, (C)0, f);
+    gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)0, (C)0, (C)0, f);
     const C bw[3] = {(C)p.bw[0], (C)p.bw[1], (C)p.bw[2]};
     C g[7][3];
-    gather_mag<S, C, WALLS, NC>(src + (size_t)Q * b.n, b, q, x, y, z, self, bw, g);
+    gather_mag<S, C, WALLS>(src + (size_t)Q * b.n, b, q, x, y, z, self, bw, g);
     const Moments<C> m = moments19(f);
     C bb[3];
     const Macro<C> a = mhd_macro<C>(m, g, p, bb);

@@ -218,8 +218,7 @@ extern "C" lbm_status lbm_autotune(lbm_ctx* c, const char* cache_path, int force
         Entry& h = hit->second;
         const int threads = (int)h["threads"];
         if (c->batch) {
-            const int cps = h.count("ctas_per_sm") ? (int)h["ctas_per_sm"] : 0;
-            if (lbm::batch_apply_config(c, threads, cps) != cudaSuccess) return LBM_ERR_CUDA;
+            if (lbm::batch_apply_config(c, threads) != cudaSuccess) return LBM_ERR_CUDA;
         } else {
             const int variant = h.count("variant") ? (int)h["variant"] : 0;
             const int stages = h.count("stages") ? (int)h["stages"] : 0;
@@ -249,24 +248,21 @@ extern "C" lbm_status lbm_autotune(lbm_ctx* c, const char* cache_path, int force
     if (c->batch) {
         const long steps = 6;
         const int threads_c[] = {128, 256};
-        const int cps_c[] = {1, 2, 3, 4, 0};
-        for (int th : threads_c)
-            for (int cps : cps_c) {
-                float ms = 0.f;
-                e = lbm::batch_time_config(c, th, cps, steps, &ms);
-                if (e != cudaSuccess) {
-                    cudaGetLastError();
-                    continue;
-                }
-                const double per = ms / steps;
-                if (per < best_ms) {
-                    best_ms = per;
-                    best = Entry{{"threads", (double)th}, {"ctas_per_sm", (double)cps}};
-                }
+        for (int th : threads_c) {
+            float ms = 0.f;
+            e = lbm::batch_time_config(c, th, steps, &ms);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                continue;
             }
+            const double per = ms / steps;
+            if (per < best_ms) {
+                best_ms = per;
+                best = Entry{{"threads", (double)th}};
+            }
+        }
         if (best.empty()) return LBM_ERR_CUDA;
-        if (lbm::batch_apply_config(c, (int)best["threads"], (int)best["ctas_per_sm"]) != cudaSuccess)
-            return LBM_ERR_CUDA;
+        if (lbm::batch_apply_config(c, (int)best["threads"]) != cudaSuccess) return LBM_ERR_CUDA;
     } else {
         struct Cand {
             int variant, threads, stages, ctas;
