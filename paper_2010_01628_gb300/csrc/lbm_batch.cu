@@ -36,22 +36,6 @@
 
 namespace lbm {
 
-// Quotient by a constant for dividends below 2^31: q = umulhi(n, mul) >> shift
-// (mul = ceil(2^p / d), p = 31 + ceil(log2 d)); mul = 0 stands for d = 1.
-struct FastDiv {
-    uint32_t mul, shift;
-};
-inline FastDiv make_fast_div(uint32_t d) {
-    if (d == 1) return {0u, 0u};
-    uint32_t l = 0;
-    while ((1ull << l) < d) ++l;
-    const uint32_t p = 31 + l;
-    return {(uint32_t)(((1ull << p) + d - 1) / d), p - 32};
-}
-__device__ __forceinline__ uint32_t fast_div(uint32_t n, FastDiv f) {
-    return f.mul ? __umulhi(n, f.mul) >> f.shift : n;
-}
-
 struct BatchDomain {
     FluidArgs fl;     // box, omega, g, lid
     MhdArgs mh;       // box, omega, tau_m, g, b_wall

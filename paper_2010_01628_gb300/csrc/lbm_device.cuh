@@ -41,12 +41,48 @@ __host__ __device__ constexpr double w_of(int i) {
 
 constexpr int Q = 19;
 
+// Quotient by a constant for dividends below 2^31: q = umulhi(n, mul) >> shift
+// (mul = ceil(2^p / d), p = 31 + ceil(log2 d)); mul = 0 stands for d = 1.
+struct FastDiv {
+    uint32_t mul, shift;
+};
+inline FastDiv make_fast_div(uint32_t d) {
+    if (d == 1) return {0u, 0u};
+    uint32_t l = 0;
+    while ((1ull << l) < d) ++l;
+    const uint32_t p = 31 + l;
+    return {(uint32_t)(((1ull << p) + d - 1) / d), p - 32};
+}
+__device__ __forceinline__ uint32_t fast_div(uint32_t n, FastDiv f) {
+    return f.mul ? __umulhi(n, f.mul) >> f.shift : n;
+}
+
 // Box boundary description used by every kernel.
 struct Box {
     int nx, ny, nz;
     unsigned periodic;  // bit 0 x, bit 1 y, bit 2 z
     size_t n;           // nx*ny*nz (plane stride)
 };
+
+// The node of this thread in z-plane blockIdx.z, rows y0 .. y0 + rows - 1.
+// FLAT: the plane's nodes are numbered through, so CTAs are full whatever nx is
+// and their accesses stay aligned (div_nx: node of the plane -> row); else a CTA
+// covers part of one x-row, y is uniform, and the index arithmetic of the pull
+// is too.
+template <bool FLAT>
+__device__ __forceinline__ bool plane_node(const Box& b, FastDiv div_nx, int y0, int rows, int& x, int& y) {
+    if (!FLAT) {
+        x = blockIdx.x * blockDim.x + threadIdx.x;
+        y = y0 + blockIdx.y;
+        return x < b.nx;
+    }
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= (uint32_t)rows * (uint32_t)b.nx) return false;
+    const uint32_t row = fast_div(k, div_nx);
+    x = (int)(k - row * (uint32_t)b.nx);
+    y = y0 + (int)row;
+    return true;
+}
 
 // ---------------------------------------------------------------------------
 // Storage formats.  FP64/FP32 hold f - w (shift by the rest state of rho0 = 1);

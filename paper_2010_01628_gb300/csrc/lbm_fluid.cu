@@ -14,24 +14,24 @@
 
 namespace lbm {
 
-template <typename S, typename C, bool WALLS, bool RM = false>
+template <typename S, typename C, bool WALLS, bool FLAT, bool RM = false>
 __global__ void __launch_bounds__(256) fluid_step_kernel(const S* __restrict__ src, S* __restrict__ dst,
-                                                         FluidArgs p) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= p.box.nx) return;
-    fluid_node<S, C, WALLS, RM>(src, dst, p, x, blockIdx.y, blockIdx.z);
+                                                         FluidArgs p, FastDiv div_nx) {
+    int x, y;
+    if (!plane_node<FLAT>(p.box, div_nx, 0, p.box.ny, x, y)) return;
+    fluid_node<S, C, WALLS, RM>(src, dst, p, x, y, blockIdx.z);
 }
 
 // Channels (x and z periodic, walls on y, ny >= 3) step in two launches: the
 // interior rows 1 .. ny-2 never pull through a wall and run the periodic node
 // code (40 registers instead of 48); a small launch then updates the two wall
 // rows with bounce-back or regularized walls.
-template <typename S, typename C>
+template <typename S, typename C, bool FLAT>
 __global__ void __launch_bounds__(256) fluid_step_interior_kernel(const S* __restrict__ src, S* __restrict__ dst,
-                                                                  FluidArgs p) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= p.box.nx) return;
-    fluid_node<S, C, false>(src, dst, p, x, blockIdx.y + 1, blockIdx.z);
+                                                                  FluidArgs p, FastDiv div_nx) {
+    int x, y;
+    if (!plane_node<FLAT>(p.box, div_nx, 1, p.box.ny - 2, x, y)) return;
+    fluid_node<S, C, false>(src, dst, p, x, y, blockIdx.z);
 }
 
 // The wall rows y = 0 (blockIdx.y = 0) and y = ny - 1 (blockIdx.y = 1) of a
@@ -255,13 +255,18 @@ __device__ __forceinline__ float pull_q(const S* __restrict__ src, const Box& b,
 // At most 128 threads and 72 registers (7 CTAs, 28 warps per SM; 78 registers
 // left 6): the kernel waits on its 38 pulls, and the extra warps hide more of
 // that latency.
-template <typename S, bool WALLS>
-__global__ void __launch_bounds__(ZPAIR_MAX_THREADS, 7) fluid_step_zpair_kernel(const S* __restrict__ src,
-                                                                              S* __restrict__ dst, FluidArgs p) {
+template <typename S, bool WALLS, bool FLAT>
+__global__ void __launch_bounds__(ZPAIR_MAX_THREADS, 7)
+    fluid_step_zpair_kernel(const S* __restrict__ src, S* __restrict__ dst, FluidArgs p, FastDiv div_nx) {
     const Box& b = p.box;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= b.nx) return;
-    const int y = blockIdx.y, za = 2 * (int)blockIdx.z;
+    int x = blockIdx.x * blockDim.x + threadIdx.x;
+    int y = blockIdx.y;
+    if constexpr (FLAT) {
+        if (!plane_node<true>(b, div_nx, 0, b.ny, x, y)) return;
+    } else {
+        if (x >= b.nx) return;
+    }
+    const int za = 2 * (int)blockIdx.z;
     const bool two = za + 1 < b.nz;
     const int zb = two ? za + 1 : za;
     const uint32_t sa = ((uint32_t)za * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
@@ -556,20 +561,31 @@ static cudaError_t launch_tma(lbm_ctx* c, const S* src, S* dst, const FluidArgs&
     return cudaSuccess;
 }
 
+template <typename S, typename C, bool RM>
+static void step_direct(lbm_ctx* c, dim3 grid, bool walls, bool flat, const S* src, S* dst, const FluidArgs& p) {
+    const int bx = c->block_x;
+    if (walls && flat)
+        fluid_step_kernel<S, C, true, true, RM><<<grid, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
+    else if (walls)
+        fluid_step_kernel<S, C, true, false, RM><<<grid, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
+    else if (flat)
+        fluid_step_kernel<S, C, false, true, RM><<<grid, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
+    else
+        fluid_step_kernel<S, C, false, false, RM><<<grid, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
+}
+
 template <typename S, typename C>
 static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
     const FluidArgs p = fluid_args(c);
     const bool walls = (c->box.periodic & 7u) != 7u;
     const int bx = c->block_x;
+    const bool flat = step_flat(c->box, bx);
+    const dim3 grid = step_grid(c->box, bx, c->box.ny, flat);
     if (c->relax.moment_space == LBM_MOMENTS_RAW) {
-        const dim3 grid = step_grid(c->box, bx);
         for (long s = 0; s < n; ++s) {
             const S* src = (const S*)c->buf[c->cur];
             S* dst = (S*)c->buf[c->cur ^ 1];
-            if (walls)
-                fluid_step_kernel<S, C, true, true><<<grid, bx, 0, c->stream>>>(src, dst, p);
-            else
-                fluid_step_kernel<S, C, false, true><<<grid, bx, 0, c->stream>>>(src, dst, p);
+            step_direct<S, C, true>(c, grid, walls, flat, src, dst, p);
             if (!dry) c->cur ^= 1;
         }
         return cudaGetLastError();
@@ -578,11 +594,14 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
     const bool channel = (c->box.periodic & 7u) == 5u && c->box.ny >= 3;
     if (channel && (reg || c->variant == 0)) {
         const unsigned gx = (unsigned)((c->box.nx + bx - 1) / bx);
-        const dim3 inner(gx, (unsigned)(c->box.ny - 2), (unsigned)c->box.nz), rows(gx, 2u, (unsigned)c->box.nz);
+        const dim3 inner = step_grid(c->box, bx, c->box.ny - 2, flat), rows(gx, 2u, (unsigned)c->box.nz);
         for (long s = 0; s < n; ++s) {
             const S* src = (const S*)c->buf[c->cur];
             S* dst = (S*)c->buf[c->cur ^ 1];
-            fluid_step_interior_kernel<S, C><<<inner, bx, 0, c->stream>>>(src, dst, p);
+            if (flat)
+                fluid_step_interior_kernel<S, C, true><<<inner, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
+            else
+                fluid_step_interior_kernel<S, C, false><<<inner, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
             if (reg)
                 fluid_step_wallrows_kernel<S, C, true><<<rows, bx, 0, c->stream>>>(src, dst, p);
             else
@@ -601,20 +620,24 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
         }
         return cudaGetLastError();
     }
-    const dim3 grid = step_grid(c->box, bx);
     const bool pair = is16<S>() && c->variant == 2 && (c->box.nx % 2 == 0);
     const bool zpair = is16<S>() && c->variant == 4;
     const dim3 grid2((unsigned)((c->box.nx / 2 + bx - 1) / bx), (unsigned)c->box.ny, (unsigned)c->box.nz);
     const dim3 gridz(grid.x, grid.y, (unsigned)((c->box.nz + 1) / 2));
+    const FastDiv div_nx = make_fast_div((uint32_t)c->box.nx);
     for (long s = 0; s < n; ++s) {
         const S* src = (const S*)c->buf[c->cur];
         S* dst = (S*)c->buf[c->cur ^ 1];
         if constexpr (is16<S>()) {
             if (zpair) {
-                if (walls)
-                    fluid_step_zpair_kernel<S, true><<<gridz, bx, 0, c->stream>>>(src, dst, p);
+                if (walls && flat)
+                    fluid_step_zpair_kernel<S, true, true><<<gridz, bx, 0, c->stream>>>(src, dst, p, div_nx);
+                else if (walls)
+                    fluid_step_zpair_kernel<S, true, false><<<gridz, bx, 0, c->stream>>>(src, dst, p, div_nx);
+                else if (flat)
+                    fluid_step_zpair_kernel<S, false, true><<<gridz, bx, 0, c->stream>>>(src, dst, p, div_nx);
                 else
-                    fluid_step_zpair_kernel<S, false><<<gridz, bx, 0, c->stream>>>(src, dst, p);
+                    fluid_step_zpair_kernel<S, false, false><<<gridz, bx, 0, c->stream>>>(src, dst, p, div_nx);
                 if (!dry) c->cur ^= 1;
                 continue;
             }
@@ -627,10 +650,7 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
                 continue;
             }
         }
-        if (walls)
-            fluid_step_kernel<S, C, true><<<grid, bx, 0, c->stream>>>(src, dst, p);
-        else
-            fluid_step_kernel<S, C, false><<<grid, bx, 0, c->stream>>>(src, dst, p);
+        step_direct<S, C, false>(c, grid, walls, flat, src, dst, p);
         if (!dry) c->cur ^= 1;
     }
     return cudaGetLastError();

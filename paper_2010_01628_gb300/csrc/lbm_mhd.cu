@@ -7,11 +7,11 @@
 
 namespace lbm {
 
-template <typename S, typename C, bool WALLS>
-__global__ void __launch_bounds__(256) mhd_step_kernel(const S* __restrict__ src, S* __restrict__ dst, MhdArgs p) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= p.box.nx) return;
-    mhd_node<S, C, WALLS>(src, dst, p, x, blockIdx.y, blockIdx.z);
+template <typename S, typename C, bool WALLS, bool FLAT>
+__global__ void __launch_bounds__(256) mhd_step_kernel(const S* __restrict__ src, S* __restrict__ dst, MhdArgs p, FastDiv div_nx) {
+    int x, y;
+    if (!plane_node<FLAT>(p.box, div_nx, 0, p.box.ny, x, y)) return;
+    mhd_node<S, C, WALLS>(src, dst, p, x, y, blockIdx.z);
 }
 
 template <typename S, typename C>
@@ -120,22 +120,24 @@ static MhdArgs mhd_args(const lbm_ctx* c) {
     return p;
 }
 
-template <typename S, typename C>
-static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
+template <typename S, typename C, bool WALLS, bool FLAT>
+static cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
     const MhdArgs p = mhd_args(c);
-    const bool walls = (c->box.periodic & 7u) != 7u;
     const int bx = c->block_x;
-    const dim3 grid = step_grid(c->box, bx);
+    const dim3 grid = step_grid(c->box, bx, c->box.ny, FLAT);
     for (long s = 0; s < n; ++s) {
-        const S* src = (const S*)c->buf[c->cur];
-        S* dst = (S*)c->buf[c->cur ^ 1];
-        if (walls)
-            mhd_step_kernel<S, C, true><<<grid, bx, 0, c->stream>>>(src, dst, p);
-        else
-            mhd_step_kernel<S, C, false><<<grid, bx, 0, c->stream>>>(src, dst, p);
+        mhd_step_kernel<S, C, WALLS, FLAT>
+            <<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], (S*)c->buf[c->cur ^ 1], p, make_fast_div((uint32_t)c->box.nx));
         if (!dry) c->cur ^= 1;
     }
     return cudaGetLastError();
+}
+template <typename S, typename C>
+static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
+    const bool flat = step_flat(c->box, c->block_x);
+    if ((c->box.periodic & 7u) != 7u)
+        return flat ? steps_t<S, C, true, true>(c, n, dry) : steps_t<S, C, true, false>(c, n, dry);
+    return flat ? steps_t<S, C, false, true>(c, n, dry) : steps_t<S, C, false, false>(c, n, dry);
 }
 
 template <typename S, typename C>

@@ -343,12 +343,12 @@ __device__ __forceinline__ Node<C> macro(const Mom<C>& m, const Args& p) {
     return s;
 }
 
-template <typename S, typename C, bool WALLS, bool RM>
-__global__ void __launch_bounds__(256) step_kernel(const S* __restrict__ src, S* __restrict__ dst, Args p) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
+template <typename S, typename C, bool WALLS, bool RM, bool FLAT>
+__global__ void __launch_bounds__(256) step_kernel(const S* __restrict__ src, S* __restrict__ dst, Args p, FastDiv div_nx) {
     const Box& b = p.box;
-    if (x >= b.nx) return;
+    const int z = blockIdx.z;
+    int x, y;
+    if (!plane_node<FLAT>(b, div_nx, 0, b.ny, x, y)) return;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
     C g[3][3][3];
@@ -457,24 +457,29 @@ static Args args_of(const lbm_ctx* c) {
     return p;
 }
 
-template <typename S, typename C>
-static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
+template <typename S, typename C, bool WALLS, bool RM, bool FLAT>
+static cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
     const Args p = args_of(c);
-    const bool walls = (c->box.periodic & 7u) != 7u, rm = c->relax.moment_space == LBM_MOMENTS_RAW;
     const int bx = c->block_x;
-    const dim3 grid = step_grid(c->box, bx);
+    const dim3 grid = step_grid(c->box, bx, c->box.ny, FLAT);
     for (long s = 0; s < n; ++s) {
-        const S* src = (const S*)c->buf[c->cur];
-        S* dst = (S*)c->buf[c->cur ^ 1];
-        if (walls)
-            rm ? step_kernel<S, C, true, true><<<grid, bx, 0, c->stream>>>(src, dst, p)
-               : step_kernel<S, C, true, false><<<grid, bx, 0, c->stream>>>(src, dst, p);
-        else
-            rm ? step_kernel<S, C, false, true><<<grid, bx, 0, c->stream>>>(src, dst, p)
-               : step_kernel<S, C, false, false><<<grid, bx, 0, c->stream>>>(src, dst, p);
+        step_kernel<S, C, WALLS, RM, FLAT>
+            <<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], (S*)c->buf[c->cur ^ 1], p, make_fast_div((uint32_t)c->box.nx));
         if (!dry) c->cur ^= 1;
     }
     return cudaGetLastError();
+}
+template <typename S, typename C, bool WALLS, bool RM>
+static cudaError_t steps_flat_t(lbm_ctx* c, long n, bool dry) {
+    return step_flat(c->box, c->block_x) ? steps_t<S, C, WALLS, RM, true>(c, n, dry)
+                                         : steps_t<S, C, WALLS, RM, false>(c, n, dry);
+}
+template <typename S, typename C>
+static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
+    const bool rm = c->relax.moment_space == LBM_MOMENTS_RAW;
+    if ((c->box.periodic & 7u) != 7u)
+        return rm ? steps_flat_t<S, C, true, true>(c, n, dry) : steps_flat_t<S, C, true, false>(c, n, dry);
+    return rm ? steps_flat_t<S, C, false, true>(c, n, dry) : steps_flat_t<S, C, false, false>(c, n, dry);
 }
 
 template <typename S, typename C>

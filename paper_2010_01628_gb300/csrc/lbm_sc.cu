@@ -23,12 +23,12 @@
 
 namespace lbm {
 
-template <typename S, typename C, bool WALLS>
-__global__ void __launch_bounds__(256) sc_psi_kernel(const S* __restrict__ src, C* __restrict__ psi, ScArgs p) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
+template <typename S, typename C, bool WALLS, bool FLAT>
+__global__ void __launch_bounds__(256) sc_psi_kernel(const S* __restrict__ src, C* __restrict__ psi, ScArgs p, FastDiv div_nx) {
     const Box& b = p.box;
-    if (x >= b.nx) return;
+    const int z = blockIdx.z;
+    int x, y;
+    if (!plane_node<FLAT>(b, div_nx, 0, b.ny, x, y)) return;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
     C f[Q];
@@ -36,13 +36,13 @@ __global__ void __launch_bounds__(256) sc_psi_kernel(const S* __restrict__ src, 
     psi[self] = pseudopotential<C>((C)1 + moments19(f).drho);
 }
 
-template <typename S, typename C, bool WALLS>
+template <typename S, typename C, bool WALLS, bool FLAT>
 __global__ void __launch_bounds__(256) sc_collide_kernel(const S* __restrict__ src, S* __restrict__ dst,
-                                                         const C* __restrict__ psi, ScArgs p) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
+                                                         const C* __restrict__ psi, ScArgs p, FastDiv div_nx) {
     const Box& b = p.box;
-    if (x >= b.nx) return;
+    const int z = blockIdx.z;
+    int x, y;
+    if (!plane_node<FLAT>(b, div_nx, 0, b.ny, x, y)) return;
     const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
     const Nbr q = make_nbr(b, x, y, z);
     C f[Q];
@@ -230,13 +230,23 @@ static ScArgs sc_args(const lbm_ctx* c) {
     return p;
 }
 
+template <typename S, typename C, bool WALLS, bool FLAT>
+static void launch_psi(lbm_ctx* c, const S* src, const ScArgs& p) {
+    sc_psi_kernel<S, C, WALLS, FLAT>
+        <<<step_grid(c->box, c->block_x, c->box.ny, FLAT), c->block_x, 0, c->stream>>>(src, (C*)c->phi, p, make_fast_div((uint32_t)c->box.nx));
+}
 template <typename S, typename C>
 static void launch_psi(lbm_ctx* c, const S* src, const ScArgs& p) {
-    const dim3 grid = step_grid(c->box, c->block_x);
-    if ((c->box.periodic & 7u) != 7u)
-        sc_psi_kernel<S, C, true><<<grid, c->block_x, 0, c->stream>>>(src, (C*)c->phi, p);
+    const bool walls = (c->box.periodic & 7u) != 7u, flat = step_flat(c->box, c->block_x);
+    if (walls)
+        flat ? launch_psi<S, C, true, true>(c, src, p) : launch_psi<S, C, true, false>(c, src, p);
     else
-        sc_psi_kernel<S, C, false><<<grid, c->block_x, 0, c->stream>>>(src, (C*)c->phi, p);
+        flat ? launch_psi<S, C, false, true>(c, src, p) : launch_psi<S, C, false, false>(c, src, p);
+}
+template <typename S, typename C, bool WALLS, bool FLAT>
+static void launch_collide(lbm_ctx* c, const S* src, S* dst, const ScArgs& p) {
+    sc_collide_kernel<S, C, WALLS, FLAT><<<step_grid(c->box, c->block_x, c->box.ny, FLAT), c->block_x, 0, c->stream>>>(
+        src, dst, (const C*)c->phi, p, make_fast_div((uint32_t)c->box.nx));
 }
 
 template <typename S, typename C, bool WALLS, int BY>
@@ -265,16 +275,15 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
         }
         return cudaGetLastError();
     }
-    const dim3 grid = step_grid(c->box, bx);
-    const C* psi = (const C*)c->phi;
+    const bool flat = step_flat(c->box, bx);
     for (long s = 0; s < n; ++s) {
         const S* src = (const S*)c->buf[c->cur];
         S* dst = (S*)c->buf[c->cur ^ 1];
         launch_psi<S, C>(c, src, p);
         if (walls)
-            sc_collide_kernel<S, C, true><<<grid, bx, 0, c->stream>>>(src, dst, psi, p);
+            flat ? launch_collide<S, C, true, true>(c, src, dst, p) : launch_collide<S, C, true, false>(c, src, dst, p);
         else
-            sc_collide_kernel<S, C, false><<<grid, bx, 0, c->stream>>>(src, dst, psi, p);
+            flat ? launch_collide<S, C, false, true>(c, src, dst, p) : launch_collide<S, C, false, false>(c, src, dst, p);
         if (!dry) c->cur ^= 1;
     }
     return cudaGetLastError();
