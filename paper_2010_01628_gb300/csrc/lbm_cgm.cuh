@@ -91,11 +91,11 @@ template <typename C>
 struct RedSrc {
     C a, vx, vy, vz;
 };
-template <typename S, typename C, bool WALLS, int I>
+template <typename S, typename C, int WALLS, int I>
 __device__ __forceinline__ void cgm_load(const S* __restrict__ src, const Box& b, const Nbr& q, int x, int y, int z,
                                          uint32_t self, C& f, RedSrc<C>& g) {
     uint32_t cell;
-    const bool wall = pull_source<I>(b, q, x, y, z, cell);
+    const bool wall = pull_source<I, WALLS>(b, q, x, y, z, cell);
     constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
     const bool bb = WALLS && wall;
     const uint32_t at = bb ? self : cell;
@@ -105,7 +105,7 @@ __device__ __forceinline__ void cgm_load(const S* __restrict__ src, const Box& b
     g.vy = cy ? cgm_ld<S, C>(src, b.n, CGM_VY, at) : (C)0;
     g.vz = cz ? cgm_ld<S, C>(src, b.n, CGM_VZ, at) : (C)0;
 }
-template <typename S, typename C, bool WALLS>
+template <typename S, typename C, int WALLS>
 __device__ __forceinline__ void cgm_pull_all(const S* __restrict__ src, const Box& b, const Nbr& q, int x, int y,
                                              int z, uint32_t self, C (&f)[Q], C (&r)[Q]) {
     RedSrc<C> g[Q];
@@ -120,7 +120,7 @@ __device__ __forceinline__ void cgm_pull_all(const S* __restrict__ src, const Bo
 #define LBM_CR(I)                                                                                     \
     {                                                                                                 \
         uint32_t cell;                                                                                \
-        const bool bb = WALLS && pull_source<I>(b, q, x, y, z, cell);                                 \
+        const bool bb = WALLS && pull_source<I, WALLS>(b, q, x, y, z, cell);                          \
         r[I] = bb ? red_pop<C, opp_of(I)>(g[I].a, g[I].vx, g[I].vy, g[I].vz, f[I])                   \
                   : red_pop<C, I>(g[I].a, g[I].vx, g[I].vy, g[I].vz, f[I]);                           \
     }
@@ -184,7 +184,7 @@ __device__ __forceinline__ void cgm_collide(C (&f)[Q], const Moments<C>& m, cons
 }
 
 // Pass 1 at one node: phi and rho_r from its pulled populations.
-template <typename S, typename C, bool WALLS>
+template <typename S, typename C, int WALLS>
 __device__ __forceinline__ void cgm_phi_node(const S* __restrict__ src, C* __restrict__ phi, C* __restrict__ rho_red,
                                              const CgmArgs& p, int x, int y, int z) {
     const Box& b = p.box;
@@ -199,7 +199,7 @@ __device__ __forceinline__ void cgm_phi_node(const S* __restrict__ src, C* __res
 
 // grad phi = (1/c_s^2) sum_i w_i c_i phi(x + c_i): the axis and the diagonal
 // neighbours are summed apart and scaled once (3/18 and 3/36).
-template <typename C, bool WALLS>
+template <typename C, int WALLS>
 __device__ __forceinline__ void grad_phi(const C* __restrict__ phi, const Box& b, const Nbr& q, int x, int y, int z,
                                          uint32_t self, C (&gr)[3]) {
     const C own = phi[self];
@@ -248,7 +248,7 @@ __device__ __forceinline__ void perturb_store(S* __restrict__ dst, size_t n, uin
 }
 
 // Pass 2 at one node: pull, collide the totals, perturb, recolour.
-template <typename S, typename C, bool WALLS>
+template <typename S, typename C, int WALLS>
 __device__ __forceinline__ void cgm_collide_node(const S* __restrict__ src, S* __restrict__ dst,
                                                  const C* __restrict__ phi, const C* __restrict__ rho_red,
                                                  const CgmArgs& p, int x, int y, int z) {

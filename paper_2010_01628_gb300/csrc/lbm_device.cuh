@@ -160,25 +160,33 @@ __device__ __forceinline__ Nbr make_nbr(const Box& b, int x, int y, int z) {
     return q;
 }
 
+// Axes that may have walls in code compiled for WALLS: 0 none (every axis
+// periodic), 1 any axis, 2 y only (channels).  The predicates and address
+// selects of the other axes are then not compiled: only 10 of the 18 pulls can
+// cross a y wall (colour-gradient collide pass at 128^3: 78.7 -> 71.8 us).
+__host__ __device__ constexpr int wall_axes(int walls) { return walls == 1 ? 7 : walls; }
+
 // Source node of the pull x - c_i and whether it lies behind a wall.
-template <int I>
+template <int I, int WALLS = 1>
 __device__ __forceinline__ bool pull_source(const Box& b, const Nbr& q, int x, int y, int z, uint32_t& cell) {
     constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
     const int sx = cx == 0 ? x : (cx > 0 ? q.xm : q.xp);
     const int sy = cy == 0 ? y : (cy > 0 ? q.ym : q.yp);
     const int sz = cz == 0 ? z : (cz > 0 ? q.zm : q.zp);
-    const bool wall = (cx > 0 && q.wxm) || (cx < 0 && q.wxp) || (cy > 0 && q.wym) || (cy < 0 && q.wyp) ||
-                      (cz > 0 && q.wzm) || (cz < 0 && q.wzp);
+    constexpr int ax = wall_axes(WALLS);
+    const bool wall = ((ax & 1) && ((cx > 0 && q.wxm) || (cx < 0 && q.wxp))) ||
+                      ((ax & 2) && ((cy > 0 && q.wym) || (cy < 0 && q.wyp))) ||
+                      ((ax & 4) && ((cz > 0 && q.wzm) || (cz < 0 && q.wzp)));
     cell = ((uint32_t)sz * (uint32_t)b.ny + (uint32_t)sy) * (uint32_t)b.nx + (uint32_t)sx;
     return wall;
 }
 
 // One pulled population f_I(x) = f*_I(x - c_I) (shifted).
-template <typename S, typename C, bool WALLS, int I>
+template <typename S, typename C, int WALLS, int I>
 __device__ __forceinline__ C gather_one(const S* __restrict__ src, const Box& b, const Nbr& q, int x, int y, int z,
                                         uint32_t self, C lx, C ly, C lz) {
     uint32_t cell;
-    const bool wall = pull_source<I>(b, q, x, y, z, cell);
+    const bool wall = pull_source<I, WALLS>(b, q, x, y, z, cell);
     if (!WALLS) return load_shifted<S, C, I>(src + (size_t)I * b.n + cell);
     // behind a wall: the node's own opposite population (same weight), chosen by
     // address rather than by a branch (+9% on the walled batch, +10% Rayleigh-Taylor)
@@ -192,7 +200,7 @@ __device__ __forceinline__ C gather_one(const S* __restrict__ src, const Box& b,
 // selects the variant with bounce-back; a pull from behind a wall reads the
 // node's own post-collision population of the opposite direction, plus
 // 6 w_i c_i . u_lid when the wall crossed is the moving +y lid.
-template <typename S, typename C, bool WALLS>
+template <typename S, typename C, int WALLS>
 __device__ __forceinline__ void gather19(const S* __restrict__ src, const Box& b, const Nbr& q, int x, int y, int z,
                                          uint32_t self, C lx, C ly, C lz, C (&f)[Q]) {
 #define LBM_G(I) f[I] = gather_one<S, C, WALLS, I>(src, b, q, x, y, z, self, lx, ly, lz);
@@ -205,15 +213,17 @@ __device__ __forceinline__ void gather19(const S* __restrict__ src, const Box& b
 // the node's own value `own`.  WALLS = false (every axis periodic) carries none
 // of the wall predicates, which cost the issue-bound collide passes about 90 of
 // their 760 (Shan-Chen) and 1004 (colour gradient) instructions.
-template <typename C, bool WALLS, int I>
+template <typename C, int WALLS, int I>
 __device__ __forceinline__ C field_nbr(const C* __restrict__ v, const Box& b, const Nbr& q, int x, int y, int z,
                                        C own) {
     constexpr int cx = cx_of(I), cy = cy_of(I), cz = cz_of(I);
     const int sx = cx == 0 ? x : (cx > 0 ? q.xp : q.xm);
     const int sy = cy == 0 ? y : (cy > 0 ? q.yp : q.ym);
     const int sz = cz == 0 ? z : (cz > 0 ? q.zp : q.zm);
-    const bool wall = WALLS && ((cx > 0 && q.wxp) || (cx < 0 && q.wxm) || (cy > 0 && q.wyp) || (cy < 0 && q.wym) ||
-                                (cz > 0 && q.wzp) || (cz < 0 && q.wzm));
+    constexpr int ax = wall_axes(WALLS);
+    const bool wall = ((ax & 1) && ((cx > 0 && q.wxp) || (cx < 0 && q.wxm))) ||
+                      ((ax & 2) && ((cy > 0 && q.wyp) || (cy < 0 && q.wym))) ||
+                      ((ax & 4) && ((cz > 0 && q.wzp) || (cz < 0 && q.wzm)));
     if (wall) return own;
     const C* a = v + ((uint32_t)sz * (uint32_t)b.ny + (uint32_t)sy) * (uint32_t)b.nx + (uint32_t)sx;
     return __ldg(a);
@@ -222,7 +232,7 @@ __device__ __forceinline__ C field_nbr(const C* __restrict__ v, const Box& b, co
 // s = sum_i w_i c_i v(x + c_i) over the 18 moving directions: the lattice
 // first moment of a node field (times 1/c_s^2 the isotropic gradient of the
 // colour-gradient model; times -G psi(x) the Shan-Chen force).
-template <typename C, bool WALLS>
+template <typename C, int WALLS>
 __device__ __forceinline__ void lattice_first_moment(const C* __restrict__ v, const Box& b, const Nbr& q, int x,
                                                      int y, int z, C own, C (&s)[3]) {
     C gx = (C)0, gy = (C)0, gz = (C)0;
