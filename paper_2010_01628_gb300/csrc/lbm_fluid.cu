@@ -12,14 +12,16 @@
 #include "lbm_internal.h"
 #include "lbm_reduce.cuh"
 
+#include <type_traits>
+
 namespace lbm {
 
-template <typename S, typename C, bool WALLS, bool FLAT, bool RM = false>
+template <typename S, typename C, bool WALLS, bool FLAT, bool RM = false, bool UNFORCED = false>
 __global__ void __launch_bounds__(256) fluid_step_kernel(const S* __restrict__ src, S* __restrict__ dst,
                                                          FluidArgs p, FastDiv div_nx) {
     int x, y;
     if (!plane_node<FLAT>(p.box, div_nx, 0, p.box.ny, x, y)) return;
-    fluid_node<S, C, WALLS, RM>(src, dst, p, x, y, blockIdx.z);
+    fluid_node<S, C, WALLS, RM, UNFORCED>(src, dst, p, x, y, blockIdx.z);
 }
 
 // Channels (x and z periodic, walls on y, ny >= 3) step in two launches: the
@@ -561,17 +563,18 @@ static cudaError_t launch_tma(lbm_ctx* c, const S* src, S* dst, const FluidArgs&
     return cudaSuccess;
 }
 
-template <typename S, typename C, bool RM>
+template <typename S, typename C, bool RM, bool UNFORCED>
 static void step_direct(lbm_ctx* c, dim3 grid, bool walls, bool flat, const S* src, S* dst, const FluidArgs& p) {
     const int bx = c->block_x;
+    const FastDiv div_nx = make_fast_div((uint32_t)c->box.nx);
     if (walls && flat)
-        fluid_step_kernel<S, C, true, true, RM><<<grid, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
+        fluid_step_kernel<S, C, true, true, RM, UNFORCED><<<grid, bx, 0, c->stream>>>(src, dst, p, div_nx);
     else if (walls)
-        fluid_step_kernel<S, C, true, false, RM><<<grid, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
+        fluid_step_kernel<S, C, true, false, RM, UNFORCED><<<grid, bx, 0, c->stream>>>(src, dst, p, div_nx);
     else if (flat)
-        fluid_step_kernel<S, C, false, true, RM><<<grid, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
+        fluid_step_kernel<S, C, false, true, RM, UNFORCED><<<grid, bx, 0, c->stream>>>(src, dst, p, div_nx);
     else
-        fluid_step_kernel<S, C, false, false, RM><<<grid, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
+        fluid_step_kernel<S, C, false, false, RM, UNFORCED><<<grid, bx, 0, c->stream>>>(src, dst, p, div_nx);
 }
 
 template <typename S, typename C>
@@ -585,7 +588,7 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
         for (long s = 0; s < n; ++s) {
             const S* src = (const S*)c->buf[c->cur];
             S* dst = (S*)c->buf[c->cur ^ 1];
-            step_direct<S, C, true>(c, grid, walls, flat, src, dst, p);
+            step_direct<S, C, true, false>(c, grid, walls, flat, src, dst, p);
             if (!dry) c->cur ^= 1;
         }
         return cudaGetLastError();
@@ -650,7 +653,14 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
                 continue;
             }
         }
-        step_direct<S, C, false>(c, grid, walls, flat, src, dst, p);
+        if constexpr (std::is_same<S, double>::value) {
+            if (p.g[0] == 0.0 && p.g[1] == 0.0 && p.g[2] == 0.0)
+                step_direct<S, C, false, true>(c, grid, walls, flat, src, dst, p);
+            else
+                step_direct<S, C, false, false>(c, grid, walls, flat, src, dst, p);
+        } else {
+            step_direct<S, C, false, false>(c, grid, walls, flat, src, dst, p);
+        }
         if (!dry) c->cur ^= 1;
     }
     return cudaGetLastError();
