@@ -17,12 +17,12 @@
 //    per (dy, dz) the 130-node row (with its x-halo) of every channel chunk
 //    is staged by 1D bulk copies of its contiguous runs, and the three
 //    x-shifted taps read it through descriptor start offsets of 16 bytes
-//    (unswizzled core matrices): 9 staged rows per tile instead of 27 boxes,
-//    three rows per ring stage.  The same kernel runs the backward data pass
+//    (unswizzled core matrices); tiles that follow one another in y share their
+//    staged rows.  The same kernel runs the backward data pass
 //    with the flipped, transposed weights.
-//  - wgrad_tc: weight gradients on the tensor cores (rows x input channels as
-//    M at one x-shift, output channels as N, voxels as K) from the same nine
-//    staged rows per tile, with the bias gradients summed from the staged dY
+//  - wgrad_slots_tc (one tile per row), wgrad_tc: weight gradients on the tensor
+//    cores (rows x input channels as M, output channels, of three x-shifts or
+//    one, as N, voxels as K) from the same staged rows, with the bias gradients summed from the staged dY
 //    tiles by the otherwise idle epilogue warps; one partial per CTA, summed
 //    in a fixed order.
 //  - adam: the optimiser step on the FP32 master weights.
@@ -88,12 +88,19 @@ __device__ __forceinline__ uint32_t bf_pack(float a, float b) {
 // TMA's 64-byte (CI = 32) or 32-byte (CI = 16) swizzle and stay in shared
 // memory for the CTA's life.
 //
-// Roles (192 threads): warp 0 stages rows into a ring of NSTAGE stages of
-// three rows each, one hand-off per stage (lane 0 waits and arms the stage,
-// lanes 0 .. 3 CI/8 - 1 issue one row chunk's copy each, the warp writes the
-// zero cells; when a row is one tile its halo cells never change, so the ring
-// is zeroed once and only rows outside the grid are written over); warp 1
-// allocates TMEM and its lane 0 issues the MMAs (M = 128, N = CO, K = 16) into
+// Roles (192 threads): warp 0 stages rows into a ring of slots, a slot holding
+// the rows (y, z - 1), (y, z), (y, z + 1) of one y (lane 0 waits and arms the
+// slot, lanes 0 .. 3 CI/8 - 1 issue one row chunk's copy each, the warp writes
+// the zero cells; when a row is one tile its halo cells never change, so the
+// ring is zeroed once and only rows outside the grid are written over).  A CTA
+// takes a contiguous range of tiles, and tile y reads the slots y - 1, y, y + 1:
+// each tile of a run stages one new slot, a third of its nine rows, with one
+// hand-off.  128^3, GB300, against restaging all nine (three hand-offs of three
+// rows a tile, MMAs issued by a single thread): 16 -> 32 122 -> 76 us, 32 -> 32
+// 173 -> 159 us (128 x 128 x 2 B of A per MMA at 128 B a cycle are 32 cycles, 50
+// measured: shared-memory reads bound it), forward pass 658 -> 565 us.  Warp 1
+// allocates TMEM and issues the MMAs (M = 128, N = CO, K = 16; the whole warp runs
+// the loop, an elected lane issues) into
 // one of two TMEM accumulators; warps 2-5 read the finished accumulator (each
 // warp its 32-lane quarter: one voxel per thread, CO columns), apply the
 // epilogue and store.  Every wait is bounded (TC_WAIT_NS); on expiry the
@@ -104,7 +111,9 @@ constexpr int ROW_NODES = TILE_M + 2;       // a staged row: the tile and its x-
 constexpr int ROW_CHUNK = ROW_NODES * 16;  // one channel chunk of a staged row (bytes)
 constexpr unsigned long long TC_WAIT_NS = 1000000000ull;
 
-// Tiles are 128-node segments of x-rows: ntx segments per row, ny * nz rows.
+// Tiles are 128-node segments of x-rows, ntx segments per row, numbered with y
+// fastest: a CTA's consecutive tiles are neighbours in y (a run) and share two
+// thirds of their staged rows.
 struct TileGeom {
     int nx, ny, nz;
     int ntx;
@@ -113,10 +122,12 @@ struct TileGeom {
 };
 
 __device__ __forceinline__ void tile_origin(const TileGeom& g, int t, int& x0, int& y0, int& z0) {
-    x0 = (t % g.ntx) * TILE_M;
-    y0 = (t / g.ntx) % g.ny;
+    y0 = t % g.ny;
+    x0 = ((t / g.ny) % g.ntx) * TILE_M;
     z0 = t / (g.ntx * g.ny);
 }
+
+__device__ __forceinline__ int tile_x0(const TileGeom& g, int t) { return ((t / g.ny) % g.ntx) * TILE_M; }
 
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
     const uint32_t a = lbm::smem_u32(p);
@@ -137,6 +148,10 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, volatile
         }
     }
     return true;
+}
+// Every lane of the warp waits; the outcome is warp-uniform.
+__device__ __forceinline__ bool tc_wait_all(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
+    return __all_sync(0xffffffffu, tc_wait(bar, parity, abort_flag, status));
 }
 // Bounded wait that ignores the abort flag (draining before exit).
 __device__ __forceinline__ void tc_drain(uint64_t* bar, uint32_t parity) {
@@ -194,64 +209,82 @@ __device__ __forceinline__ void copy_row_chunk(uint8_t* slot, const __nv_bfloat1
         lbm::bulk_g2s(slot + c * ROW_CHUNK + r.c0 * 16, X + ((size_t)c * P + r.src) * 8, (uint32_t)r.n * 16u, bar);
 }
 
-// A ring stage holds RPS staged rows (RPS = 3: the rows dy = -1, 0, 1 of one
-// dz), handed from the producer to the MMAs by one barrier.
-template <int CI, int CO, int NSTAGE, int RPS>
+// A ring slot holds the three staged rows dz = -1, 0, 1 of one y, handed from
+// the producer to the MMAs by one barrier.
+template <int CI, int CO>
 struct ConvLayout {
+    static constexpr int NSLOT = 6;  // three in use, three in flight
+    static constexpr int CTAS = CI == 32 ? 1 : 2;  // per SM: shared memory
     static constexpr int A_BYTES = (CI / 8) * ROW_CHUNK;          // a staged row, all chunks
     static constexpr int A_STRIDE = (A_BYTES + 127) / 128 * 128;  // row slots on 128-byte boundaries
-    static constexpr int STAGE_BYTES = RPS * A_STRIDE;
+    static constexpr int SLOT_BYTES = 3 * A_STRIDE;
     static constexpr int W_BYTES = 27 * CO * CI * 2;
     static constexpr int A_OFF = (W_BYTES + 1023) / 1024 * 1024;
-    static constexpr int BAR_OFF = (A_OFF + NSTAGE * STAGE_BYTES + 7) / 8 * 8;
-    static constexpr int NBAR = 2 * NSTAGE + 6;  // full, empty, tmem full x2, tmem empty x2, weights, drain
+    static constexpr int BAR_OFF = (A_OFF + NSLOT * SLOT_BYTES + 7) / 8 * 8;
+    static constexpr int NBAR = 2 * NSLOT + 6;  // full, empty, tmem full x2, tmem empty x2, weights, drain
     static constexpr int BYTES = BAR_OFF + NBAR * 8 + 16 + 1024;  // + TMEM slot, abort flag, alignment slack
     static constexpr uint32_t TCOLS = 2 * CO <= 32 ? 32 : 64;       // two accumulators of CO columns
     static constexpr uint32_t SWZ_W = CI == 32 ? tc::SW_64B : tc::SW_32B;
     static constexpr uint32_t IDESC = tc::idesc_bf16_f32(TILE_M, CO, false, false);
     static_assert(A_OFF % 1024 == 0 && A_STRIDE % 128 == 0, "weights on the swizzle period, slots 128-byte aligned");
-    static_assert(9 % RPS == 0, "a tile's nine rows fill whole stages");
-    static_assert(RPS * (CI / 8) <= 32, "one producer lane per row chunk of a stage");
+    static_assert(3 * (CI / 8) <= 32, "one producer lane per row chunk of a slot");
+    static_assert(CTAS * (BYTES + 1024) <= 228 * 1024 && BYTES <= 227 * 1024, "CTAS per SM must fit");
 };
 
-constexpr int CONV_STAGES = 2;
-constexpr int CONV_RPS = 3;
+// Position and phase of the next slot of a ring of N.
+template <int N>
+struct RingPos {
+    int pos = 0;
+    uint32_t phase = 0;
+    __device__ __forceinline__ void next() {
+        if (++pos == N) {
+            pos = 0;
+            phase ^= 1u;
+        }
+    }
+};
+// Tiles of the run that starts at tile t: y-neighbours of one x-segment and z,
+// within this CTA's range.
+__device__ __forceinline__ int run_length(const TileGeom& g, int t, int t_end, int y0) {
+    return min(t_end - t, g.ny - y0);
+}
 
 // EPI: 0 = +bias, ReLU, BF16 out (chunked); 1 = +bias, FP32 out [P][4] (the
 // output layer's real channels); 2 = zero where `gate` (this layer's forward
 // activation, chunked) is not positive, BF16 out (chunked), no bias.
 template <int CI, int CO, int EPI>
-__global__ void __launch_bounds__(192, 2) conv_tc(const __nv_bfloat16* __restrict__ X,
+__global__ void __launch_bounds__(192, ConvLayout<CI, CO>::CTAS) conv_tc(const __nv_bfloat16* __restrict__ X,
                                                const __grid_constant__ CUtensorMap mapW, const float* __restrict__ bias,
                                                void* __restrict__ Y, const __nv_bfloat16* __restrict__ gate,
                                                TileGeom g, int* status) {
-    using Lay = ConvLayout<CI, CO, CONV_STAGES, CONV_RPS>;
-    constexpr int RPS = CONV_RPS;
-    constexpr int NSTAGE = CONV_STAGES;
+    using Lay = ConvLayout<CI, CO>;
+    constexpr int NSLOT = Lay::NSLOT;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = align1024(smem_raw);
     uint8_t* sW = sm;
     uint8_t* sA = sm + Lay::A_OFF;
     uint64_t* full = reinterpret_cast<uint64_t*>(sm + Lay::BAR_OFF);
-    uint64_t* empty = full + NSTAGE;
-    uint64_t* tfull = empty + NSTAGE;
+    uint64_t* empty = full + NSLOT;
+    uint64_t* tfull = empty + NSLOT;
     uint64_t* tempty = tfull + 2;
     uint64_t* wfull = tempty + 2;
     uint64_t* drain = wfull + 1;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int per = (g.ntiles + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int t_begin = min(g.ntiles, (int)blockIdx.x * per), t_end = min(g.ntiles, t_begin + per);
     // Rows of one tile: the copies always fill cells 1 .. nx, so the halo
     // cells stay as zeroed here; only rows outside the grid are written over.
     const bool fixed_halo = g.ntx == 1;
     if (fixed_halo) {
-        for (int i = threadIdx.x; i < NSTAGE * Lay::STAGE_BYTES / 16; i += blockDim.x)
+        for (int i = threadIdx.x; i < NSLOT * Lay::SLOT_BYTES / 16; i += blockDim.x)
             reinterpret_cast<uint4*>(sA)[i] = make_uint4(0u, 0u, 0u, 0u);
         lbm::fence_proxy_async();
     }
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < NSTAGE; ++s) {
+        for (int s = 0; s < NSLOT; ++s) {
             lbm::mbar_init(&full[s], 1);
             lbm::mbar_init(&empty[s], 1);
         }
@@ -274,32 +307,32 @@ __global__ void __launch_bounds__(192, 2) conv_tc(const __nv_bfloat16* __restric
     const uint32_t tbase = *tslot;
 
     if (warp == 0) {
-        // ---- producer warp: 9 staged rows per tile, RPS per stage ----
+        // ---- producer warp: one slot per tile and two more per run ----
         if (lane == 0) {
             tc::prefetch_map(&mapW);
             lbm::mbar_arrive_expect_tx(wfull, Lay::W_BYTES);
             tc::tma_load_3d(sW, &mapW, 0, 0, 0, wfull);
         }
-        int armed[NSTAGE];
-        for (int s = 0; s < NSTAGE; ++s) armed[s] = -1;
-        int stage = 0;
-        uint32_t phase = 0;
+        int armed[NSLOT];
+#pragma unroll
+        for (int s = 0; s < NSLOT; ++s) armed[s] = -1;
+        RingPos<NSLOT> ring;
         bool ok = true;
-        for (int t = blockIdx.x; t < g.ntiles && ok; t += gridDim.x) {
+        for (int t = t_begin; t < t_end && ok;) {
             int x0, y0, z0;
             tile_origin(g, t, x0, y0, z0);
-            for (int r0 = 0; r0 < 9; r0 += RPS) {
-                if (!tc_wait_warp(&empty[stage], phase ^ 1u, abort_flag, status, lane)) {
+            const int len = run_length(g, t, t_end, y0);
+            for (int y = y0 - 1; y <= y0 + len; ++y) {
+                if (!tc_wait_warp(&empty[ring.pos], ring.phase ^ 1u, abort_flag, status, lane)) {
                     ok = false;
                     break;
                 }
-                uint8_t* st = sA + stage * Lay::STAGE_BYTES;
+                uint8_t* st = sA + ring.pos * Lay::SLOT_BYTES;
                 uint32_t bytes = 0;
                 bool zeroed = false;
 #pragma unroll
-                for (int j = 0; j < RPS; ++j) {
-                    const int r = r0 + j;
-                    const RowRun run = row_run(g, x0, y0 + r % 3 - 1, z0 + r / 3 - 1);
+                for (int j = 0; j < 3; ++j) {
+                    const RowRun run = row_run(g, x0, y, z0 + j - 1);
                     if (!fixed_halo || run.n == 0) {
                         zero_row_cells<CI / 8>(st + j * Lay::A_STRIDE, run, lane);
                         zeroed = true;
@@ -308,74 +341,88 @@ __global__ void __launch_bounds__(192, 2) conv_tc(const __nv_bfloat16* __restric
                 }
                 if (zeroed) lbm::fence_proxy_async();
                 __syncwarp();
-                // lane 0 arms the stage, the lanes issue one row chunk each
+                // lane 0 arms the slot, the lanes issue one row chunk each
                 if (lane == 0) {
-                    lbm::mbar_arrive_expect_tx(&full[stage], bytes);
-                    armed[stage] = (int)phase;
+                    lbm::mbar_arrive_expect_tx(&full[ring.pos], bytes);
+#pragma unroll
+                    for (int s = 0; s < NSLOT; ++s)
+                        if (s == ring.pos) armed[s] = (int)ring.phase;
                 }
                 __syncwarp();
-                if (lane < RPS * (CI / 8)) {
-                    const int j = lane / (CI / 8), r = r0 + j;
-                    copy_row_chunk(st + j * Lay::A_STRIDE, X, g.P, row_run(g, x0, y0 + r % 3 - 1, z0 + r / 3 - 1),
-                                   lane % (CI / 8), &full[stage]);
+                if (lane < 3 * (CI / 8)) {
+                    const int j = lane / (CI / 8);
+                    copy_row_chunk(st + j * Lay::A_STRIDE, X, g.P, row_run(g, x0, y, z0 + j - 1), lane % (CI / 8),
+                                   &full[ring.pos]);
                 }
-                if (++stage == NSTAGE) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
+                ring.next();
             }
+            t += len;
         }
         if (lane == 0) {
-            // the copies land by themselves: wait for the last one of every stage
-            for (int s = 0; s < NSTAGE; ++s)
+            // the copies land by themselves: wait for the last one of every slot
+#pragma unroll
+            for (int s = 0; s < NSLOT; ++s)
                 if (armed[s] >= 0) tc_drain(&full[s], (uint32_t)armed[s]);
             tc_drain(wfull, 0);
         }
-    } else if (threadIdx.x == 32) {
+    } else if (warp == 1) {
         // ---- MMA issuer: the three taps (dx = -1, 0, 1) of each staged row ----
-        if (tc_wait(wfull, 0, abort_flag, status)) {
+        if (tc_wait_all(wfull, 0, abort_flag, status)) {
             tc::fence_after_sync();
-            int stage = 0;
-            uint32_t phase = 0;
             int it = 0;
             bool ok = true;
+            RingPos<NSLOT> ring;  // the next slot to wait for
             // descriptors built once, advanced by byte offsets per operand
             const uint64_t adesc0 = tc::smem_desc(lbm::smem_u32(sA), ROW_CHUNK, 128, tc::SW_NONE);
             const uint64_t wdesc0 = tc::smem_desc(lbm::smem_u32(sW), 16, 8 * CI * 2, Lay::SWZ_W);
-            for (int t = blockIdx.x; t < g.ntiles && ok; t += gridDim.x, ++it) {
-                const int acc = it & 1;
-                if (!tc_wait(&tempty[acc], (((uint32_t)it >> 1) & 1u) ^ 1u, abort_flag, status)) break;
-                tc::fence_after_sync();
-                const uint32_t d = tbase + (uint32_t)(acc * CO);
-                for (int r0 = 0; r0 < 9; r0 += RPS) {
-                    if (!tc_wait(&full[stage], phase, abort_flag, status)) {
-                        ok = false;
-                        break;
+            for (int t = t_begin; t < t_end && ok;) {
+                int x0, y0, z0;
+                tile_origin(g, t, x0, y0, z0);
+                const int len = run_length(g, t, t_end, y0);
+                int pos[3] = {0, 0, 0};  // the slots y - 1, y, y + 1 of the current tile
+                for (int i = 0; i < len && ok; ++i, ++it) {
+                    const int acc = it & 1;
+                    ok = tc_wait_all(&tempty[acc], (((uint32_t)it >> 1) & 1u) ^ 1u, abort_flag, status);
+                    for (int w = i == 0 ? 0 : 2; w < 3 && ok; ++w) {
+                        ok = tc_wait_all(&full[ring.pos], ring.phase, abort_flag, status);
+                        if (i > 0) {
+                            pos[0] = pos[1];
+                            pos[1] = pos[2];
+                        }
+                        pos[w] = ring.pos;
+                        ring.next();
                     }
+                    if (!ok) break;
                     tc::fence_after_sync();
-                    const uint64_t astage = tc::desc_advance(adesc0, stage * Lay::STAGE_BYTES);
-                    const uint64_t wstage = tc::desc_advance(wdesc0, r0 * 3 * CO * CI * 2);  // tap 3 r0 onwards
+                    const uint32_t d = tbase + (uint32_t)(acc * CO);
+                    uint64_t aslot[3];
 #pragma unroll
-                    for (int j = 0; j < RPS; ++j) {
+                    for (int dy = 0; dy < 3; ++dy) aslot[dy] = tc::desc_advance(adesc0, pos[dy] * Lay::SLOT_BYTES);
 #pragma unroll
-                        for (int dxi = 0; dxi < 3; ++dxi) {
-                            // tap (r0 + j) * 3 + dxi = (dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)
+                    for (int dz = 0; dz < 3; ++dz) {
 #pragma unroll
-                            for (int k = 0; k < CI / 16; ++k) {
-                                const uint64_t ad =
-                                    tc::desc_advance(astage, j * Lay::A_STRIDE + dxi * 16 + k * 2 * ROW_CHUNK);
-                                const uint64_t bd = tc::desc_advance(wstage, (j * 3 + dxi) * CO * CI * 2 + k * 32);
-                                tc::mma_bf16(d, ad, bd, Lay::IDESC, r0 > 0 || j > 0 || dxi > 0 || k > 0);
+                        for (int dy = 0; dy < 3; ++dy) {
+#pragma unroll
+                            for (int dxi = 0; dxi < 3; ++dxi) {
+                                const int tap = dz * 9 + dy * 3 + dxi;
+#pragma unroll
+                                for (int k = 0; k < CI / 16; ++k)
+                                    tc::mma_bf16(d,
+                                                 tc::desc_advance(aslot[dy], dz * Lay::A_STRIDE + dxi * 16 +
+                                                                                 k * 2 * ROW_CHUNK),
+                                                 tc::desc_advance(wdesc0, tap * CO * CI * 2 + k * 32), Lay::IDESC,
+                                                 tap > 0 || k > 0);
                             }
                         }
                     }
-                    tc::mma_commit(&empty[stage]);
-                    if (++stage == NSTAGE) {
-                        stage = 0;
-                        phase ^= 1u;
+                    tc::mma_commit(&empty[pos[0]]);
+                    if (i == len - 1) {
+                        tc::mma_commit(&empty[pos[1]]);
+                        tc::mma_commit(&empty[pos[2]]);
                     }
+                    tc::mma_commit(&tfull[acc]);
                 }
-                if (ok) tc::mma_commit(&tfull[acc]);
+                t += len;
             }
         }
         tc::mma_commit(drain);
@@ -388,8 +435,19 @@ __global__ void __launch_bounds__(192, 2) conv_tc(const __nv_bfloat16* __restric
 #pragma unroll
         for (int co = 0; co < CO; ++co) bvals[co] = (EPI == 2) ? 0.f : __ldg(bias + co);
         int it = 0;
-        for (int t = blockIdx.x; t < g.ntiles; t += gridDim.x, ++it) {
+        for (int t = t_begin; t < t_end; ++t, ++it) {
             const int acc = it & 1;
+            int x0, y0, z0;
+            tile_origin(g, t, x0, y0, z0);
+            const int x = x0 + row;
+            const long p = ((long)z0 * g.ny + y0) * g.nx + x;
+            uint4 gw[EPI == 2 ? CO / 8 : 1];  // the gate values, loaded while the MMAs run
+            if (EPI == 2) {
+#pragma unroll
+                for (int j = 0; j < CO / 8; ++j)
+                    gw[j] = x < g.nx ? __ldg(reinterpret_cast<const uint4*>(gate) + (size_t)j * g.P + p)
+                                     : make_uint4(0u, 0u, 0u, 0u);
+            }
             const uint32_t tl = tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * CO);
             if (!tc_wait_warp(&tfull[acc], ((uint32_t)it >> 1) & 1u, abort_flag, status, lane)) break;
             tc::fence_after_sync();
@@ -402,11 +460,7 @@ __global__ void __launch_bounds__(192, 2) conv_tc(const __nv_bfloat16* __restric
             float v[CO];
 #pragma unroll
             for (int co = 0; co < CO; ++co) v[co] = __uint_as_float(r[co]);
-            int x0, y0, z0;
-            tile_origin(g, t, x0, y0, z0);
-            const int x = x0 + row;
             if (x >= g.nx) continue;
-            const long p = ((long)z0 * g.ny + y0) * g.nx + x;
 #pragma unroll
             for (int co = 0; co < CO; ++co) v[co] += bvals[co];
             if (EPI == 0) {
@@ -416,8 +470,7 @@ __global__ void __launch_bounds__(192, 2) conv_tc(const __nv_bfloat16* __restric
             if (EPI == 2) {
 #pragma unroll
                 for (int j = 0; j < CO / 8; ++j) {
-                    const uint4 gw = __ldg(reinterpret_cast<const uint4*>(gate) + (size_t)j * g.P + p);
-                    const uint32_t w4[4] = {gw.x, gw.y, gw.z, gw.w};
+                    const uint32_t w4[4] = {gw[j].x, gw[j].y, gw[j].z, gw[j].w};
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {
                         if (!(bf_lo(w4[h]) > 0.f)) v[8 * j + 2 * h] = 0.f;
@@ -581,7 +634,7 @@ __global__ void __launch_bounds__(192) wgrad_tc(const __nv_bfloat16* __restrict_
         if (lane == 0)
             for (int s = 0; s < NSTAGE; ++s)
                 if (armed[s] >= 0) tc_drain(&full[s], (uint32_t)armed[s]);
-    } else if (threadIdx.x == 32) {
+    } else if (warp == 1) {
         // ---- MMA issuer ----
         const uint64_t xdesc0 = tc::smem_desc(lbm::smem_u32(sm), 128, ROW_CHUNK, tc::SW_NONE);
         const uint64_t ydesc0 = tc::smem_desc(lbm::smem_u32(sm) + Lay::XB, 128, Lay::YCHUNK, tc::SW_NONE);
@@ -589,12 +642,12 @@ __global__ void __launch_bounds__(192) wgrad_tc(const __nv_bfloat16* __restrict_
         uint32_t phase = 0;
         bool ok = true;
         for (int t = t_begin, it = 0; t < t_end; ++t, ++it) {
-            if (!tc_wait(&full[stage], phase, abort_flag, status)) {
+            if (!tc_wait_all(&full[stage], phase, abort_flag, status)) {
                 ok = false;
                 break;
             }
             tc::fence_after_sync();
-            const int nk = (min(TILE_M, g.nx - (t % g.ntx) * TILE_M) + 15) / 16;
+            const int nk = (min(TILE_M, g.nx - tile_x0(g, t)) + 15) / 16;
             const uint64_t xst = tc::desc_advance(xdesc0, stage * Lay::STAGE);
             const uint64_t yst = tc::desc_advance(ydesc0, stage * Lay::STAGE);
             // 16 voxels per K-step: 16 x 16 bytes into every chunk
@@ -645,7 +698,7 @@ __global__ void __launch_bounds__(192) wgrad_tc(const __nv_bfloat16* __restrict_
                     ok = false;
                     break;
                 }
-                if (m < min(TILE_M, g.nx - (t % g.ntx) * TILE_M)) {
+                if (m < min(TILE_M, g.nx - tile_x0(g, t))) {
                     const uint4* yt = reinterpret_cast<const uint4*>(sm + stage * Lay::STAGE + Lay::XB);
 #pragma unroll
                     for (int c = 0; c < CO / 8; ++c) {
@@ -716,11 +769,322 @@ __global__ void __launch_bounds__(192) wgrad_tc(const __nv_bfloat16* __restrict_
     }
 }
 
+// Weight gradient for grids of one tile per row (nx <= 128), the
+// warm-start network's own.  dW[tap][co][ci] = sum_p' X[p' + (dy, dz)][ci]
+// dY[p' - dx][co]: the three dx share one X operand and ride on N = 3 CO against
+// dY staged three times, shifted by one voxel (the voxels this moves out of the
+// row meet X's zero halo).  An MMA's time is its operands' shared-memory reads
+// (MN-major: about 80 cycles for 128 x 16 by 16 x 32), so 24 MMAs of N = 96 a
+// tile replace 72 of N = 32.  X comes in the convolution's slots (three staged
+// rows dz = -1, 0, 1 of one y): tile y takes the slots y - 1, y, y + 1, so each
+// tile of a run stages one new slot instead of nine rows.  M = 128 is the slot's
+// three rows x CI channels and the rows that follow them in shared memory,
+// whose products are discarded.  128^3, GB300: 32 -> 32 313 -> 162 us, 32 -> 16
+// 300 -> 140, 16 -> 32 201 -> 141, the gradient 2.40 -> 1.71 ms.  Grids of several
+// tiles per row keep wgrad_tc.
+template <int CI, int CO>
+struct WgSlotLayout {
+    static constexpr int TG = TILE_M / CI;  // rows that M = 128 spans
+    static constexpr int ROW = (CI / 8) * ROW_CHUNK;
+    static constexpr int SLOT = 3 * ROW;
+    static constexpr int NSLOT = 5;  // three in use, two in flight
+    static constexpr int YCHUNK = TILE_M * 16;
+    static constexpr int YB = 3 * (CO / 8) * YCHUNK;  // [dx][chunk][128][8]
+    static constexpr int NY = 3;
+    static constexpr int Y_OFF = (NSLOT * SLOT + (TG - 3) * ROW + 127) / 128 * 128;  // rows read past the last slot
+    static constexpr int BAR_OFF = Y_OFF + NY * YB;
+    static constexpr int NBAR = 2 * NSLOT + 2 * NY + 2;  // X full, empty; dY full, empty; accumulators full, drain
+    static constexpr int BYTES = BAR_OFF + NBAR * 8 + 16 + 4 * CO * 4 + 1024;
+    static constexpr int NGRP = 9;  // (dy, dx) accumulators of CO columns
+    static constexpr uint32_t TCOLS = NGRP * CO <= 256 ? 256 : 512;
+    static constexpr uint32_t IDESC = tc::idesc_bf16_f32(TILE_M, 3 * CO, true, true);
+    static_assert((3 * CO) % 16 == 0, "N of an M = 128 MMA");
+    static_assert(ROW % 16 == 0 && BYTES <= 227 * 1024 && NGRP * CO <= 512, "staging and accumulators must fit");
+};
+
+template <int CI, int CO>
+__global__ void __launch_bounds__(192) wgrad_slots_tc(const __nv_bfloat16* __restrict__ X,
+                                                      const __nv_bfloat16* __restrict__ dY,
+                                                      float* __restrict__ partial, TileGeom g, int* status) {
+    using Lay = WgSlotLayout<CI, CO>;
+    constexpr int NSLOT = Lay::NSLOT, NY = Lay::NY;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* sm = align1024(smem_raw);
+    uint64_t* xfull = reinterpret_cast<uint64_t*>(sm + Lay::BAR_OFF);
+    uint64_t* xempty = xfull + NSLOT;
+    uint64_t* yfull = xempty + NSLOT;
+    uint64_t* yempty = yfull + NY;
+    uint64_t* accfull = yempty + NY;
+    uint64_t* drain = accfull + 1;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
+    float* sbias = reinterpret_cast<float*>(tslot + 4);  // [4 warps][CO]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int per = (g.ntiles + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int t_begin = min(g.ntiles, (int)blockIdx.x * per), t_end = min(g.ntiles, t_begin + per);
+
+    // every staged value the MMAs read is finite; X's halo cells and the dY cells
+    // that no copy reaches (the shifted copies' first or last, those past the
+    // row) stay zero
+    for (int i = threadIdx.x; i < Lay::BAR_OFF / 16; i += blockDim.x)
+        reinterpret_cast<uint4*>(sm)[i] = make_uint4(0u, 0u, 0u, 0u);
+    lbm::fence_proxy_async();
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < NSLOT; ++s) {
+            lbm::mbar_init(&xfull[s], 1);
+            lbm::mbar_init(&xempty[s], 1);
+        }
+        for (int s = 0; s < NY; ++s) {
+            lbm::mbar_init(&yfull[s], 1);
+            lbm::mbar_init(&yempty[s], 5);  // the MMAs' commit and the four epilogue warps
+        }
+        lbm::mbar_init(accfull, 1);
+        lbm::mbar_init(drain, 1);
+        *abort_flag = 0;
+        lbm::fence_barrier_init();
+    }
+    if (warp == 1) {
+        tc::tmem_alloc(tslot, Lay::TCOLS);
+        tc::tmem_relinquish();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tbase = *tslot;
+
+    if (warp == 0) {
+        // ---- producer warp: a run's slots, and each tile's dY behind its last slot ----
+        int xarmed[NSLOT], yarmed[NY];
+#pragma unroll
+        for (int s = 0; s < NSLOT; ++s) xarmed[s] = -1;
+#pragma unroll
+        for (int s = 0; s < NY; ++s) yarmed[s] = -1;
+        RingPos<NSLOT> xr;
+        RingPos<NY> yr;
+        bool ok = true;
+        const uint32_t ybytes = (uint32_t)((CO / 8) * 16 * (g.nx + 2 * (g.nx - 1)));
+        for (int t = t_begin; t < t_end && ok;) {
+            int x0, y0, z0;
+            tile_origin(g, t, x0, y0, z0);
+            const int len = run_length(g, t, t_end, y0);
+            for (int y = y0 - 1; y <= y0 + len; ++y) {
+                if (!tc_wait_warp(&xempty[xr.pos], xr.phase ^ 1u, abort_flag, status, lane)) {
+                    ok = false;
+                    break;
+                }
+                uint8_t* st = sm + xr.pos * Lay::SLOT;
+                uint32_t bytes = 0;
+                bool zeroed = false;
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    const RowRun run = row_run(g, 0, y, z0 + j - 1);
+                    if (run.n == 0) {
+                        zero_row_cells<CI / 8>(st + j * Lay::ROW, run, lane);
+                        zeroed = true;
+                    }
+                    bytes += (uint32_t)((CI / 8) * run.n * 16);
+                }
+                if (zeroed) lbm::fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) {
+                    lbm::mbar_arrive_expect_tx(&xfull[xr.pos], bytes);
+#pragma unroll
+                    for (int s = 0; s < NSLOT; ++s)
+                        if (s == xr.pos) xarmed[s] = (int)xr.phase;
+                }
+                __syncwarp();
+                if (lane < 3 * (CI / 8)) {
+                    const int j = lane / (CI / 8);
+                    copy_row_chunk(st + j * Lay::ROW, X, g.P, row_run(g, 0, y, z0 + j - 1), lane % (CI / 8),
+                                   &xfull[xr.pos]);
+                }
+                xr.next();
+                const int yt = y - 1;  // the tile that this slot completes
+                if (yt < y0) continue;
+                if (!tc_wait_warp(&yempty[yr.pos], yr.phase ^ 1u, abort_flag, status, lane)) {
+                    ok = false;
+                    break;
+                }
+                if (lane == 0) {
+                    lbm::mbar_arrive_expect_tx(&yfull[yr.pos], ybytes);
+#pragma unroll
+                    for (int s = 0; s < NY; ++s)
+                        if (s == yr.pos) yarmed[s] = (int)yr.phase;
+                }
+                __syncwarp();
+                if (lane < 3 * (CO / 8)) {
+                    // shift dx: voxel p goes to cell p + dx, where that is a voxel of the row
+                    const int dx = lane / (CO / 8) - 1, c = lane % (CO / 8);
+                    const int p = dx < 0 ? 1 : 0, n = g.nx - (dx != 0 ? 1 : 0);
+                    const long p0 = ((long)z0 * g.ny + yt) * g.nx + p;
+                    if (n > 0)
+                        lbm::bulk_g2s(sm + Lay::Y_OFF + yr.pos * Lay::YB + lane * Lay::YCHUNK + (p + dx) * 16,
+                                      dY + ((size_t)c * g.P + p0) * 8, (uint32_t)n * 16u, &yfull[yr.pos]);
+                }
+                yr.next();
+            }
+            t += len;
+        }
+        if (lane == 0) {
+#pragma unroll
+            for (int s = 0; s < NSLOT; ++s)
+                if (xarmed[s] >= 0) tc_drain(&xfull[s], (uint32_t)xarmed[s]);
+#pragma unroll
+            for (int s = 0; s < NY; ++s)
+                if (yarmed[s] >= 0) tc_drain(&yfull[s], (uint32_t)yarmed[s]);
+        }
+    } else if (warp == 1) {
+        // ---- MMA issuer ----
+        const uint64_t xdesc0 = tc::smem_desc(lbm::smem_u32(sm), 128, ROW_CHUNK, tc::SW_NONE);
+        const uint64_t ydesc0 = tc::smem_desc(lbm::smem_u32(sm) + Lay::Y_OFF, 128, Lay::YCHUNK, tc::SW_NONE);
+        RingPos<NSLOT> xr;
+        RingPos<NY> yr;
+        bool ok = true;
+        int it = 0;
+        for (int t = t_begin; t < t_end && ok;) {
+            int x0, y0, z0;
+            tile_origin(g, t, x0, y0, z0);
+            const int len = run_length(g, t, t_end, y0);
+            const int nk = (g.nx + 15) / 16;
+            int pos[3] = {0, 0, 0};  // the slots y - 1, y, y + 1 of the current tile
+            for (int i = 0; i < len; ++i, ++it) {
+                for (int w = i == 0 ? 0 : 2; w < 3 && ok; ++w) {
+                    ok = tc_wait_all(&xfull[xr.pos], xr.phase, abort_flag, status);
+                    if (i > 0) {
+                        pos[0] = pos[1];
+                        pos[1] = pos[2];
+                    }
+                    pos[w] = xr.pos;
+                    xr.next();
+                }
+                ok = ok && tc_wait_all(&yfull[yr.pos], yr.phase, abort_flag, status);
+                if (!ok) break;
+                tc::fence_after_sync();
+                const uint64_t yst = tc::desc_advance(ydesc0, yr.pos * Lay::YB);
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy) {
+                    const uint64_t xst = tc::desc_advance(xdesc0, pos[dy] * Lay::SLOT + 16);  // cell 1: node 0
+                    const uint32_t d = tbase + (uint32_t)(dy * 3 * CO);
+                    if (nk == TILE_M / 16) {
+#pragma unroll
+                        for (int k = 0; k < TILE_M / 16; ++k)
+                            tc::mma_bf16(d, tc::desc_advance(xst, k * 256), tc::desc_advance(yst, k * 256), Lay::IDESC,
+                                         it > 0 || k > 0);
+                    } else {
+                        for (int k = 0; k < nk; ++k)
+                            tc::mma_bf16(d, tc::desc_advance(xst, k * 256), tc::desc_advance(yst, k * 256), Lay::IDESC,
+                                         it > 0 || k > 0);
+                    }
+                }
+                tc::mma_commit(&xempty[pos[0]]);
+                if (i == len - 1) {
+                    tc::mma_commit(&xempty[pos[1]]);
+                    tc::mma_commit(&xempty[pos[2]]);
+                }
+                tc::mma_commit(&yempty[yr.pos]);
+                yr.next();
+            }
+            t += len;
+        }
+        if (ok) tc::mma_commit(accfull);
+        tc::mma_commit(drain);
+        tc_drain(drain, 0);
+    } else {
+        // ---- epilogue: bias sums over the staged dY tiles, then the
+        // accumulated groups -> this CTA's partial ----
+        const int q = warp & 3;
+        const int m = q * 32 + lane;
+        const int dz = m / CI, ci = m % CI;  // the slot's row, and past it the discarded ones
+        float* out = partial + (size_t)blockIdx.x * (27 * CO * CI + CO);
+        const bool have = t_end > t_begin;
+        bool ok = true;
+        float db[CO];
+#pragma unroll
+        for (int co = 0; co < CO; ++co) db[co] = 0.f;
+        RingPos<NY> yr;
+        for (int t = t_begin; t < t_end; ++t) {
+            if (!tc_wait_warp(&yfull[yr.pos], yr.phase, abort_flag, status, lane)) {
+                ok = false;
+                break;
+            }
+            if (m < g.nx) {  // the unshifted copy, dx = 0
+                const uint4* yt = reinterpret_cast<const uint4*>(sm + Lay::Y_OFF + yr.pos * Lay::YB +
+                                                                 (CO / 8) * Lay::YCHUNK);
+#pragma unroll
+                for (int c = 0; c < CO / 8; ++c) {
+                    const uint4 w = yt[c * (Lay::YCHUNK / 16) + m];
+                    const uint32_t w4[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        db[8 * c + 2 * h] += bf_lo(w4[h]);
+                        db[8 * c + 2 * h + 1] += bf_hi(w4[h]);
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&yempty[yr.pos]);
+            yr.next();
+        }
+#pragma unroll
+        for (int co = 0; co < CO; ++co) {
+            float v = db[co];
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            db[co] = v;
+        }
+        if (lane == 0)
+#pragma unroll
+            for (int co = 0; co < CO; ++co) sbias[q * CO + co] = db[co];
+        asm volatile("bar.sync 1, 128;" ::: "memory");  // the four epilogue warps
+        if (q == 0 && lane < CO)
+            out[27 * CO * CI + lane] =
+                ok ? ((sbias[lane] + sbias[CO + lane]) + sbias[2 * CO + lane]) + sbias[3 * CO + lane] : 0.f;
+        if (have && ok) {
+            ok = tc_wait_warp(accfull, 0, abort_flag, status, lane);
+            if (ok) tc::fence_after_sync();
+        }
+        if (ok) {
+            for (int gi = 0; gi < Lay::NGRP; ++gi) {
+                uint32_t r[CO];
+                if (have) {
+                    if constexpr (CO == 32)
+                        tc::tmem_ld32(tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(gi * CO), r);
+                    else
+                        tc::tmem_ld16(tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(gi * CO), r);
+                    tc::tmem_ld_wait();
+                } else {
+#pragma unroll
+                    for (int co = 0; co < CO; ++co) r[co] = 0u;
+                }
+                if (dz < 3) {
+                    const int tap = dz * 9 + gi;  // gi = dy * 3 + dx
+#pragma unroll
+                    for (int co = 0; co < CO; ++co) out[((size_t)tap * CO + co) * CI + ci] = __uint_as_float(r[co]);
+                }
+            }
+        }
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 1) {
+        tc::fence_after_sync();
+        tc::tmem_dealloc(tbase, Lay::TCOLS);
+    }
+}
+
 __global__ void sum_partials(const float* __restrict__ partial, int nblocks, int width, float* __restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= width) return;
     float s = 0.f;
-    for (int b = 0; b < nblocks; ++b) s += partial[(size_t)b * width + i];
+    int b = 0;
+    for (; b + 8 <= nblocks; b += 8) {  // eight loads in flight, added in order
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = partial[(size_t)(b + k) * width + i];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += v[k];
+    }
+    for (; b < nblocks; ++b) s += partial[(size_t)b * width + i];
     out[i] = s;
 }
 
@@ -978,20 +1342,29 @@ bool make_maps(lbm_cnn* c) {
 template <int CI, int CO, int EPI>
 cudaError_t conv(lbm_cnn* c, const __nv_bfloat16* X, const CUtensorMap& mapW, const float* bias, void* Y,
                  const __nv_bfloat16* gate) {
-    const int smem = cnn::ConvLayout<CI, CO, cnn::CONV_STAGES, cnn::CONV_RPS>::BYTES;
+    using Lay = cnn::ConvLayout<CI, CO>;
+    const int smem = Lay::BYTES;
     cudaError_t e = cudaFuncSetAttribute(cnn::conv_tc<CI, CO, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    const int blocks = std::min(c->geom.ntiles, 2 * c->nsm);
+    const int blocks = std::min(c->geom.ntiles, Lay::CTAS * c->nsm);
     cnn::conv_tc<CI, CO, EPI><<<blocks, 192, smem, c->stream>>>(X, mapW, bias, Y, gate, c->geom, c->status);
     return cudaGetLastError();
 }
 
 template <int CI, int CO>
 cudaError_t wgrad(lbm_cnn* c, const __nv_bfloat16* X, const __nv_bfloat16* dY, float* gpad) {
-    const int smem = cnn::WgLayout<CI, CO>::BYTES;
-    cudaError_t e = cudaFuncSetAttribute(cnn::wgrad_tc<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    cnn::wgrad_tc<CI, CO><<<c->wg_blocks, 192, smem, c->stream>>>(X, dY, c->partial, c->geom, c->status);
+    if (c->geom.ntx == 1) {
+        const int smem = cnn::WgSlotLayout<CI, CO>::BYTES;
+        cudaError_t e =
+            cudaFuncSetAttribute(cnn::wgrad_slots_tc<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        cnn::wgrad_slots_tc<CI, CO><<<c->wg_blocks, 192, smem, c->stream>>>(X, dY, c->partial, c->geom, c->status);
+    } else {
+        const int smem = cnn::WgLayout<CI, CO>::BYTES;
+        cudaError_t e = cudaFuncSetAttribute(cnn::wgrad_tc<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        cnn::wgrad_tc<CI, CO><<<c->wg_blocks, 192, smem, c->stream>>>(X, dY, c->partial, c->geom, c->status);
+    }
     const int width = 27 * CO * CI + CO;
     cnn::sum_partials<<<(width + 255) / 256, 256, 0, c->stream>>>(c->partial, c->wg_blocks, width, gpad);
     return cudaGetLastError();
