@@ -470,29 +470,26 @@ __global__ void fluid_fields_kernel(const S* __restrict__ src, FieldsOut out, Fl
 template <typename S, typename C, bool WALLS, bool REG = false>
 __global__ void __launch_bounds__(RED_THREADS) fluid_reduce_kernel(const S* __restrict__ src, FluidArgs p,
                                                                    C* __restrict__ uprev, bool have_prev,
-                                                                   bool record, double* __restrict__ partials) {
+                                                                   bool record, double* __restrict__ partials,
+                                                                 NodeDiv div) {
     const Box& b = p.box;
-    const int chunks_x = (b.nx + RED_THREADS - 1) / RED_THREADS;
-    const long total = (long)chunks_x * b.ny * b.nz;
     RedAcc acc;
     acc.zero();
-    for (long ch = blockIdx.x; ch < total; ch += gridDim.x) {
-        const int cxk = (int)(ch % chunks_x);
-        const long row = ch / chunks_x;
-        const int y = (int)(row % b.ny), z = (int)(row / b.ny);
-        const int x = cxk * RED_THREADS + threadIdx.x;
-        if (x < b.nx) {
-            const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
-            const Nbr q = make_nbr(b, x, y, z);
-            C f[Q];
-            if (REG)
-                gather_regularized<S, C>(src, p, q, x, y, z, self, f);
-            else
-                gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
-            const Moments<C> mo = moments19(f);
-            const Macro<C> a = fluid_macro(mo, (C)p.g[0], (C)p.g[1], (C)p.g[2]);
-            reduce_node<C>(acc, a.rho, a.ux, a.uy, a.uz, uprev, b.n, self, have_prev, record);
-        }
+    for (uint32_t self = blockIdx.x * RED_THREADS + threadIdx.x; self < (uint32_t)b.n;
+         self += gridDim.x * RED_THREADS) {
+        int x, y, z;
+        node_of(self, b, div, x, y, z);
+        C up[3];
+        load_prev(uprev, b.n, self, have_prev, up);
+        const Nbr q = make_nbr(b, x, y, z);
+        C f[Q];
+        if (REG)
+            gather_regularized<S, C>(src, p, q, x, y, z, self, f);
+        else
+            gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
+        const Moments<C> mo = moments19(f);
+        const Macro<C> a = fluid_macro(mo, (C)p.g[0], (C)p.g[1], (C)p.g[2]);
+        reduce_node<C>(acc, a.rho, a.ux, a.uy, a.uz, up, uprev, b.n, self, have_prev, record);
     }
     block_reduce_store(acc, partials);
 }
@@ -693,13 +690,13 @@ static cudaError_t reduce_t(lbm_ctx* c, bool record) {
     const FluidArgs p = fluid_args(c);
     if (c->grid.wall_model == LBM_WALL_REGULARIZED)
         fluid_reduce_kernel<S, C, true, true><<<RED_BLOCKS, RED_THREADS, 0, c->stream>>>(
-            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials);
+            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials, node_div(c->box));
     else if ((c->box.periodic & 7u) != 7u)
         fluid_reduce_kernel<S, C, true><<<RED_BLOCKS, RED_THREADS, 0, c->stream>>>(
-            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials);
+            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials, node_div(c->box));
     else
         fluid_reduce_kernel<S, C, false><<<RED_BLOCKS, RED_THREADS, 0, c->stream>>>(
-            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials);
+            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials, node_div(c->box));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return reduce_finalize(c);
@@ -742,25 +739,26 @@ cudaError_t fluid_reduce(lbm_ctx* c, bool record) {
     return cudaErrorInvalidValue;
 }
 
-// Deterministic final sum of the per-block partials (one block).
+// Deterministic final sum of the per-block partials (one block): thread t sums
+// value t % 8 of every 32nd block, eight loads in flight, then the 32 sums of each
+// value are added within the warps and across them.
 __global__ void reduce_finalize_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
-    __shared__ double sh[RED_THREADS][RED_WIDTH];
-    double acc[RED_WIDTH];
-#pragma unroll
-    for (int k = 0; k < RED_WIDTH; ++k) acc[k] = 0.0;
-    for (int i = threadIdx.x; i < nblocks; i += blockDim.x)
-#pragma unroll
-        for (int k = 0; k < RED_WIDTH; ++k) acc[k] += partials[(size_t)i * RED_WIDTH + k];
-#pragma unroll
-    for (int k = 0; k < RED_WIDTH; ++k) sh[threadIdx.x][k] = acc[k];
+    static_assert(RED_WIDTH == 8 && RED_THREADS == 256, "one thread per value and block residue");
+    __shared__ double sh[RED_THREADS / 32][RED_WIDTH];
+    const int k = threadIdx.x & 7, first = threadIdx.x >> 3;
+    double x = 0.0;
+#pragma unroll 8
+    for (int i = first; i < nblocks; i += RED_THREADS / RED_WIDTH) x += partials[(size_t)i * RED_WIDTH + k];
+    x += __shfl_xor_sync(0xffffffffu, x, 8);
+    x += __shfl_xor_sync(0xffffffffu, x, 16);
+    if ((threadIdx.x & 31) < RED_WIDTH) sh[threadIdx.x >> 5][k] = x;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
+    if (threadIdx.x < RED_WIDTH) {
+        double s = 0.0;
 #pragma unroll
-            for (int k = 0; k < RED_WIDTH; ++k) sh[threadIdx.x][k] += sh[threadIdx.x + s][k];
-        __syncthreads();
+        for (int w = 0; w < RED_THREADS / 32; ++w) s += sh[w][threadIdx.x];
+        out[threadIdx.x] = s;
     }
-    if (threadIdx.x < RED_WIDTH) out[threadIdx.x] = sh[0][threadIdx.x];
 }
 
 cudaError_t reduce_finalize(lbm_ctx* c) {

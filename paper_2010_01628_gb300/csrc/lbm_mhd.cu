@@ -8,7 +8,8 @@
 namespace lbm {
 
 template <typename S, typename C, bool WALLS, bool FLAT>
-__global__ void __launch_bounds__(256) mhd_step_kernel(const S* __restrict__ src, S* __restrict__ dst, MhdArgs p, FastDiv div_nx) {
+__global__ void __launch_bounds__(256) mhd_step_kernel(const S* __restrict__ src, S* __restrict__ dst, MhdArgs p,
+                                                       FastDiv div_nx) {
     int x, y;
     if (!plane_node<FLAT>(p.box, div_nx, 0, p.box.ny, x, y)) return;
     mhd_node<S, C, WALLS>(src, dst, p, x, y, blockIdx.z);
@@ -77,30 +78,27 @@ __global__ void mhd_fields_kernel(const S* __restrict__ src, FieldsOut out, MhdA
 template <typename S, typename C, bool WALLS>
 __global__ void __launch_bounds__(RED_THREADS) mhd_reduce_kernel(const S* __restrict__ src, MhdArgs p,
                                                                  C* __restrict__ uprev, bool have_prev, bool record,
-                                                                 double* __restrict__ partials) {
+                                                                 double* __restrict__ partials,
+                                                                 NodeDiv div) {
     const Box& b = p.box;
-    const int chunks_x = (b.nx + RED_THREADS - 1) / RED_THREADS;
-    const long total = (long)chunks_x * b.ny * b.nz;
     RedAcc acc;
     acc.zero();
     const C bw[3] = {(C)p.bw[0], (C)p.bw[1], (C)p.bw[2]};
-    for (long ch = blockIdx.x; ch < total; ch += gridDim.x) {
-        const int cxk = (int)(ch % chunks_x);
-        const long row = ch / chunks_x;
-        const int y = (int)(row % b.ny), z = (int)(row / b.ny);
-        const int x = cxk * RED_THREADS + threadIdx.x;
-        if (x < b.nx) {
-            const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
-            const Nbr q = make_nbr(b, x, y, z);
-            C f[Q];
-            gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)0, (C)0, (C)0, f);
-            C g[7][3];
-            gather_mag<S, C, WALLS>(src + (size_t)Q * b.n, b, q, x, y, z, self, bw, g);
-            const Moments<C> mo = moments19(f);
-            C bb[3];
-            const Macro<C> a = mhd_macro<C>(mo, g, p, bb);
-            reduce_node<C>(acc, a.rho, a.ux, a.uy, a.uz, uprev, b.n, self, have_prev, record);
-        }
+    for (uint32_t self = blockIdx.x * RED_THREADS + threadIdx.x; self < (uint32_t)b.n;
+         self += gridDim.x * RED_THREADS) {
+        int x, y, z;
+        node_of(self, b, div, x, y, z);
+        C up[3];
+        load_prev(uprev, b.n, self, have_prev, up);
+        const Nbr q = make_nbr(b, x, y, z);
+        C f[Q];
+        gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)0, (C)0, (C)0, f);
+        C g[7][3];
+        gather_mag<S, C, WALLS>(src + (size_t)Q * b.n, b, q, x, y, z, self, bw, g);
+        const Moments<C> mo = moments19(f);
+        C bb[3];
+        const Macro<C> a = mhd_macro<C>(mo, g, p, bb);
+        reduce_node<C>(acc, a.rho, a.ux, a.uy, a.uz, up, uprev, b.n, self, have_prev, record);
     }
     block_reduce_store(acc, partials);
 }
@@ -127,7 +125,8 @@ static cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
     const dim3 grid = step_grid(c->box, bx, c->box.ny, FLAT);
     for (long s = 0; s < n; ++s) {
         mhd_step_kernel<S, C, WALLS, FLAT>
-            <<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], (S*)c->buf[c->cur ^ 1], p, make_fast_div((uint32_t)c->box.nx));
+            <<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], (S*)c->buf[c->cur ^ 1], p,
+                                         make_fast_div((uint32_t)c->box.nx));
         if (!dry) c->cur ^= 1;
     }
     return cudaGetLastError();
@@ -165,10 +164,10 @@ static cudaError_t reduce_t(lbm_ctx* c, bool record) {
     const MhdArgs p = mhd_args(c);
     if ((c->box.periodic & 7u) != 7u)
         mhd_reduce_kernel<S, C, true><<<RED_BLOCKS, RED_THREADS, 0, c->stream>>>(
-            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials);
+            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials, node_div(c->box));
     else
         mhd_reduce_kernel<S, C, false><<<RED_BLOCKS, RED_THREADS, 0, c->stream>>>(
-            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials);
+            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials, node_div(c->box));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return reduce_finalize(c);

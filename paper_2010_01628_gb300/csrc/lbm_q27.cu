@@ -344,7 +344,8 @@ __device__ __forceinline__ Node<C> macro(const Mom<C>& m, const Args& p) {
 }
 
 template <typename S, typename C, bool WALLS, bool RM, bool FLAT>
-__global__ void __launch_bounds__(256) step_kernel(const S* __restrict__ src, S* __restrict__ dst, Args p, FastDiv div_nx) {
+__global__ void __launch_bounds__(256) step_kernel(const S* __restrict__ src, S* __restrict__ dst, Args p,
+                                                   FastDiv div_nx) {
     const Box& b = p.box;
     const int z = blockIdx.z;
     int x, y;
@@ -423,25 +424,22 @@ __global__ void fields_kernel(const S* __restrict__ src, FieldsOut out, Args p, 
 
 template <typename S, typename C, bool WALLS>
 __global__ void __launch_bounds__(RED_THREADS) reduce_kernel(const S* __restrict__ src, Args p, C* __restrict__ uprev,
-                                                             bool have_prev, bool record, double* __restrict__ partials) {
+                                                             bool have_prev, bool record, double* __restrict__ partials,
+                                                                 NodeDiv div) {
     const Box& b = p.box;
-    const int chunks_x = (b.nx + RED_THREADS - 1) / RED_THREADS;
-    const long total = (long)chunks_x * b.ny * b.nz;
     RedAcc acc;
     acc.zero();
-    for (long ch = blockIdx.x; ch < total; ch += gridDim.x) {
-        const int cxk = (int)(ch % chunks_x);
-        const long row = ch / chunks_x;
-        const int y = (int)(row % b.ny), z = (int)(row / b.ny);
-        const int x = cxk * RED_THREADS + threadIdx.x;
-        if (x < b.nx) {
-            const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
-            const Nbr q = make_nbr(b, x, y, z);
-            C g[3][3][3];
-            gather<S, C, WALLS>(src, b, q, x, y, z, self, p, g);
-            const Node<C> s = macro<C>(moments<C>(g), p);
-            reduce_node<C>(acc, s.rho, s.ux, s.uy, s.uz, uprev, b.n, self, have_prev, record);
-        }
+    for (uint32_t self = blockIdx.x * RED_THREADS + threadIdx.x; self < (uint32_t)b.n;
+         self += gridDim.x * RED_THREADS) {
+        int x, y, z;
+        node_of(self, b, div, x, y, z);
+        C up[3];
+        load_prev(uprev, b.n, self, have_prev, up);
+        const Nbr q = make_nbr(b, x, y, z);
+        C g[3][3][3];
+        gather<S, C, WALLS>(src, b, q, x, y, z, self, p, g);
+        const Node<C> s = macro<C>(moments<C>(g), p);
+        reduce_node<C>(acc, s.rho, s.ux, s.uy, s.uz, up, uprev, b.n, self, have_prev, record);
     }
     block_reduce_store(acc, partials);
 }
@@ -464,7 +462,8 @@ static cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
     const dim3 grid = step_grid(c->box, bx, c->box.ny, FLAT);
     for (long s = 0; s < n; ++s) {
         step_kernel<S, C, WALLS, RM, FLAT>
-            <<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], (S*)c->buf[c->cur ^ 1], p, make_fast_div((uint32_t)c->box.nx));
+            <<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], (S*)c->buf[c->cur ^ 1], p,
+                                         make_fast_div((uint32_t)c->box.nx));
         if (!dry) c->cur ^= 1;
     }
     return cudaGetLastError();
@@ -507,10 +506,10 @@ static cudaError_t reduce_t(lbm_ctx* c, bool record) {
     const Args p = args_of(c);
     if ((c->box.periodic & 7u) != 7u)
         reduce_kernel<S, C, true><<<RED_BLOCKS, RED_THREADS, 0, c->stream>>>((const S*)c->buf[c->cur], p, (C*)c->uprev,
-                                                                             c->have_prev, record, c->partials);
+                                                                             c->have_prev, record, c->partials, node_div(c->box));
     else
         reduce_kernel<S, C, false><<<RED_BLOCKS, RED_THREADS, 0, c->stream>>>(
-            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials);
+            (const S*)c->buf[c->cur], p, (C*)c->uprev, c->have_prev, record, c->partials, node_div(c->box));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return reduce_finalize(c);

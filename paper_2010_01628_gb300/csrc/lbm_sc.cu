@@ -192,26 +192,23 @@ __global__ void sc_fields_kernel(const S* __restrict__ src, const C* __restrict_
 template <typename S, typename C, bool WALLS>
 __global__ void __launch_bounds__(RED_THREADS) sc_reduce_kernel(const S* __restrict__ src, const C* __restrict__ psi,
                                                                 ScArgs p, C* __restrict__ uprev, bool have_prev,
-                                                                bool record, double* __restrict__ partials) {
+                                                                bool record, double* __restrict__ partials,
+                                                                 NodeDiv div) {
     const Box& b = p.box;
-    const int chunks_x = (b.nx + RED_THREADS - 1) / RED_THREADS;
-    const long total = (long)chunks_x * b.ny * b.nz;
     RedAcc acc;
     acc.zero();
-    for (long ch = blockIdx.x; ch < total; ch += gridDim.x) {
-        const int cxk = (int)(ch % chunks_x);
-        const long row = ch / chunks_x;
-        const int y = (int)(row % b.ny), z = (int)(row / b.ny);
-        const int x = cxk * RED_THREADS + threadIdx.x;
-        if (x < b.nx) {
-            const uint32_t self = ((uint32_t)z * (uint32_t)b.ny + (uint32_t)y) * (uint32_t)b.nx + (uint32_t)x;
-            const Nbr q = make_nbr(b, x, y, z);
-            C f[Q];
-            gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
-            const Moments<C> mo = moments19(f);
-            const Macro<C> a = sc_macro<C, WALLS>(mo, psi, b, q, x, y, z, self, p);
-            reduce_node<C>(acc, a.rho, a.ux, a.uy, a.uz, uprev, b.n, self, have_prev, record);
-        }
+    for (uint32_t self = blockIdx.x * RED_THREADS + threadIdx.x; self < (uint32_t)b.n;
+         self += gridDim.x * RED_THREADS) {
+        int x, y, z;
+        node_of(self, b, div, x, y, z);
+        C up[3];
+        load_prev(uprev, b.n, self, have_prev, up);
+        const Nbr q = make_nbr(b, x, y, z);
+        C f[Q];
+        gather19<S, C, WALLS>(src, b, q, x, y, z, self, (C)p.lid[0], (C)p.lid[1], (C)p.lid[2], f);
+        const Moments<C> mo = moments19(f);
+        const Macro<C> a = sc_macro<C, WALLS>(mo, psi, b, q, x, y, z, self, p);
+        reduce_node<C>(acc, a.rho, a.ux, a.uy, a.uz, up, uprev, b.n, self, have_prev, record);
     }
     block_reduce_store(acc, partials);
 }
@@ -310,10 +307,10 @@ static cudaError_t reduce_t(lbm_ctx* c, bool record) {
     launch_psi<S, C>(c, src, p);
     if ((c->box.periodic & 7u) != 7u)
         sc_reduce_kernel<S, C, true><<<RED_BLOCKS, RED_THREADS, 0, c->stream>>>(
-            src, (const C*)c->phi, p, (C*)c->uprev, c->have_prev, record, c->partials);
+            src, (const C*)c->phi, p, (C*)c->uprev, c->have_prev, record, c->partials, node_div(c->box));
     else
         sc_reduce_kernel<S, C, false><<<RED_BLOCKS, RED_THREADS, 0, c->stream>>>(
-            src, (const C*)c->phi, p, (C*)c->uprev, c->have_prev, record, c->partials);
+            src, (const C*)c->phi, p, (C*)c->uprev, c->have_prev, record, c->partials, node_div(c->box));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return reduce_finalize(c);
