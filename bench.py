@@ -545,8 +545,8 @@ def _channel(L, timed, steps, peak, n=512):
     return {f"fluid_regularized_channel_{n}": {
         "MLUPS": n ** 3 * n_c / t / 1e6, "steps": n_c, "bytes_per_lup": 152, "achieved_GBps": ach,
         "frac_of_hbm_peak": ach / peak,
-        "note": "fluid_step_interior_kernel (rows 1..n-2, periodic node code) + fluid_step_wallrows_kernel "
-                "(regularized rebuild of rows 0 and n-1)"}}
+        "note": "fluid_step_channel_kernel (rows 1..n-2 in the periodic node code, regularized rebuild of rows 0 and "
+                "n-1)"}}
 
 
 def apply_launch(L, ctx, spec, tune_cache):

@@ -24,27 +24,46 @@ __global__ void __launch_bounds__(256) fluid_step_kernel(const S* __restrict__ s
     fluid_node<S, C, WALLS, RM, UNFORCED>(src, dst, p, x, y, blockIdx.z);
 }
 
-// Channels (x and z periodic, walls on y, ny >= 3) step in two launches: the
-// interior rows 1 .. ny-2 never pull through a wall and run the periodic node
-// code (40 registers instead of 48); a small launch then updates the two wall
-// rows with bounce-back or regularized walls.
-template <typename S, typename C, bool FLAT>
-__global__ void __launch_bounds__(256) fluid_step_interior_kernel(const S* __restrict__ src, S* __restrict__ dst,
-                                                                  FluidArgs p, FastDiv div_nx) {
-    int x, y;
-    if (!plane_node<FLAT>(p.box, div_nx, 1, p.box.ny - 2, x, y)) return;
-    fluid_node<S, C, false>(src, dst, p, x, y, blockIdx.z);
-}
-
-// The wall rows y = 0 (blockIdx.y = 0) and y = ny - 1 (blockIdx.y = 1) of a
-// channel.  REG: regularized on-node walls; else half-way bounce-back with the lid.
-template <typename S, typename C, bool REG>
-__global__ void __launch_bounds__(256) fluid_step_wallrows_kernel(const S* __restrict__ src, S* __restrict__ dst,
-                                                                  FluidArgs p) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+// Channels (x and z periodic, walls on y, ny >= 3) step in one launch whose CTAs
+// hold either interior rows 1 .. ny-2, which never pull through a wall and run the
+// periodic node code, or wall rows (REG: regularized on-node walls; else half-way
+// bounce-back with the lid): the branch is uniform in a CTA.  FLAT: the first
+// inner_ctas CTAs of a plane number its interior nodes through and the last ones
+// take the wall rows; else CTA row blockIdx.y is y.  The rows of a step are bound by
+// DRAM; the wall rows as a second launch cost its gap and a nearly empty chip (us per
+// step, two launches -> one, FP32 regularized: 250 x 129 x 190 154.7 -> 148.6,
+// 64^3 7.7 -> 6.1, 100 x 3 x 100 4.7 -> 3.3).  The register bound keeps the wall
+// code from taking CTAs from the interior: 48 in FP32 (40, with 16 bytes spilled
+// by the regularized walls: 151.5), 80 in FP64.  In 16 bits, regularized, us per
+// step with 4, 5 or 7 CTAs of 256 per SM: numbered through (250 x 129 x 190)
+// 106.5, 112.3, 114.6 (two launches 107.6), full rows (256 x 128 x 128) 76.1,
+// 71.9, 77.9 (two launches 76.9).  FP64, bound by its pipe: bounce-back 2805 ->
+// 2801, regularized 2853 -> 2867.
+template <typename S, typename C, bool FLAT, bool REG>
+__global__ void __launch_bounds__(256, sizeof(C) == 8 ? 3 : sizeof(S) == 2 && FLAT ? 4 : 5)
+    fluid_step_channel_kernel(const S* __restrict__ src, S* __restrict__ dst, FluidArgs p, FastDiv div_nx,
+                              unsigned inner_ctas) {
     const Box& b = p.box;
-    const int y = blockIdx.y == 0 ? 0 : b.ny - 1, z = blockIdx.z;
-    if (x >= b.nx) return;
+    int x, y;
+    const int z = blockIdx.z;
+    bool wall;
+    if (FLAT) {
+        wall = blockIdx.x >= inner_ctas;
+        if (wall) {
+            const unsigned k = (blockIdx.x - inner_ctas) * blockDim.x + threadIdx.x, nx = (unsigned)b.nx;
+            if (k >= 2 * nx) return;
+            y = k >= nx ? b.ny - 1 : 0;
+            x = (int)(k >= nx ? k - nx : k);
+        } else if (!plane_node<true>(b, div_nx, 1, b.ny - 2, x, y))
+            return;
+    } else {
+        if (!plane_node<false>(b, div_nx, 0, b.ny, x, y)) return;
+        wall = y == 0 || y == b.ny - 1;
+    }
+    if (!wall) {
+        fluid_node<S, C, false>(src, dst, p, x, y, z);
+        return;
+    }
     if (!REG) {
         fluid_node<S, C, true>(src, dst, p, x, y, z);
         return;
@@ -593,19 +612,19 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
     const bool reg = c->grid.wall_model == LBM_WALL_REGULARIZED;
     const bool channel = (c->box.periodic & 7u) == 5u && c->box.ny >= 3;
     if (channel && (reg || c->variant == 0)) {
-        const unsigned gx = (unsigned)((c->box.nx + bx - 1) / bx);
-        const dim3 inner = step_grid(c->box, bx, c->box.ny - 2, flat), rows(gx, 2u, (unsigned)c->box.nz);
+        const unsigned inner = (unsigned)(((size_t)c->box.nx * (c->box.ny - 2) + bx - 1) / bx);
+        dim3 g = grid;
+        if (flat) g.x = inner + (unsigned)((2 * (size_t)c->box.nx + bx - 1) / bx);
         for (long s = 0; s < n; ++s) {
             const S* src = (const S*)c->buf[c->cur];
             S* dst = (S*)c->buf[c->cur ^ 1];
-            if (flat)
-                fluid_step_interior_kernel<S, C, true><<<inner, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
-            else
-                fluid_step_interior_kernel<S, C, false><<<inner, bx, 0, c->stream>>>(src, dst, p, make_fast_div((uint32_t)c->box.nx));
+            const FastDiv div_nx = make_fast_div((uint32_t)c->box.nx);
             if (reg)
-                fluid_step_wallrows_kernel<S, C, true><<<rows, bx, 0, c->stream>>>(src, dst, p);
+                flat ? fluid_step_channel_kernel<S, C, true, true><<<g, bx, 0, c->stream>>>(src, dst, p, div_nx, inner)
+                     : fluid_step_channel_kernel<S, C, false, true><<<g, bx, 0, c->stream>>>(src, dst, p, div_nx, 0);
             else
-                fluid_step_wallrows_kernel<S, C, false><<<rows, bx, 0, c->stream>>>(src, dst, p);
+                flat ? fluid_step_channel_kernel<S, C, true, false><<<g, bx, 0, c->stream>>>(src, dst, p, div_nx, inner)
+                     : fluid_step_channel_kernel<S, C, false, false><<<g, bx, 0, c->stream>>>(src, dst, p, div_nx, 0);
             if (!dry) c->cur ^= 1;
         }
         return cudaGetLastError();
