@@ -501,7 +501,7 @@ lbm_status lbm_batch_info(const lbm_ctx* c, int* threads, int* grid, int* graph,
     if (!c || !c->batch) return LBM_ERR_ARG;
     if (threads) *threads = c->batch->threads;
     if (grid) *grid = (int)c->batch->ntiles;
-    if (graph) *graph = c->graph_failed ? 0 : 1;
+    if (graph) *graph = c->graphs.failed ? 0 : 1;
     if (tiles) *tiles = (long)c->batch->ntiles;
     return LBM_OK;
 }

@@ -108,83 +108,11 @@ cudaError_t phys_reduce(lbm_ctx* c, bool record) {
     return cudaErrorInvalidValue;
 }
 
-// Steps of one captured graph (even, so that a replay leaves buf[cur] current).
-// On this GPU a kernel that follows another in a stream starts 2.4 us later
-// than the same kernel as the next node of a graph (chains of small dependent
-// kernels: 4.1 us each in a stream, 1.8 us in a graph; at 1 M nodes 24.7 and
-// 22.3 us), so steps are replayed 16 at a time and the rest of a call 4 at a time.
-// More steps per graph gain nothing (the stream's gap between two graphs is
-// 0.15 us a step at 16) and make the capture, paid once per context and launch
-// shape, longer.
-constexpr long STEP_GRAPH[2] = {16, 4};
-
-void drop_step_graphs(lbm_ctx* c, bool wait) {
-    bool any = false;
-    for (auto& of_size : c->step_graph)
-        for (cudaGraphExec_t& g : of_size) {
-            if (g && wait && !any) cudaStreamSynchronize(c->stream);  // may still be running
-            any = any || g;
-            if (g) cudaGraphExecDestroy(g);
-            g = nullptr;
-        }
-}
-
-// The graph of STEP_GRAPH[size] steps from the current buffer, captured on the
-// context's own copy stream (idle between field transfers) at first use and
-// again after a change of launch shape; nullptr if it cannot be made.
-cudaGraphExec_t step_graph(lbm_ctx* c, int size) {
-    const int shape[6] = {c->variant, c->block_x, c->tma_stages, c->tma_ctas, c->zchunk, c->fused_threads};
-    if (std::memcmp(shape, c->step_graph_shape, sizeof(shape)) != 0) {
-        drop_step_graphs(c, true);
-        std::memcpy(c->step_graph_shape, shape, sizeof(shape));
-    }
-    const int k = c->cur;
-    cudaGraphExec_t& exec = c->step_graph[size][k];
-    if (exec) return exec;
-    cudaGraph_t g = nullptr;
-    const cudaStream_t user = c->stream;
-    // relaxed: neither disturbs nor is disturbed by a capture on another thread
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    if (cudaStreamBeginCapture(c->copy_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
-        cudaGetLastError();
-        cudaThreadExchangeStreamCaptureMode(&mode);
-        return nullptr;
-    }
-    c->stream = c->copy_stream;
-    const cudaError_t el = phys_step(c, STEP_GRAPH[size]);
-    c->stream = user;
-    c->cur = k;
-    cudaError_t e = cudaStreamEndCapture(c->copy_stream, &g);
-    if (e == cudaSuccess) e = el;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
-    if (g) cudaGraphDestroy(g);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        exec = nullptr;
-    }
-    c->graph_failed = e != cudaSuccess;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    return exec;
-}
-
-// n steps on the context stream: whole graphs, then single launches.  While
-// the caller is capturing the stream every step is a plain launch, which the
-// capture records.
+// n steps on the context stream (lbm_step_graphs.h).
 cudaError_t run_steps(lbm_ctx* c, long n) {
-    if (n >= STEP_GRAPH[0]) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        const bool plain = cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
-        if (plain) cudaGetLastError();
-        for (int size = 0; size < 2 && !plain; ++size) {
-            const cudaGraphExec_t g = n >= STEP_GRAPH[size] ? step_graph(c, size) : nullptr;
-            for (; g && n >= STEP_GRAPH[size]; n -= STEP_GRAPH[size]) {
-                const cudaError_t e = cudaGraphLaunch(g, c->stream);
-                if (e != cudaSuccess) return e;
-            }
-        }
-    }
-    return n > 0 ? phys_step(c, n) : cudaSuccess;
+    const int shape[6] = {c->variant, c->block_x, c->tma_stages, c->tma_ctas, c->zchunk, c->fused_threads};
+    return lbm::run_steps(c->graphs, shape, c->stream, c->copy_stream, c->cur, n,
+                          [c](long steps) { return phys_step(c, steps); });
 }
 
 // Initialisation from, and fields to, whole-domain arrays: one launch (more for
@@ -217,7 +145,7 @@ cudaError_t fields_in_place(lbm_ctx* c, const lbm::FieldsOut& out) {
 
 void release_all(lbm_ctx* c) {
     if (!c->owns) return;
-    drop_step_graphs(c, false);
+    c->graphs.drop(nullptr);
     for (int k = 0; k < 2; ++k) dev_free(c, c->buf[k]);
     dev_free(c, c->phi);
     dev_free(c, c->uprev);

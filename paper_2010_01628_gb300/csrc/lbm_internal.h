@@ -5,9 +5,9 @@
 
 #include <string>
 
-
 #include "../../include/lbm.h"
 #include "lbm_device.cuh"
+#include "lbm_step_graphs.h"
 
 struct BatchState;
 
@@ -51,9 +51,7 @@ struct lbm_ctx {
     int sms = 0;
     int* status = nullptr;  // device status word written by bounded waits
     bool bounded_waits = false;  // a kernel that may write `status` has been launched
-    cudaGraphExec_t step_graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [STEP_GRAPH size][buf current]
-    bool graph_failed = false;  // a capture did not succeed: steps are launched one by one
-    int step_graph_shape[6] = {-1, -1, -1, -1, -1, -1};  // launch shape the graphs were captured with
+    lbm::StepGraphs graphs;
     std::string err;
     bool owns = true;            // false for the per-domain views of a batch
     lbm_ctx* parent = nullptr;   // the batch a view belongs to
