@@ -22,7 +22,7 @@ constexpr long STEP_GRAPH[2] = {16, 4};
 struct StepGraphs {
     cudaGraphExec_t exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [STEP_GRAPH size][buf current]
     int shape[6] = {-1, -1, -1, -1, -1, -1};  // launch shape of the graphs
-    bool failed = false;  // of this shape's graphs one could not be made: steps are launched one by one
+    bool failed = false;  // of this shape's graphs one could not be made or launched: steps are launched one by one
 
     bool any() const { return exec[0][0] || exec[0][1] || exec[1][0] || exec[1][1]; }
 
@@ -93,9 +93,12 @@ cudaError_t run_steps(StepGraphs& g, const int (&shape)[6], cudaStream_t& stream
             g.failed = !exec;
         }
         for (long s = 0; s < steps && !g.failed; s += STEP_GRAPH[size]) {
-            const cudaError_t e = cudaGraphLaunch(exec, stream);
-            if (e != cudaSuccess) return e;
-            n -= STEP_GRAPH[size];
+            // a refused replay (no device memory left for the graph) has run nothing
+            g.failed = cudaGraphLaunch(exec, stream) != cudaSuccess;
+            if (g.failed)
+                cudaGetLastError();
+            else
+                n -= STEP_GRAPH[size];
         }
     }
     return n > 0 ? launch(n) : cudaSuccess;

@@ -1,4 +1,4 @@
-"""When steps are replayed from captured graphs, and what follows a failed capture or instantiation: the host
+"""When steps are replayed from captured graphs, and what follows a failed capture, instantiation or replay: the host
 code of lbm_step_graphs.h against a fake of the CUDA runtime that records its calls and fails the wanted one."""
 import os
 import shutil
@@ -128,6 +128,10 @@ def test_a_failed_capture_is_not_tried_again(harness, call):
     assert out == ["0/64/1F", "0/64/0F", "0/64/0F"]
     # the graph of 4 steps fails after that of 16 was made
     assert harness(32, f"fail:{call}:-1", 44, f"ok:{call}", 44) == ["32/0/1", "32/12/1F", "0/44/0F"]
+
+
+def test_a_refused_replay_falls_back_to_launches(harness):
+    assert harness("fail:replay:2", 64, 64) == ["16/48/1F", "0/64/0F"]
 
 
 def test_a_new_launch_shape_starts_over(harness):
