@@ -18,9 +18,20 @@ namespace lbm {
 // 0.15 us a step at 16) and make the capture, paid once per context and launch
 // shape, longer.  Calls of fewer than 16 steps are launched step by step.
 constexpr long STEP_GRAPH[2] = {16, 4};
+// A graph is made once the steps it could have replayed, those of the present
+// call among them, reach these counts: its capture and instantiation cost what it
+// saves over about as many steps (16 steps of one launch: 60 us against 2.3 us a
+// step; Shan-Chen, two launches: 90 against 4.4; a batch, with up to 32 KB of
+// parameters a launch: 185 against 5.8).  A context that is stepped little then
+// pays for plain launches alone.  Made at once, the first 16 steps of a fresh
+// context took 109 us instead of 88 (256^2 fluid), 169 instead of 153 (32^3
+// Shan-Chen), 321 instead of 258 (four 32^3 Shan-Chen domains), and calls of 31
+// steps of that batch 470 instead of 440.
+constexpr long STEP_GRAPH_AFTER[2] = {32, 16};
 
 struct StepGraphs {
     cudaGraphExec_t exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [STEP_GRAPH size][buf current]
+    long missed[2][2] = {{0, 0}, {0, 0}};  // steps that the graph could have replayed
     int shape[6] = {-1, -1, -1, -1, -1, -1};  // launch shape of the graphs
     bool failed = false;  // of this shape's graphs one could not be made or launched: steps are launched one by one
 
@@ -33,6 +44,7 @@ struct StepGraphs {
             for (int k = 0; k < 2; ++k) {
                 if (exec[size][k]) cudaGraphExecDestroy(exec[size][k]);
                 exec[size][k] = nullptr;
+                missed[size][k] = 0;
             }
         failed = false;
     }
@@ -85,6 +97,8 @@ cudaError_t run_steps(StepGraphs& g, const int (&shape)[6], cudaStream_t& stream
         const long steps = (size == 0 ? n : n % STEP_GRAPH[0]) / STEP_GRAPH[size] * STEP_GRAPH[size];
         cudaGraphExec_t& exec = g.exec[size][k];
         if (!exec && steps > 0) {
+            g.missed[size][k] += steps;
+            if (g.missed[size][k] < STEP_GRAPH_AFTER[size]) continue;
             const cudaStream_t user = stream;
             stream = capture;
             exec = capture_graph(capture, [&] { return launch(STEP_GRAPH[size]); });

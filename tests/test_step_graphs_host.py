@@ -115,11 +115,18 @@ def harness(tmp_path_factory):
     return run
 
 
-def test_long_calls_replay_and_short_ones_never(harness):
+def test_long_calls_replay_at_once_and_short_ones_never(harness):
     assert harness(32) == ["32/0/1"]
-    assert harness(100, 100, 100) == ["100/0/2", "100/0/0", "100/0/0"]
-    assert harness(47, 47) == ["44/3/2", "44/3/2"]  # the other buffer is current in the second call
+    assert harness(100, 100, 100, 100) == ["96/4/1", "96/4/0", "96/4/0", "100/0/1"]
+    assert harness(47, 47) == ["32/15/1", "32/15/1"]  # the other buffer is current in the second call
     assert harness(*[15] * 20) == ["0/15/0"] * 20
+
+
+def test_first_short_calls_of_a_context_are_not_captured(harness):
+    assert harness(16) == ["0/16/0"]
+    assert harness(16, 16, 16) == ["0/16/0", "16/0/1", "16/0/0"]
+    # 31 = 16 + 12 + 3, the buffers in turn
+    assert harness(*[31] * 6) == ["0/31/0", "0/31/0", "28/3/2", "28/3/2", "28/3/0", "28/3/0"]
 
 
 @pytest.mark.parametrize("call", ["begin", "end", "instantiate"])
@@ -127,7 +134,7 @@ def test_a_failed_capture_is_not_tried_again(harness, call):
     out = harness(f"fail:{call}:-1", 64, f"ok:{call}", 64, 64)
     assert out == ["0/64/1F", "0/64/0F", "0/64/0F"]
     # the graph of 4 steps fails after that of 16 was made
-    assert harness(32, f"fail:{call}:-1", 44, f"ok:{call}", 44) == ["32/0/1", "32/12/1F", "0/44/0F"]
+    assert harness(44, f"fail:{call}:-1", 44, f"ok:{call}", 44) == ["32/12/1", "32/12/1F", "0/44/0F"]
 
 
 def test_a_refused_replay_falls_back_to_launches(harness):
@@ -136,7 +143,7 @@ def test_a_refused_replay_falls_back_to_launches(harness):
 
 def test_a_new_launch_shape_starts_over(harness):
     assert harness("fail:instantiate:-1", 64, "ok:instantiate", "shape:2", 64, 64) == ["0/64/1F", "64/0/1", "64/0/0"]
-    assert harness(64, "shape:2", 16, 64) == ["64/0/1", "16/0/1", "64/0/0"]
+    assert harness(64, "shape:2", 16, 64) == ["64/0/1", "0/16/0", "64/0/1"]
 
 
 def test_a_callers_capture_records_plain_launches(harness):
