@@ -187,6 +187,8 @@ struct BatchState {
     int nd = 0;
     std::vector<lbm_ctx*> views;
     std::vector<BatchDomain> doms;
+    std::vector<unsigned char> tabs;  // a BatchTab per launch of a pass (configure)
+    std::vector<uint32_t> tiles;      // CTAs of each
     uint32_t ntiles = 0;
     int threads = 256;
     size_t state_elems = 0;
@@ -196,34 +198,32 @@ struct BatchState {
 
 namespace {
 
-// Tiles of the current CTA size.
-void configure(lbm_ctx* c) {
-    BatchState* B = c->batch;
-    B->ntiles = 0;
-    for (auto& d : B->doms) {
-        d.ntiles = (uint32_t)((d.fl.box.n + B->threads - 1) / B->threads);
-        B->ntiles += d.ntiles;
-    }
-    c->block_x = B->threads;  // part of the launch shape that captured graphs are kept for
-}
-
 const lbm::FluidArgs& args_of(const BatchDomain& d, lbm::FluidArgs*) { return d.fl; }
 const lbm::MhdArgs& args_of(const BatchDomain& d, lbm::MhdArgs*) { return d.mh; }
 const lbm::CgmArgs& args_of(const BatchDomain& d, lbm::CgmArgs*) { return d.cg; }
 const lbm::ScArgs& args_of(const BatchDomain& d, lbm::ScArgs*) { return d.sc; }
 
-template <int PHYS, typename S, typename C, bool WALLS>
-cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
+template <int PHYS>
+using TabOf = lbm::BatchTab<typename lbm::BatchArgs<PHYS>::T>;
+size_t tab_bytes(lbm_physics p) {
+    switch (p) {
+        case LBM_PHYS_MHD: return sizeof(TabOf<LBM_PHYS_MHD>);
+        case LBM_PHYS_CGM: return sizeof(TabOf<LBM_PHYS_CGM>);
+        case LBM_PHYS_SC: return sizeof(TabOf<LBM_PHYS_SC>);
+        default: return sizeof(TabOf<LBM_PHYS_FLUID>);
+    }
+}
+int launches_per_pass(int ndomains) { return (ndomains + lbm::BATCH_TAB - 1) / lbm::BATCH_TAB; }
+
+template <int PHYS>
+void fill_tabs(BatchState* B) {
     using Args = typename lbm::BatchArgs<PHYS>::T;
-    using Tab = lbm::BatchTab<Args>;
-    static_assert(sizeof(Tab) <= 32000, "kernel parameters are limited to 32,764 bytes");
-    BatchState* B = c->batch;
-    const int chunks = (B->nd + lbm::BATCH_TAB - 1) / lbm::BATCH_TAB;
-    std::vector<Tab> tabs((size_t)chunks);
-    std::vector<uint32_t> tiles((size_t)chunks, 0u);
+    static_assert(sizeof(TabOf<PHYS>) <= 32000, "kernel parameters are limited to 32,764 bytes");
+    TabOf<PHYS>* tabs = (TabOf<PHYS>*)B->tabs.data();
+    std::fill(B->tiles.begin(), B->tiles.end(), 0u);
     for (int d = 0; d < B->nd; ++d) {
-        Tab& t = tabs[d / lbm::BATCH_TAB];
-        uint32_t& next = tiles[d / lbm::BATCH_TAB];
+        TabOf<PHYS>& t = tabs[d / lbm::BATCH_TAB];
+        uint32_t& next = B->tiles[d / lbm::BATCH_TAB];
         const int k = d % lbm::BATCH_TAB;
         const BatchDomain& D = B->doms[d];
         t.nd = k + 1;
@@ -235,6 +235,32 @@ cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
         t.rec[k].div_ny = D.div_ny;
         next += D.ntiles;
     }
+}
+
+// Tiles and tables of the current CTA size.  A step allocates nothing: it runs
+// inside stream captures and behind a C entry point.
+void configure(lbm_ctx* c) {
+    BatchState* B = c->batch;
+    B->ntiles = 0;
+    for (auto& d : B->doms) {
+        d.ntiles = (uint32_t)((d.fl.box.n + B->threads - 1) / B->threads);
+        B->ntiles += d.ntiles;
+    }
+    switch (c->physics) {
+        case LBM_PHYS_MHD: fill_tabs<LBM_PHYS_MHD>(B); break;
+        case LBM_PHYS_CGM: fill_tabs<LBM_PHYS_CGM>(B); break;
+        case LBM_PHYS_SC: fill_tabs<LBM_PHYS_SC>(B); break;
+        default: fill_tabs<LBM_PHYS_FLUID>(B); break;
+    }
+    c->block_x = B->threads;  // part of the launch shape that captured graphs are kept for
+}
+
+template <int PHYS, typename S, typename C, bool WALLS>
+cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
+    BatchState* B = c->batch;
+    const TabOf<PHYS>* tabs = (const TabOf<PHYS>*)B->tabs.data();
+    const std::vector<uint32_t>& tiles = B->tiles;
+    const int chunks = (int)tiles.size();
     for (long s = 0; s < n; ++s) {
         const S* src = (const S*)c->buf[c->cur];
         S* dst = (S*)c->buf[c->cur ^ 1];
@@ -369,7 +395,16 @@ lbm_status lbm_batch_create(lbm_ctx** out, int ndomains, const lbm_grid* grids, 
     c->box.nx = c->box.ny = c->box.nz = 0;
     c->box.n = cells;
     B->nd = ndomains;
-    lbm_status st = lbm_internal_alloc_batch(c, total, cells, max_plane);
+    lbm_status st = LBM_OK;
+    try {
+        B->doms.reserve(ndomains);
+        B->views.reserve(ndomains);
+        B->tiles.resize(launches_per_pass(ndomains));
+        B->tabs.resize(B->tiles.size() * tab_bytes(physics));
+    } catch (const std::bad_alloc&) {
+        st = LBM_ERR_OOM;
+    }
+    if (st == LBM_OK) st = lbm_internal_alloc_batch(c, total, cells, max_plane);
     if (st != LBM_OK) {
         lbm::batch_destroy(c);
         lbm_internal_release(c);
