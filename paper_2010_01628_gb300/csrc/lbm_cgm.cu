@@ -226,8 +226,9 @@ static cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
 }
 template <typename S, typename C>
 static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
-    const bool flat = step_flat(c->box, c->block_x);
-    switch (c->box.periodic & 7u) {
+    const unsigned periodic = c->box.periodic & 7u;
+    const bool flat = step_flat(c->box, c->block_x, sizeof(S) != 4 || periodic == 7u ? 0 : periodic == 5u ? 20 : 15);
+    switch (periodic) {
         case 7u: return flat ? steps_t<S, C, 0, true>(c, n, dry) : steps_t<S, C, 0, false>(c, n, dry);
         case 5u: return flat ? steps_t<S, C, 2, true>(c, n, dry) : steps_t<S, C, 2, false>(c, n, dry);
         default: return flat ? steps_t<S, C, 1, true>(c, n, dry) : steps_t<S, C, 1, false>(c, n, dry);

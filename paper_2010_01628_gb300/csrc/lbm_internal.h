@@ -149,7 +149,24 @@ void batch_destroy(lbm_ctx* c);
 // fluid 37.6 -> 42.6, Shan-Chen 22.7 -> 25.6, colour gradient 13.9 -> 15.8).
 // Full rows keep the row form, whose index arithmetic is uniform (256^3
 // Shan-Chen 27.5 against 26.4, 64 x 256 x 64 colour gradient 15.2 against 13.3).
-inline bool step_flat(const Box& b, int bx) { return b.nx % bx != 0; }
+// Where that arithmetic costs a kernel more than rows that nearly fill their warps
+// waste, rows are kept there too: `worth` is the idle share of a row's threads, in
+// percent of nx, from which the kernel is faster numbered through.  Threads are
+// counted in whole warps (empty warps of a CTA leave at once), in CTAs up to 64
+// threads.  Time numbered through / in rows, nx x 128 x 64, FP32, default CTAs:
+//   nx (idle %)               72 (78) 100 (28) 112 (14) 136 (18) 160 (0) 240 (7) 252 (2)
+//   colour gradient, y walls    0.76    1.01     1.08     1.03     1.14    1.17    1.19
+//   colour gradient, walls      0.72    0.95     1.05     0.97     1.09    1.14    1.16
+//   D3Q27, walls                0.80    0.97     1.03     0.97     1.05    1.05    1.06
+//   Shan-Chen, periodic         0.63    0.86     0.95     0.93     1.02    1.02    1.03
+// and the other kernels, FP64 and 16 bits among them, 0.5 .. 1.02 at every width.
+// (With every ragged row numbered through, walled colour-gradient boxes of 160 to
+// 500 nodes a row were up to 14 % slower than before there was a numbered form.)
+inline bool step_flat(const Box& b, int bx, int worth = 0) {
+    if (b.nx % bx == 0) return false;
+    const long unit = bx <= 64 ? bx : 32, idle = (b.nx + unit - 1) / unit * unit - b.nx;
+    return idle * 100 >= (long)worth * b.nx;
+}
 inline dim3 step_grid(const Box& b, int bx, int rows, bool flat) {
     return flat ? dim3((unsigned)(((size_t)b.nx * rows + bx - 1) / bx), 1u, (unsigned)b.nz)
                 : dim3((unsigned)((b.nx + bx - 1) / bx), (unsigned)rows, (unsigned)b.nz);

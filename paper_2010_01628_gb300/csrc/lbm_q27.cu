@@ -470,8 +470,9 @@ static cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
 }
 template <typename S, typename C, bool WALLS, bool RM>
 static cudaError_t steps_flat_t(lbm_ctx* c, long n, bool dry) {
-    return step_flat(c->box, c->block_x) ? steps_t<S, C, WALLS, RM, true>(c, n, dry)
-                                         : steps_t<S, C, WALLS, RM, false>(c, n, dry);
+    return step_flat(c->box, c->block_x, sizeof(S) == 4 && WALLS && !RM ? 15 : 0)
+               ? steps_t<S, C, WALLS, RM, true>(c, n, dry)
+               : steps_t<S, C, WALLS, RM, false>(c, n, dry);
 }
 template <typename S, typename C>
 static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {

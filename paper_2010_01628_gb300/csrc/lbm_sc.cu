@@ -232,9 +232,13 @@ static void launch_psi(lbm_ctx* c, const S* src, const ScArgs& p) {
     sc_psi_kernel<S, C, WALLS, FLAT>
         <<<step_grid(c->box, c->block_x, c->box.ny, FLAT), c->block_x, 0, c->stream>>>(src, (C*)c->phi, p, make_fast_div((uint32_t)c->box.nx));
 }
+template <typename S>
+static bool sc_flat(const lbm_ctx* c) {
+    return step_flat(c->box, c->block_x, sizeof(S) == 4 && (c->box.periodic & 7u) == 7u ? 7 : 0);
+}
 template <typename S, typename C>
 static void launch_psi(lbm_ctx* c, const S* src, const ScArgs& p) {
-    const bool walls = (c->box.periodic & 7u) != 7u, flat = step_flat(c->box, c->block_x);
+    const bool walls = (c->box.periodic & 7u) != 7u, flat = sc_flat<S>(c);
     if (walls)
         flat ? launch_psi<S, C, true, true>(c, src, p) : launch_psi<S, C, true, false>(c, src, p);
     else
@@ -272,7 +276,7 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
         }
         return cudaGetLastError();
     }
-    const bool flat = step_flat(c->box, bx);
+    const bool flat = sc_flat<S>(c);
     for (long s = 0; s < n; ++s) {
         const S* src = (const S*)c->buf[c->cur];
         S* dst = (S*)c->buf[c->cur ^ 1];
