@@ -16,9 +16,13 @@
  *  - Lattice units (dx = dt = 1), c_s^2 = 1/3, omega = 1/(nu/c_s^2 + 1/2).
  *  - Fields are FP64, layout [nz][ny][nx] with x fastest; vectors (u, B) are
  *    three such planes back to back (x, y, z components).
- *  - Field pointers may be host memory (pageable or pinned) or device memory
- *    of the context's GPU; the library copies with cudaMemcpyAsync on the
- *    context stream and synchronises before returning.
+ *  - Field pointers may be host memory (pageable or pinned), device memory of
+ *    the context's GPU or managed memory.  When every array of a call is device
+ *    memory of that GPU, aligned to 8 bytes and inside one allocation each,
+ *    kernels on the context stream read or write the arrays where they are;
+ *    otherwise they are copied through staging slabs on a stream of the
+ *    library's own, ordered after the context stream.  The call synchronises
+ *    before returning.
  *  - The caller owns every pointer it passes in.  The library owns its device
  *    buffers (populations, scratch), obtained from the allocator installed with
  *    lbm_set_allocator, else cudaMalloc.
