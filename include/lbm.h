@@ -205,7 +205,7 @@ lbm_status lbm_set_populations(lbm_ctx *ctx, const void *src, size_t bytes);
  * Many independent domains (uneven sizes, per-domain omega, force, wall field,
  * density ratio, surface tension) advanced together: a step is one launch over
  * the nodes of all domains (two for the two-phase modules: order parameter or
- * pseudopotential, then collision; more launches beyond 128 domains), and 16
+ * pseudopotential, then collision; more for over 128 large domains), and 16
  * steps at a time are replayed from a captured CUDA graph.  Physics:
  * LBM_PHYS_FLUID, LBM_PHYS_MHD, LBM_PHYS_CGM (App. E colour gradient) or
  * LBM_PHYS_SC (Sec. III.G Shan-Chen), whose batch holds the phi and rho_r (psi)

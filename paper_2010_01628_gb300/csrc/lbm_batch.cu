@@ -9,8 +9,9 @@
 // parameters: a CTA finds its domain by a binary search in the constant bank and
 // starts its pulls at once (the same tables in global memory put two dependent
 // loads before them: 64-domain Shan-Chen sweep 18.6 GLUPS instead of 27.4).
-// More domains take more launches.  The colour-gradient and Shan-Chen steps take two passes
-// (order parameter or pseudopotential, then collision).
+// More domains take more launches, or one with the tables in device memory
+// (batch_many).  The colour-gradient and Shan-Chen steps take two passes (order
+// parameter or pseudopotential, then collision).
 //
 // A launch per pass beats a persistent kernel that holds both passes and
 // synchronises the grid between them: each pass keeps its own register count
@@ -44,7 +45,6 @@ struct BatchDomain {
     size_t off;       // element offset of the domain's plane 0 in a state copy
     size_t soff;      // offset of the domain's node 0 in each scratch plane (colour gradient)
     FastDiv div_nx, div_ny;
-    uint32_t ntiles;
 };
 
 struct BarrierState {
@@ -114,6 +114,17 @@ struct BatchTab {
     uint32_t tile0[BATCH_TAB];
     BatchRec<Args> rec[BATCH_TAB];
 };
+// All domains of the batch, in global memory.
+template <class Args>
+struct BatchRecAt {
+    BatchRec<Args> r;
+    uint32_t tile0;
+};
+template <class Args>
+struct BatchMany {
+    const BatchRecAt<Args>* rec;
+    const uint32_t* domain;  // of each tile
+};
 
 template <int PHYS> struct BatchArgs;
 template <> struct BatchArgs<LBM_PHYS_FLUID> { using T = FluidArgs; };
@@ -136,10 +147,8 @@ constexpr int batch_ctas(int phys, int pass, size_t elem) {
     if (phys == LBM_PHYS_CGM) return 5;
     return 6;
 }
-template <int PHYS, int PASS, typename S, typename C, bool WALLS>
-__global__ void __launch_bounds__(256, batch_ctas(PHYS, PASS, sizeof(S)))
-    batch_pass_kernel(const S* __restrict__ src, S* __restrict__ dst, C* __restrict__ scratch, size_t scratch_n,
-                      const __grid_constant__ BatchTab<typename BatchArgs<PHYS>::T> tab) {
+template <class Args>
+__device__ __forceinline__ const BatchRec<Args>& batch_domain(const BatchTab<Args>& tab, uint32_t& tile0) {
     int lo = 0, hi = tab.nd - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -148,9 +157,23 @@ __global__ void __launch_bounds__(256, batch_ctas(PHYS, PASS, sizeof(S)))
         else
             hi = mid - 1;
     }
-    const auto& D = tab.rec[lo];
+    tile0 = tab.tile0[lo];
+    return tab.rec[lo];
+}
+template <class Args>
+__device__ __forceinline__ const BatchRec<Args>& batch_domain(const BatchMany<Args>& tab, uint32_t& tile0) {
+    const BatchRecAt<Args>& at = tab.rec[__ldg(tab.domain + blockIdx.x)];
+    tile0 = at.tile0;
+    return at.r;
+}
+template <int PHYS, int PASS, typename S, typename C, bool WALLS, class Tab>
+__global__ void __launch_bounds__(256, batch_ctas(PHYS, PASS, sizeof(S)))
+    batch_pass_kernel(const S* __restrict__ src, S* __restrict__ dst, C* __restrict__ scratch, size_t scratch_n,
+                      const __grid_constant__ Tab tab) {
+    uint32_t tile0;
+    const auto& D = batch_domain(tab, tile0);
     const Box& b = D.a.box;
-    const uint32_t cell = (blockIdx.x - tab.tile0[lo]) * blockDim.x + threadIdx.x;
+    const uint32_t cell = (blockIdx.x - tile0) * blockDim.x + threadIdx.x;
     if (cell >= (uint32_t)b.n) return;
     const uint32_t row = fast_div(cell, D.div_nx);
     const int x = (int)(cell - row * (uint32_t)b.nx);
@@ -187,8 +210,16 @@ struct BatchState {
     int nd = 0;
     std::vector<lbm_ctx*> views;
     std::vector<BatchDomain> doms;
-    std::vector<unsigned char> tabs;  // a BatchTab per launch of a pass (configure)
-    std::vector<uint32_t> tiles;      // CTAs of each
+    bool many = false;                // tables in device memory, one launch a pass
+    std::vector<unsigned char> tabs;  // a BatchTab per launch of a pass, or (many) all records
+    std::vector<uint32_t> tiles;      // CTAs of each launch
+    std::vector<uint32_t> domain;     // many: domain of each tile
+    // many: device copies, by threads / 32; written once, as a caller's graph may
+    // hold steps of an earlier CTA size
+    struct {
+        void* rec = nullptr;
+        uint32_t* domain = nullptr;
+    } device[256 / 32 + 1];
     uint32_t ntiles = 0;
     int threads = 256;
     size_t state_elems = 0;
@@ -198,6 +229,19 @@ struct BatchState {
 
 namespace {
 
+// Whether a batch keeps its tables in device memory: more domains than one
+// launch's parameters hold, and few nodes a launch.  One launch of all domains
+// then beats a launch of 32 KB of parameters per 128 of them; large domains hide
+// the launches, and in FP32 the parameters' constant bank is the faster table.
+// us per step, 16-step graphs, parameters -> device memory: 1000 x 8^3 fluid FP32
+// 24.6 -> 11.2, colour gradient 83 -> 38, 4000 x 6^3 Shan-Chen 170 -> 39, 129 x 8^3
+// Shan-Chen FP64 80 -> 53; 512 x 16^3 (2^19 nodes a launch) FP32 0.92 .. 1.03, 1000
+// x 20^3 (10^6) 0.93 .. 1.06, 130 x 64^3 1.00 .. 1.13; FP64 0.92 .. 1.01 at every size.
+bool batch_many(int ndomains, size_t cells, lbm_precision prec) {
+    const size_t launches = (size_t)(ndomains + lbm::BATCH_TAB - 1) / lbm::BATCH_TAB;
+    return launches > 1 && (prec == LBM_FP64 || cells < launches << 19);
+}
+
 const lbm::FluidArgs& args_of(const BatchDomain& d, lbm::FluidArgs*) { return d.fl; }
 const lbm::MhdArgs& args_of(const BatchDomain& d, lbm::MhdArgs*) { return d.mh; }
 const lbm::CgmArgs& args_of(const BatchDomain& d, lbm::CgmArgs*) { return d.cg; }
@@ -205,72 +249,110 @@ const lbm::ScArgs& args_of(const BatchDomain& d, lbm::ScArgs*) { return d.sc; }
 
 template <int PHYS>
 using TabOf = lbm::BatchTab<typename lbm::BatchArgs<PHYS>::T>;
-size_t tab_bytes(lbm_physics p) {
-    switch (p) {
-        case LBM_PHYS_MHD: return sizeof(TabOf<LBM_PHYS_MHD>);
-        case LBM_PHYS_CGM: return sizeof(TabOf<LBM_PHYS_CGM>);
-        case LBM_PHYS_SC: return sizeof(TabOf<LBM_PHYS_SC>);
-        default: return sizeof(TabOf<LBM_PHYS_FLUID>);
+template <int PHYS>
+using RecOf = lbm::BatchRecAt<typename lbm::BatchArgs<PHYS>::T>;
+template <int PHYS>
+size_t table_bytes_of(const BatchState* B) {
+    static_assert(sizeof(TabOf<PHYS>) <= 32000, "kernel parameters are limited to 32,764 bytes");
+    return B->many ? B->nd * sizeof(RecOf<PHYS>) : B->tiles.size() * sizeof(TabOf<PHYS>);
+}
+size_t table_bytes(const lbm_ctx* c) {
+    switch (c->physics) {
+        case LBM_PHYS_MHD: return table_bytes_of<LBM_PHYS_MHD>(c->batch);
+        case LBM_PHYS_CGM: return table_bytes_of<LBM_PHYS_CGM>(c->batch);
+        case LBM_PHYS_SC: return table_bytes_of<LBM_PHYS_SC>(c->batch);
+        default: return table_bytes_of<LBM_PHYS_FLUID>(c->batch);
     }
 }
-int launches_per_pass(int ndomains) { return (ndomains + lbm::BATCH_TAB - 1) / lbm::BATCH_TAB; }
+uint32_t tiles_of(const BatchDomain& d, int threads) { return (uint32_t)((d.fl.box.n + threads - 1) / threads); }
 
 template <int PHYS>
-void fill_tabs(BatchState* B) {
+void fill_tables(BatchState* B) {
     using Args = typename lbm::BatchArgs<PHYS>::T;
-    static_assert(sizeof(TabOf<PHYS>) <= 32000, "kernel parameters are limited to 32,764 bytes");
-    TabOf<PHYS>* tabs = (TabOf<PHYS>*)B->tabs.data();
     std::fill(B->tiles.begin(), B->tiles.end(), 0u);
     for (int d = 0; d < B->nd; ++d) {
-        TabOf<PHYS>& t = tabs[d / lbm::BATCH_TAB];
-        uint32_t& next = B->tiles[d / lbm::BATCH_TAB];
-        const int k = d % lbm::BATCH_TAB;
         const BatchDomain& D = B->doms[d];
-        t.nd = k + 1;
-        t.tile0[k] = next;
-        t.rec[k].a = args_of(D, (Args*)nullptr);
-        t.rec[k].off = D.off;
-        t.rec[k].soff = D.soff;
-        t.rec[k].div_nx = D.div_nx;
-        t.rec[k].div_ny = D.div_ny;
-        next += D.ntiles;
+        const int launch = B->many ? 0 : d / lbm::BATCH_TAB;
+        const uint32_t tile0 = B->tiles[launch], n = tiles_of(D, B->threads);
+        lbm::BatchRec<Args>* r;
+        if (B->many) {
+            RecOf<PHYS>& at = ((RecOf<PHYS>*)B->tabs.data())[d];
+            at.tile0 = tile0;
+            std::fill_n(B->domain.begin() + tile0, n, (uint32_t)d);
+            r = &at.r;
+        } else {
+            TabOf<PHYS>& t = ((TabOf<PHYS>*)B->tabs.data())[launch];
+            const int k = d % lbm::BATCH_TAB;
+            t.nd = k + 1;
+            t.tile0[k] = tile0;
+            r = &t.rec[k];
+        }
+        r->a = args_of(D, (Args*)nullptr);
+        r->off = D.off;
+        r->soff = D.soff;
+        r->div_nx = D.div_nx;
+        r->div_ny = D.div_ny;
+        B->tiles[launch] += n;
     }
 }
 
 // Tiles and tables of the current CTA size.  A step allocates nothing: it runs
 // inside stream captures and behind a C entry point.
-void configure(lbm_ctx* c) {
+cudaError_t configure(lbm_ctx* c) {
     BatchState* B = c->batch;
-    B->ntiles = 0;
-    for (auto& d : B->doms) {
-        d.ntiles = (uint32_t)((d.fl.box.n + B->threads - 1) / B->threads);
-        B->ntiles += d.ntiles;
-    }
     switch (c->physics) {
-        case LBM_PHYS_MHD: fill_tabs<LBM_PHYS_MHD>(B); break;
-        case LBM_PHYS_CGM: fill_tabs<LBM_PHYS_CGM>(B); break;
-        case LBM_PHYS_SC: fill_tabs<LBM_PHYS_SC>(B); break;
-        default: fill_tabs<LBM_PHYS_FLUID>(B); break;
+        case LBM_PHYS_MHD: fill_tables<LBM_PHYS_MHD>(B); break;
+        case LBM_PHYS_CGM: fill_tables<LBM_PHYS_CGM>(B); break;
+        case LBM_PHYS_SC: fill_tables<LBM_PHYS_SC>(B); break;
+        default: fill_tables<LBM_PHYS_FLUID>(B); break;
     }
+    B->ntiles = 0;
+    for (uint32_t t : B->tiles) B->ntiles += t;
     c->block_x = B->threads;  // part of the launch shape that captured graphs are kept for
+    auto& dev = B->device[B->threads / 32];
+    if (!B->many || dev.domain) return cudaSuccess;
+    void* rec = lbm_internal_dev_alloc(c, B->tabs.size());
+    uint32_t* domain = (uint32_t*)lbm_internal_dev_alloc(c, sizeof(uint32_t) * B->ntiles);
+    cudaError_t e = rec && domain ? cudaSuccess : cudaErrorMemoryAllocation;
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(rec, B->tabs.data(), B->tabs.size(), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(domain, B->domain.data(), sizeof(uint32_t) * B->ntiles, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e == cudaSuccess) {
+        dev.rec = rec;
+        dev.domain = domain;
+    } else {
+        lbm_internal_dev_free(c, rec);
+        lbm_internal_dev_free(c, domain);
+    }
+    return e;
+}
+
+template <int PHYS, typename S, typename C, bool WALLS, class Tab>
+void step_launch(lbm_ctx* c, uint32_t tiles, const Tab& tab) {
+    const S* src = (const S*)c->buf[c->cur];
+    S* dst = (S*)c->buf[c->cur ^ 1];
+    BatchState* B = c->batch;
+    if constexpr (PHYS == LBM_PHYS_SC || PHYS == LBM_PHYS_CGM)
+        lbm::batch_pass_kernel<PHYS, 0, S, C, WALLS>
+            <<<tiles, B->threads, 0, c->stream>>>(src, dst, (C*)c->phi, B->scratch_n, tab);
+    lbm::batch_pass_kernel<PHYS, 1, S, C, WALLS>
+        <<<tiles, B->threads, 0, c->stream>>>(src, dst, (C*)c->phi, B->scratch_n, tab);
 }
 
 template <int PHYS, typename S, typename C, bool WALLS>
 cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
     BatchState* B = c->batch;
-    const TabOf<PHYS>* tabs = (const TabOf<PHYS>*)B->tabs.data();
-    const std::vector<uint32_t>& tiles = B->tiles;
-    const int chunks = (int)tiles.size();
     for (long s = 0; s < n; ++s) {
-        const S* src = (const S*)c->buf[c->cur];
-        S* dst = (S*)c->buf[c->cur ^ 1];
-        for (int k = 0; k < chunks; ++k) {
-            if constexpr (PHYS == LBM_PHYS_SC || PHYS == LBM_PHYS_CGM)
-                lbm::batch_pass_kernel<PHYS, 0, S, C, WALLS><<<tiles[k], B->threads, 0, c->stream>>>(
-                    src, dst, (C*)c->phi, B->scratch_n, tabs[k]);
-            lbm::batch_pass_kernel<PHYS, 1, S, C, WALLS><<<tiles[k], B->threads, 0, c->stream>>>(
-                src, dst, (C*)c->phi, B->scratch_n, tabs[k]);
-        }
+        if (B->many)
+            step_launch<PHYS, S, C, WALLS>(
+                c, B->ntiles,
+                lbm::BatchMany<typename lbm::BatchArgs<PHYS>::T>{(const RecOf<PHYS>*)B->device[B->threads / 32].rec,
+                                                                 B->device[B->threads / 32].domain});
+        else
+            for (size_t k = 0; k < B->tiles.size(); ++k)
+                step_launch<PHYS, S, C, WALLS>(c, B->tiles[k], ((const TabOf<PHYS>*)B->tabs.data())[k]);
         if (!dry) c->cur ^= 1;
     }
     return cudaGetLastError();
@@ -318,15 +400,24 @@ cudaError_t batch_time_config(lbm_ctx* c, int threads, long steps, float* ms) {
 
 cudaError_t batch_apply_config(lbm_ctx* c, int threads) {
     if (threads < BATCH_MIN_THREADS || threads > 256 || threads % 32 != 0) return cudaErrorInvalidValue;
+    const int before = c->batch->threads;
     c->batch->threads = threads;
-    configure(c);
-    return cudaSuccess;
+    const cudaError_t e = configure(c);
+    if (e != cudaSuccess) {  // the former size's tables are there
+        c->batch->threads = before;
+        configure(c);
+    }
+    return e;
 }
 
 void batch_destroy(lbm_ctx* c) {
     BatchState* B = c->batch;
     if (!B) return;
     for (lbm_ctx* v : B->views) delete v;
+    for (auto& dev : B->device) {
+        lbm_internal_dev_free(c, dev.rec);
+        lbm_internal_dev_free(c, dev.domain);
+    }
     delete B;
     c->batch = nullptr;
 }
@@ -347,7 +438,7 @@ lbm_status lbm_batch_create(lbm_ctx** out, int ndomains, const lbm_grid* grids, 
     if ((physics == LBM_PHYS_MHD || physics == LBM_PHYS_CGM || physics == LBM_PHYS_SC) && !phys) return LBM_ERR_ARG;
     const int planes = physics == LBM_PHYS_MHD ? 40 : (physics == LBM_PHYS_CGM ? 24 : 19);
     const size_t elem = precision == LBM_FP64 ? 8 : 4;
-    size_t total = 0, max_plane = 0, cells = 0;
+    size_t total = 0, max_plane = 0, cells = 0, max_tiles = 0;
     for (int d = 0; d < ndomains; ++d) {
         const lbm_grid& g = grids[d];
         if (g.nx < 1 || g.ny < 1 || g.nz < 1) return LBM_ERR_ARG;
@@ -372,6 +463,7 @@ lbm_status lbm_batch_create(lbm_ctx** out, int ndomains, const lbm_grid* grids, 
         total += ((size_t)planes * nn + 63) / 64 * 64;  // each domain block starts 256-byte aligned
         max_plane = std::max(max_plane, (size_t)g.nx * g.ny);
         cells += nn;
+        max_tiles += (nn + lbm::BATCH_MIN_THREADS - 1) / lbm::BATCH_MIN_THREADS;
     }
     lbm_ctx* c = new (std::nothrow) lbm_ctx();
     BatchState* B = new (std::nothrow) BatchState();
@@ -399,8 +491,10 @@ lbm_status lbm_batch_create(lbm_ctx** out, int ndomains, const lbm_grid* grids, 
     try {
         B->doms.reserve(ndomains);
         B->views.reserve(ndomains);
-        B->tiles.resize(launches_per_pass(ndomains));
-        B->tabs.resize(B->tiles.size() * tab_bytes(physics));
+        B->many = batch_many(ndomains, cells, precision);
+        B->tiles.resize(B->many ? 1 : (ndomains + lbm::BATCH_TAB - 1) / lbm::BATCH_TAB);
+        B->tabs.resize(table_bytes(c));
+        if (B->many) B->domain.resize(max_tiles);
     } catch (const std::bad_alloc&) {
         st = LBM_ERR_OOM;
     }
@@ -495,7 +589,7 @@ lbm_status lbm_batch_create(lbm_ctx** out, int ndomains, const lbm_grid* grids, 
         uoff += 3 * D.fl.box.n;
         soff += D.fl.box.n;
     }
-    if (e == cudaSuccess) configure(c);
+    if (e == cudaSuccess) e = configure(c);
     // rest state for every domain
     for (int d = 0; d < ndomains && e == cudaSuccess; ++d) {
         lbm_ctx* v = B->views[d];
@@ -507,7 +601,7 @@ lbm_status lbm_batch_create(lbm_ctx** out, int ndomains, const lbm_grid* grids, 
         lbm_internal_release(c);
         delete c;
         cudaGetLastError();
-        return LBM_ERR_CUDA;
+        return e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA;
     }
     *out = c;
     return LBM_OK;
