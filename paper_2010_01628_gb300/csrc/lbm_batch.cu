@@ -136,12 +136,14 @@ template <> struct BatchArgs<LBM_PHYS_SC> { using T = ScArgs; };
 // every domain's nodes, then rho_r, each `scratch_n` values long.  WALLS: false
 // when every domain is periodic in all three directions (the node code then
 // carries no bounce-back).
-// CTAs of 256 threads per SM the FP32 passes are held to.  Unbounded, the
+// CTAs of 256 threads per SM the passes are held to.  Unbounded, the
 // parameters picked from the constant bank at a run-time index fill up to 128
-// registers (Shan-Chen sweep 19.7 GLUPS, 27.4 at these bounds; colour gradient
-// 14.4, 15.2 at 4 and 16.0 at 5 CTAs).
+// registers (FP32 Shan-Chen sweep 19.7 GLUPS, 27.4 at these bounds; colour gradient
+// 14.4, 15.2 at 4 and 16.0 at 5 CTAs).  In FP64 MHD (136 registers) and the colour
+// gradient (156) left one CTA per SM, whose start and end nothing covered: 64 x 64^3
+// 12.2 -> 11.6 ms and 19.1 -> 18.5 ms a step at two.
 constexpr int batch_ctas(int phys, int pass, size_t elem) {
-    if (elem != 4) return 1;
+    if (elem != 4) return phys == LBM_PHYS_MHD || phys == LBM_PHYS_CGM ? 2 : 1;
     if (phys == LBM_PHYS_MHD) return 4;
     if (phys == LBM_PHYS_SC) return pass == 0 ? 6 : 5;
     if (phys == LBM_PHYS_CGM) return 5;
