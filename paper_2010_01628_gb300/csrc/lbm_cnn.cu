@@ -278,7 +278,10 @@ __global__ void __launch_bounds__(192, ConvLayout<CI, CO>::CTAS) conv_tc(const _
     // cells stay as zeroed here; only rows outside the grid are written over.
     const bool fixed_halo = g.ntx == 1;
     if (fixed_halo) {
-        for (int i = threadIdx.x; i < NSLOT * Lay::SLOT_BYTES / 16; i += blockDim.x)
+        // the slots this CTA will stage: one per tile and two more per run
+        const int runs = t_begin < t_end ? (t_end - 1) / g.ny - t_begin / g.ny + 1 : 0;
+        const int slots = min(NSLOT, t_end - t_begin + 2 * runs);
+        for (int i = threadIdx.x; i < slots * Lay::SLOT_BYTES / 16; i += blockDim.x)
             reinterpret_cast<uint4*>(sA)[i] = make_uint4(0u, 0u, 0u, 0u);
         lbm::fence_proxy_async();
     }
