@@ -243,10 +243,12 @@ lbm_status lbm_mbarrier_selftest(double timeout_s, int arrive, int *observed);
 
 /* ---- Autotuner ---------------------------------------------------------------
  * Chooses the launch shape of a context by timed trials that leave its state
- * unchanged: threads per block of the single-domain or batched step kernels.  Results are cached
- * in a JSON file (cache_path, may be NULL = no cache) keyed by device, physics,
- * precision and geometry; a cached entry is applied without timing unless
- * force != 0.  Reports the chosen throughput in MLUPS (may be NULL). */
+ * unchanged, steps replayed from a captured graph as in long calls: variant and
+ * threads per block of the single-domain step kernels, threads of the batched
+ * ones.  Results are cached in a JSON file (cache_path, may be NULL = no cache)
+ * keyed by device, physics, precision, geometry and a revision of the kernels and
+ * their timing; a cached entry is applied without timing unless force != 0.
+ * Reports the chosen throughput in MLUPS (may be NULL). */
 lbm_status lbm_autotune(lbm_ctx *ctx, const char *cache_path, int force, double *mlups);
 
 /* Set the launch shape of a single-domain context by hand (what lbm_autotune

@@ -382,24 +382,6 @@ cudaError_t batch_step(lbm_ctx* c, long n, bool dry) {
     }
 }
 
-// Timed dry run (state unchanged) for the autotuner.
-cudaError_t batch_time_config(lbm_ctx* c, int threads, long steps, float* ms) {
-    cudaError_t e = batch_apply_config(c, threads);
-    if (e != cudaSuccess) return e;
-    cudaEvent_t a, b;
-    cudaEventCreate(&a);
-    cudaEventCreate(&b);
-    e = batch_step(c, 2, true);  // warm-up
-    if (e == cudaSuccess) e = cudaEventRecord(a, c->stream);
-    if (e == cudaSuccess) e = batch_step(c, steps, true);
-    if (e == cudaSuccess) e = cudaEventRecord(b, c->stream);
-    if (e == cudaSuccess) e = cudaEventSynchronize(b);
-    if (e == cudaSuccess) e = cudaEventElapsedTime(ms, a, b);
-    cudaEventDestroy(a);
-    cudaEventDestroy(b);
-    return e;
-}
-
 cudaError_t batch_apply_config(lbm_ctx* c, int threads) {
     if (threads < BATCH_MIN_THREADS || threads > 256 || threads % 32 != 0) return cudaErrorInvalidValue;
     const int before = c->batch->threads;

@@ -139,7 +139,6 @@ cudaError_t reduce_finalize(lbm_ctx* c);
 // Batched step (lbm_batch.cu): CTAs of BATCH_MIN_THREADS to 256 threads.
 constexpr int BATCH_MIN_THREADS = 128;
 cudaError_t batch_step(lbm_ctx* c, long n, bool dry = false);
-cudaError_t batch_time_config(lbm_ctx* c, int threads, long steps, float* ms);
 cudaError_t batch_apply_config(lbm_ctx* c, int threads);
 void batch_destroy(lbm_ctx* c);
 

@@ -115,16 +115,20 @@ const char* prec_name(lbm_precision p) {
     return p == LBM_FP64 ? "fp64" : (p == LBM_FP32 ? "fp32" : (p == LBM_FP16_SHIFTED ? "fp16" : "bf16"));
 }
 
+// Revision of the step kernels and of the way they are timed: entries of another
+// one are left alone and not applied.
+const char TUNE_REVISION[] = "graph-1";
+
 std::string cache_key(const lbm_ctx* c, const std::vector<long>& domain_sizes) {
     cudaDeviceProp prop;
     std::string dev = "gpu";
     if (cudaGetDeviceProperties(&prop, c->device) == cudaSuccess) dev = prop.name;
     char buf[256];
     if (!c->batch) {
-        std::snprintf(buf, sizeof(buf), "%s|%s|%s|%dx%dx%d|p%u%s%s%s", dev.c_str(), phys_name(c->physics),
+        std::snprintf(buf, sizeof(buf), "%s|%s|%s|%dx%dx%d|p%u%s%s%s|%s", dev.c_str(), phys_name(c->physics),
                       prec_name(c->prec), c->box.nx, c->box.ny, c->box.nz, c->box.periodic,
                       c->grid.wall_model == LBM_WALL_REGULARIZED ? "|reg" : "",
-                      c->relax.moment_space == LBM_MOMENTS_RAW ? "|rm" : "", c->q == 27 ? "|q27" : "");
+                      c->relax.moment_space == LBM_MOMENTS_RAW ? "|rm" : "", c->q == 27 ? "|q27" : "", TUNE_REVISION);
         return buf;
     }
     unsigned long long h = 1469598103934665603ull;  // FNV-1a over the domain sizes
@@ -132,25 +136,52 @@ std::string cache_key(const lbm_ctx* c, const std::vector<long>& domain_sizes) {
         h ^= (unsigned long long)v;
         h *= 1099511628211ull;
     }
-    std::snprintf(buf, sizeof(buf), "%s|%s|%s|batch%zu|h%016llx", dev.c_str(), phys_name(c->physics),
-                  prec_name(c->prec), domain_sizes.size(), h);
+    std::snprintf(buf, sizeof(buf), "%s|%s|%s|batch%zu|h%016llx|%s", dev.c_str(), phys_name(c->physics),
+                  prec_name(c->prec), domain_sizes.size(), h, TUNE_REVISION);
     return buf;
 }
 
-float time_dry_steps(lbm_ctx* c, long reps, cudaError_t* err) {
+// Milliseconds per dry step over about `reps` of them: replays of a captured
+// graph, or plain launches where it cannot be made.
+double time_dry_steps(lbm_ctx* c, long reps, cudaError_t* err) {
+    const long steps = reps < lbm::STEP_GRAPH[0] ? reps : lbm::STEP_GRAPH[0];
+    const long replays = reps / steps;
+    cudaGraphExec_t exec = nullptr;
+    if (reps > 1) {
+        const cudaStream_t user = c->stream;
+        c->stream = c->copy_stream;
+        exec = lbm::capture_graph(c->copy_stream, [&] { return lbm_internal_step(c, steps, true); });
+        c->stream = user;
+    }
     cudaEvent_t a, b;
     cudaEventCreate(&a);
     cudaEventCreate(&b);
     float ms = -1.f;
-    cudaError_t e = cudaEventRecord(a, c->stream);
-    if (e == cudaSuccess) e = lbm_internal_step(c, reps, true);
+    cudaError_t e = exec ? cudaGraphUpload(exec, c->stream) : cudaSuccess;
+    if (e == cudaSuccess) e = cudaEventRecord(a, c->stream);
+    for (long r = 0; r < replays && e == cudaSuccess; ++r)
+        e = exec ? cudaGraphLaunch(exec, c->stream) : lbm_internal_step(c, steps, true);
     if (e == cudaSuccess) e = cudaEventRecord(b, c->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(b);
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
     cudaEventDestroy(a);
     cudaEventDestroy(b);
+    if (exec) {
+        cudaStreamSynchronize(c->stream);
+        cudaGraphExecDestroy(exec);
+    }
     *err = e;
-    return ms;
+    return ms / (double)(replays * steps);
+}
+
+// Milliseconds per step at the current launch shape.
+double time_shape(lbm_ctx* c, cudaError_t* err) {
+    const double one = time_dry_steps(c, 1, err);  // warm-up and size estimate
+    if (*err != cudaSuccess) return one;
+    long reps = one > 0.0 ? (long)(30.0 / one) : 10;
+    if (reps < 3) reps = 3;
+    if (reps > 200) reps = 200;
+    return time_dry_steps(c, reps, err);
 }
 
 }  // namespace
@@ -214,12 +245,12 @@ extern "C" lbm_status lbm_autotune(lbm_ctx* c, const char* cache_path, int force
     const double cells = (double)c->box.n;
 
     auto hit = cache.find(key);
-    if (!force && hit != cache.end() && hit->second.count("threads")) {
+    // an entry that this batch cannot take is timed again
+    if (!force && hit != cache.end() && hit->second.count("threads") &&
+        (!c->batch || lbm::batch_apply_config(c, (int)hit->second["threads"]) == cudaSuccess)) {
         Entry& h = hit->second;
         const int threads = (int)h["threads"];
-        if (c->batch) {
-            if (lbm::batch_apply_config(c, threads) != cudaSuccess) return LBM_ERR_CUDA;
-        } else {
+        if (!c->batch) {
             const int variant = h.count("variant") ? (int)h["variant"] : 0;
             const int stages = h.count("stages") ? (int)h["stages"] : 0;
             const int ctas = h.count("ctas") ? (int)h["ctas"] : 1;
@@ -246,23 +277,21 @@ extern "C" lbm_status lbm_autotune(lbm_ctx* c, const char* cache_path, int force
     Entry best;
     double best_ms = 1e30;
     if (c->batch) {
-        const long steps = 6;
-        const int threads_c[] = {128, 256};
-        for (int th : threads_c) {
-            float ms = 0.f;
-            e = lbm::batch_time_config(c, th, steps, &ms);
+        const int saved = c->block_x;
+        for (int th : {128, 256}) {
+            e = lbm::batch_apply_config(c, th);
+            const double per = e == cudaSuccess ? time_shape(c, &e) : 0.0;
             if (e != cudaSuccess) {
                 cudaGetLastError();
                 continue;
             }
-            const double per = ms / steps;
             if (per < best_ms) {
                 best_ms = per;
                 best = Entry{{"threads", (double)th}};
             }
         }
+        lbm::batch_apply_config(c, best.empty() ? saved : (int)best["threads"]);
         if (best.empty()) return LBM_ERR_CUDA;
-        if (lbm::batch_apply_config(c, (int)best["threads"]) != cudaSuccess) return LBM_ERR_CUDA;
     } else {
         struct Cand {
             int variant, threads, stages, ctas;
@@ -295,20 +324,11 @@ extern "C" lbm_status lbm_autotune(lbm_ctx* c, const char* cache_path, int force
             }
             c->tma_stages = k.variant == 1 && k.stages > 0 ? k.stages : saved_st;
             c->tma_ctas = k.ctas;
-            float one = time_dry_steps(c, 1, &e);  // warm-up and size estimate
+            const double per = time_shape(c, &e);
             if (e != cudaSuccess) {
                 cudaGetLastError();
                 continue;
             }
-            long reps = one > 0.f ? (long)(30.0f / one) : 10;
-            if (reps < 3) reps = 3;
-            if (reps > 200) reps = 200;
-            const float ms = time_dry_steps(c, reps, &e);
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                continue;
-            }
-            const double per = ms / reps;
             if (per < best_ms) {
                 best_ms = per;
                 best = Entry{{"variant", (double)k.variant},
