@@ -206,7 +206,7 @@ lbm_status lbm_set_populations(lbm_ctx *ctx, const void *src, size_t bytes);
  * density ratio, surface tension) advanced together: a step is one launch over
  * the nodes of all domains (two for the two-phase modules: order parameter or
  * pseudopotential, then collision; more for over 128 large domains), and 16
- * steps at a time are replayed from a captured CUDA graph.  Physics:
+ * steps at a time are replayed from a CUDA graph.  Physics:
  * LBM_PHYS_FLUID, LBM_PHYS_MHD, LBM_PHYS_CGM (App. E colour gradient) or
  * LBM_PHYS_SC (Sec. III.G Shan-Chen), whose batch holds the phi and rho_r (psi)
  * planes for all domains; FP64 or FP32.  grids/relax/forcing/phys are arrays of
@@ -224,7 +224,7 @@ lbm_status lbm_batch_create(lbm_ctx **out, int ndomains, const lbm_grid *grids, 
 lbm_status lbm_batch_domain(lbm_ctx *batch, int domain, lbm_ctx **view);
 lbm_status lbm_batch_step(lbm_ctx *batch, long n);
 /* Launch shape of a step: threads per CTA, CTAs, whether calls of 16 and more
- * steps may be replayed from captured graphs (0 once one could not be made at
+ * steps may be replayed from graphs (0 once one could not be made at
  * this shape: steps are then launched one by one), number of tiles (one CTA
  * each). */
 lbm_status lbm_batch_info(const lbm_ctx *batch, int *threads, int *grid, int *graph, long *tiles);
@@ -243,7 +243,7 @@ lbm_status lbm_mbarrier_selftest(double timeout_s, int arrive, int *observed);
 
 /* ---- Autotuner ---------------------------------------------------------------
  * Chooses the launch shape of a context by timed trials that leave its state
- * unchanged, steps replayed from a captured graph as in long calls: variant and
+ * unchanged, steps replayed from a graph as in long calls: variant and
  * threads per block of the single-domain step kernels, threads of the batched
  * ones.  Results are cached in a JSON file (cache_path, may be NULL = no cache)
  * keyed by device, physics, precision, geometry and a revision of the kernels and

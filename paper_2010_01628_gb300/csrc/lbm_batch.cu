@@ -1,6 +1,6 @@
 // lbm_batch.cu -- batched parameter sweeps: many independent domains of
 // uneven sizes advanced together, one launch per pass of a step over the nodes
-// of all of them (lbm_step replays 16 steps per captured graph).
+// of all of them (lbm_step replays 16 steps per graph).
 //
 // Work decomposition: every domain is cut into tiles of `threads` consecutive
 // nodes (x fastest), one CTA per tile.  The first tiles and the parameters (size,
@@ -299,7 +299,7 @@ void fill_tables(BatchState* B) {
 }
 
 // Tiles and tables of the current CTA size.  A step allocates nothing: it runs
-// inside stream captures and behind a C entry point.
+// behind a C entry point.
 cudaError_t configure(lbm_ctx* c) {
     BatchState* B = c->batch;
     switch (c->physics) {
@@ -310,7 +310,7 @@ cudaError_t configure(lbm_ctx* c) {
     }
     B->ntiles = 0;
     for (uint32_t t : B->tiles) B->ntiles += t;
-    c->block_x = B->threads;  // part of the launch shape that captured graphs are kept for
+    c->block_x = B->threads;  // part of the launch shape that graphs are kept for
     auto& dev = B->device[B->threads / 32];
     if (!B->many || dev.domain) return cudaSuccess;
     void* rec = lbm_internal_dev_alloc(c, B->tabs.size());
@@ -337,10 +337,10 @@ void step_launch(lbm_ctx* c, uint32_t tiles, const Tab& tab) {
     S* dst = (S*)c->buf[c->cur ^ 1];
     BatchState* B = c->batch;
     if constexpr (PHYS == LBM_PHYS_SC || PHYS == LBM_PHYS_CGM)
-        lbm::batch_pass_kernel<PHYS, 0, S, C, WALLS>
-            <<<tiles, B->threads, 0, c->stream>>>(src, dst, (C*)c->phi, B->scratch_n, tab);
-    lbm::batch_pass_kernel<PHYS, 1, S, C, WALLS>
-        <<<tiles, B->threads, 0, c->stream>>>(src, dst, (C*)c->phi, B->scratch_n, tab);
+        launch_step(c, lbm::batch_pass_kernel<PHYS, 0, S, C, WALLS, Tab>, tiles, B->threads, 0, src, dst, (C*)c->phi,
+                    B->scratch_n, tab);
+    launch_step(c, lbm::batch_pass_kernel<PHYS, 1, S, C, WALLS, Tab>, tiles, B->threads, 0, src, dst, (C*)c->phi,
+                B->scratch_n, tab);
 }
 
 template <int PHYS, typename S, typename C, bool WALLS>

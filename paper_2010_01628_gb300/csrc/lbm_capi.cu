@@ -111,7 +111,7 @@ cudaError_t phys_reduce(lbm_ctx* c, bool record) {
 // n steps on the context stream (lbm_step_graphs.h).
 cudaError_t run_steps(lbm_ctx* c, long n) {
     const int shape[6] = {c->variant, c->block_x, c->tma_stages, c->tma_ctas, c->zchunk, c->fused_threads};
-    return lbm::run_steps(c->graphs, shape, c->stream, c->copy_stream, c->cur, n,
+    return lbm::run_steps(c->graphs, shape, c->stream, c->record, c->cur, n,
                           [c](long steps) { return phys_step(c, steps); });
 }
 

@@ -218,8 +218,8 @@ static cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
         const S* src = (const S*)c->buf[c->cur];
         S* dst = (S*)c->buf[c->cur ^ 1];
         // (with y-only predicates the first pass's loads are scheduled worse: 64.7 instead of 51.4 us at 128^3)
-        cgm_phi_kernel<S, C, WALLS != 0, FLAT><<<grid, bx, 0, c->stream>>>(src, phi, rho_red, p, div_nx);
-        cgm_collide_kernel<S, C, WALLS, FLAT><<<grid, bx, 0, c->stream>>>(src, dst, phi, rho_red, p, div_nx);
+        launch_step(c, cgm_phi_kernel<S, C, WALLS != 0, FLAT>, grid, bx, 0, src, phi, rho_red, p, div_nx);
+        launch_step(c, cgm_collide_kernel<S, C, WALLS, FLAT>, grid, bx, 0, src, dst, phi, rho_red, p, div_nx);
         if (!dry) c->cur ^= 1;
     }
     return cudaGetLastError();

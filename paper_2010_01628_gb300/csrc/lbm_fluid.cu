@@ -575,7 +575,7 @@ static cudaError_t launch_tma(lbm_ctx* c, const S* src, S* dst, const FluidArgs&
     int block = ((c->box.nx + 31) / 32) * 32;
     if (block > 256) block = 256;
     c->bounded_waits = true;
-    fluid_step_tma_kernel<S, C, WALLS><<<(unsigned)grid, block, smem, c->stream>>>(src, dst, p, stages, c->status);
+    launch_step(c, fluid_step_tma_kernel<S, C, WALLS>, (unsigned)grid, block, smem, src, dst, p, stages, c->status);
     return cudaSuccess;
 }
 
@@ -584,13 +584,13 @@ static void step_direct(lbm_ctx* c, dim3 grid, bool walls, bool flat, const S* s
     const int bx = c->block_x;
     const FastDiv div_nx = make_fast_div((uint32_t)c->box.nx);
     if (walls && flat)
-        fluid_step_kernel<S, C, true, true, RM, UNFORCED><<<grid, bx, 0, c->stream>>>(src, dst, p, div_nx);
+        launch_step(c, fluid_step_kernel<S, C, true, true, RM, UNFORCED>, grid, bx, 0, src, dst, p, div_nx);
     else if (walls)
-        fluid_step_kernel<S, C, true, false, RM, UNFORCED><<<grid, bx, 0, c->stream>>>(src, dst, p, div_nx);
+        launch_step(c, fluid_step_kernel<S, C, true, false, RM, UNFORCED>, grid, bx, 0, src, dst, p, div_nx);
     else if (flat)
-        fluid_step_kernel<S, C, false, true, RM, UNFORCED><<<grid, bx, 0, c->stream>>>(src, dst, p, div_nx);
+        launch_step(c, fluid_step_kernel<S, C, false, true, RM, UNFORCED>, grid, bx, 0, src, dst, p, div_nx);
     else
-        fluid_step_kernel<S, C, false, false, RM, UNFORCED><<<grid, bx, 0, c->stream>>>(src, dst, p, div_nx);
+        launch_step(c, fluid_step_kernel<S, C, false, false, RM, UNFORCED>, grid, bx, 0, src, dst, p, div_nx);
 }
 
 template <typename S, typename C>
@@ -625,11 +625,14 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
             S* dst = (S*)c->buf[c->cur ^ 1];
             const FastDiv div_nx = make_fast_div((uint32_t)c->box.nx);
             if (reg)
-                flat ? fluid_step_channel_kernel<S, C, true, true><<<g, bx, 0, c->stream>>>(src, dst, p, div_nx, inner)
-                     : fluid_step_channel_kernel<S, C, false, true><<<g, bx, 0, c->stream>>>(src, dst, p, div_nx, 0);
+                flat ? launch_step(c, fluid_step_channel_kernel<S, C, true, true>,
+                                   g, bx, 0, src, dst, p, div_nx, inner)
+                     : launch_step(c, fluid_step_channel_kernel<S, C, false, true>, g, bx, 0, src, dst, p, div_nx, 0);
             else
-                flat ? fluid_step_channel_kernel<S, C, true, false><<<g, bx, 0, c->stream>>>(src, dst, p, div_nx, inner)
-                     : fluid_step_channel_kernel<S, C, false, false><<<g, bx, 0, c->stream>>>(src, dst, p, div_nx, 0);
+                flat ? launch_step(c, fluid_step_channel_kernel<S, C, true, false>,
+                                   g, bx, 0, src, dst, p, div_nx, inner)
+                     : launch_step(c, fluid_step_channel_kernel<S, C, false, false>,
+                                   g, bx, 0, src, dst, p, div_nx, 0);
             if (!dry) c->cur ^= 1;
         }
         return cudaGetLastError();
@@ -655,21 +658,21 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
         if constexpr (is16<S>()) {
             if (zpair) {
                 if (walls && flat)
-                    fluid_step_zpair_kernel<S, true, true><<<gridz, bx, 0, c->stream>>>(src, dst, p, div_nx);
+                    launch_step(c, fluid_step_zpair_kernel<S, true, true>, gridz, bx, 0, src, dst, p, div_nx);
                 else if (walls)
-                    fluid_step_zpair_kernel<S, true, false><<<gridz, bx, 0, c->stream>>>(src, dst, p, div_nx);
+                    launch_step(c, fluid_step_zpair_kernel<S, true, false>, gridz, bx, 0, src, dst, p, div_nx);
                 else if (flat)
-                    fluid_step_zpair_kernel<S, false, true><<<gridz, bx, 0, c->stream>>>(src, dst, p, div_nx);
+                    launch_step(c, fluid_step_zpair_kernel<S, false, true>, gridz, bx, 0, src, dst, p, div_nx);
                 else
-                    fluid_step_zpair_kernel<S, false, false><<<gridz, bx, 0, c->stream>>>(src, dst, p, div_nx);
+                    launch_step(c, fluid_step_zpair_kernel<S, false, false>, gridz, bx, 0, src, dst, p, div_nx);
                 if (!dry) c->cur ^= 1;
                 continue;
             }
             if (pair) {
                 if (walls)
-                    fluid_step_pair_kernel<S, true><<<grid2, bx, 0, c->stream>>>(src, dst, p);
+                    launch_step(c, fluid_step_pair_kernel<S, true>, grid2, bx, 0, src, dst, p);
                 else
-                    fluid_step_pair_kernel<S, false><<<grid2, bx, 0, c->stream>>>(src, dst, p);
+                    launch_step(c, fluid_step_pair_kernel<S, false>, grid2, bx, 0, src, dst, p);
                 if (!dry) c->cur ^= 1;
                 continue;
             }

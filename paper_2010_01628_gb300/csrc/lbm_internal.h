@@ -52,6 +52,7 @@ struct lbm_ctx {
     int* status = nullptr;  // device status word written by bounded waits
     bool bounded_waits = false;  // a kernel that may write `status` has been launched
     lbm::StepGraphs graphs;
+    lbm::GraphRecord* record = nullptr;  // a graph of steps is being made
     std::string err;
     bool owns = true;            // false for the per-domain views of a batch
     lbm_ctx* parent = nullptr;   // the batch a view belongs to
@@ -92,6 +93,31 @@ struct FieldsOut {
     double* phase = nullptr;
     double* B[3] = {nullptr, nullptr, nullptr};
 };
+
+// A kernel of a step, launched on the context's stream or added to the graph that
+// is being made.  Parameters are taken by reference (a batch's tables are 32 KB).
+template <class T>
+struct Param {
+    using type = T;
+};
+template <class... P>
+void launch_step(lbm_ctx* c, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                 const typename Param<P>::type&... params) {
+    void* args[] = {const_cast<void*>(static_cast<const void*>(&params))...};
+    if (!c->record) {
+        cudaLaunchKernel((const void*)kernel, grid, block, args, smem, c->stream);  // read by cudaGetLastError
+        return;
+    }
+    cudaKernelNodeParams node = {};
+    node.func = (void*)kernel;
+    node.gridDim = grid;
+    node.blockDim = block;
+    node.sharedMemBytes = (unsigned)smem;
+    node.kernelParams = args;
+    cudaGraphNode_t added;
+    if (cudaGraphAddKernelNode(&added, c->record->graph, &c->record->last, c->record->last ? 1 : 0, &node) == cudaSuccess)
+        c->record->last = added;
+}
 
 // Kernel launchers, one per physics module; each returns cudaGetLastError().
 // A "dry" step reads the current state and writes the other buffer without

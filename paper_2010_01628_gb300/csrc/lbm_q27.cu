@@ -461,9 +461,8 @@ static cudaError_t steps_t(lbm_ctx* c, long n, bool dry) {
     const int bx = c->block_x;
     const dim3 grid = step_grid(c->box, bx, c->box.ny, FLAT);
     for (long s = 0; s < n; ++s) {
-        step_kernel<S, C, WALLS, RM, FLAT>
-            <<<grid, bx, 0, c->stream>>>((const S*)c->buf[c->cur], (S*)c->buf[c->cur ^ 1], p,
-                                         make_fast_div((uint32_t)c->box.nx));
+        launch_step(c, step_kernel<S, C, WALLS, RM, FLAT>, grid, bx, 0, (const S*)c->buf[c->cur],
+                    (S*)c->buf[c->cur ^ 1], p, make_fast_div((uint32_t)c->box.nx));
         if (!dry) c->cur ^= 1;
     }
     return cudaGetLastError();

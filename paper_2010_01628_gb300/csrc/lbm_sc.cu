@@ -229,8 +229,8 @@ static ScArgs sc_args(const lbm_ctx* c) {
 
 template <typename S, typename C, bool WALLS, bool FLAT>
 static void launch_psi(lbm_ctx* c, const S* src, const ScArgs& p) {
-    sc_psi_kernel<S, C, WALLS, FLAT>
-        <<<step_grid(c->box, c->block_x, c->box.ny, FLAT), c->block_x, 0, c->stream>>>(src, (C*)c->phi, p, make_fast_div((uint32_t)c->box.nx));
+    launch_step(c, sc_psi_kernel<S, C, WALLS, FLAT>, step_grid(c->box, c->block_x, c->box.ny, FLAT), c->block_x, 0, src,
+                (C*)c->phi, p, make_fast_div((uint32_t)c->box.nx));
 }
 template <typename S>
 static bool sc_flat(const lbm_ctx* c) {
@@ -246,8 +246,8 @@ static void launch_psi(lbm_ctx* c, const S* src, const ScArgs& p) {
 }
 template <typename S, typename C, bool WALLS, bool FLAT>
 static void launch_collide(lbm_ctx* c, const S* src, S* dst, const ScArgs& p) {
-    sc_collide_kernel<S, C, WALLS, FLAT><<<step_grid(c->box, c->block_x, c->box.ny, FLAT), c->block_x, 0, c->stream>>>(
-        src, dst, (const C*)c->phi, p, make_fast_div((uint32_t)c->box.nx));
+    launch_step(c, sc_collide_kernel<S, C, WALLS, FLAT>, step_grid(c->box, c->block_x, c->box.ny, FLAT), c->block_x, 0,
+                src, dst, (const C*)c->phi, p, make_fast_div((uint32_t)c->box.nx));
 }
 
 template <typename S, typename C, bool WALLS, int BY>
@@ -255,7 +255,7 @@ static void launch_fused(lbm_ctx* c, const S* src, S* dst, const ScArgs& p) {
     const int lz = c->zchunk > 0 ? c->zchunk : 32;
     const dim3 grid((unsigned)((c->box.nx + 29) / 30), (unsigned)((c->box.ny + BY - 3) / (BY - 2)),
                     (unsigned)((c->box.nz + lz - 1) / lz));
-    sc_fused_kernel<S, C, WALLS, BY><<<grid, dim3(32, BY), 0, c->stream>>>(src, dst, p, lz);
+    launch_step(c, sc_fused_kernel<S, C, WALLS, BY>, grid, dim3(32, BY), 0, src, dst, p, lz);
 }
 
 template <typename S, typename C>

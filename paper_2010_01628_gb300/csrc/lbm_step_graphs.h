@@ -1,4 +1,4 @@
-// lbm_step_graphs.h -- steps replayed from captured graphs: when a graph is
+// lbm_step_graphs.h -- steps replayed from graphs: when a graph is
 // made, which steps of a call replay it, and what follows a failure.  Host code
 // of the CUDA runtime only.
 #pragma once
@@ -9,17 +9,17 @@
 
 namespace lbm {
 
-// Steps of one captured graph (even, so that a replay leaves buf[cur] current).
+// Steps of one graph (even, so that a replay leaves buf[cur] current).
 // On this GPU a kernel that follows another in a stream starts 2.4 us later
 // than the same kernel as the next node of a graph (chains of small dependent
 // kernels: 4.1 us each in a stream, 1.8 us in a graph; at 1 M nodes 24.7 and
 // 22.3 us), so steps are replayed 16 at a time and the rest of a call 4 at a time.
 // More steps per graph gain nothing (the stream's gap between two graphs is
-// 0.15 us a step at 16) and make the capture, paid once per context and launch
-// shape, longer.  Calls of fewer than 16 steps are launched step by step.
+// 0.15 us a step at 16) and make the graph, paid once per context and launch
+// shape, longer to build.  Calls of fewer than 16 steps are launched step by step.
 constexpr long STEP_GRAPH[2] = {16, 4};
 // A graph is made once the steps it could have replayed, those of the present
-// call among them, reach these counts: its capture and instantiation cost what it
+// call among them, reach these counts: making it costs what it
 // saves over about as many steps (16 steps of one launch: 60 us against 2.3 us a
 // step; Shan-Chen, two launches: 90 against 4.4; a batch, with up to 32 KB of
 // parameters a launch: 185 against 5.8).  A context that is stepped little then
@@ -50,23 +50,32 @@ struct StepGraphs {
     }
 };
 
-// Captures what `launch(capture)` enqueues on `capture` (an idle stream of the
-// context's own); nullptr if it cannot be made into a graph.
+// A graph being made of the kernels that launch_step would launch, a chain.  It
+// is built node by node and not by capturing a stream: while any stream of the
+// context is captured CUDA refuses device-wide synchronisations, those of the
+// program's other threads too.
+struct GraphRecord {
+    cudaGraph_t graph = nullptr;
+    cudaGraphNode_t last = nullptr;
+};
+
+// The graph of what `launch()` launches through launch_step while `record`
+// points to it; nullptr if it cannot be made.
 template <class Launch>
-cudaGraphExec_t capture_graph(cudaStream_t capture, Launch launch) {
-    // relaxed: neither disturbs nor is disturbed by a capture on another thread
+cudaGraphExec_t record_graph(GraphRecord*& record, Launch launch) {
+    // relaxed: not disturbed by a capture on another thread
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaThreadExchangeStreamCaptureMode(&mode);
     cudaGraphExec_t exec = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(capture, cudaStreamCaptureModeRelaxed);
+    GraphRecord r;
+    cudaError_t e = cudaGraphCreate(&r.graph, 0);
     if (e == cudaSuccess) {
-        cudaGraph_t g = nullptr;
-        const cudaError_t el = launch();
-        e = cudaStreamEndCapture(capture, &g);
-        if (e == cudaSuccess) e = el;
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
-        if (g) cudaGraphDestroy(g);
+        record = &r;
+        e = launch();
+        record = nullptr;
     }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, r.graph, 0);
+    if (r.graph) cudaGraphDestroy(r.graph);
     if (e != cudaSuccess) {
         cudaGetLastError();
         exec = nullptr;
@@ -76,11 +85,11 @@ cudaGraphExec_t capture_graph(cudaStream_t capture, Launch launch) {
 }
 
 // n steps on `stream`: whole graphs, then single launches.  `launch(n)` enqueues
-// n steps on `stream` as it then is and flips `cur` once per step; graphs are
-// captured on `capture`.  While the caller is capturing the stream every step is
-// a plain launch, which the capture records.
+// n steps on `stream`, or adds them to the graph at `record`, and flips `cur` once
+// per step.  While the caller is capturing the stream every step is a plain
+// launch, which the capture records.
 template <class Launch>
-cudaError_t run_steps(StepGraphs& g, const int (&shape)[6], cudaStream_t& stream, cudaStream_t capture, int& cur,
+cudaError_t run_steps(StepGraphs& g, const int (&shape)[6], cudaStream_t stream, GraphRecord*& record, int& cur,
                       long n, Launch launch) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     bool replay = n >= STEP_GRAPH[0];
@@ -99,10 +108,7 @@ cudaError_t run_steps(StepGraphs& g, const int (&shape)[6], cudaStream_t& stream
         if (!exec && steps > 0) {
             g.missed[size][k] += steps;
             if (g.missed[size][k] < STEP_GRAPH_AFTER[size]) continue;
-            const cudaStream_t user = stream;
-            stream = capture;
-            exec = capture_graph(capture, [&] { return launch(STEP_GRAPH[size]); });
-            stream = user;
+            exec = record_graph(record, [&] { return launch(STEP_GRAPH[size]); });
             cur = k;
             g.failed = !exec;
         }

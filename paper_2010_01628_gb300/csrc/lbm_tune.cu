@@ -2,9 +2,13 @@
 //
 // Candidates are timed with CUDA events on the context stream in "dry" runs
 // that read the current state and write the other buffer without making it
-// current, so tuning never advances or alters the simulation.  The winner is
-// applied to the context and cached in a small JSON file:
-//   { "<device>|<physics>|<precision>|<geometry>": {"threads": 256, ...}, ... }
+// current, so tuning never advances or alters the simulation.  They are timed as
+// lbm_step runs long calls, replayed from a graph: launched singly, a candidate
+// of two launches a step pays the stream's longer launch interval twice (100^3
+// Shan-Chen: the fused kernel was taken, 21.8 GLUPS, where the two passes replay
+// at 25.6), and all candidates of a small box time alike.  The winner is applied
+// to the context and cached in a small JSON file:
+//   { "<device>|<physics>|<precision>|<geometry>|<revision>": {"threads": 256, ...}, ... }
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -141,18 +145,13 @@ std::string cache_key(const lbm_ctx* c, const std::vector<long>& domain_sizes) {
     return buf;
 }
 
-// Milliseconds per dry step over about `reps` of them: replays of a captured
-// graph, or plain launches where it cannot be made.
+// Milliseconds per dry step over about `reps` of them: replays of a graph, or
+// plain launches where it cannot be made.
 double time_dry_steps(lbm_ctx* c, long reps, cudaError_t* err) {
     const long steps = reps < lbm::STEP_GRAPH[0] ? reps : lbm::STEP_GRAPH[0];
     const long replays = reps / steps;
     cudaGraphExec_t exec = nullptr;
-    if (reps > 1) {
-        const cudaStream_t user = c->stream;
-        c->stream = c->copy_stream;
-        exec = lbm::capture_graph(c->copy_stream, [&] { return lbm_internal_step(c, steps, true); });
-        c->stream = user;
-    }
+    if (reps > 1) exec = lbm::record_graph(c->record, [&] { return lbm_internal_step(c, steps, true); });
     cudaEvent_t a, b;
     cudaEventCreate(&a);
     cudaEventCreate(&b);

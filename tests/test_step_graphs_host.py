@@ -1,4 +1,4 @@
-"""When steps are replayed from captured graphs, and what follows a failed capture, instantiation or replay: the host
+"""When steps are replayed from graphs, and what follows a graph that cannot be made, instantiated or replayed: the host
 code of lbm_step_graphs.h against a fake of the CUDA runtime that records its calls and fails the wanted one."""
 import os
 import shutil
@@ -20,25 +20,17 @@ static cudaError_t call(const char* what) {
     auto f = fail.find(what);
     return f != fail.end() && (f->second < 0 || f->second == k) ? cudaErrorMemoryAllocation : cudaSuccess;
 }
-static bool capturing = false, user_capture = false;
+static bool user_capture = false;
 static long recorded = 0, ran_plain = 0, ran_graph = 0;
-static cudaStream_t U = (cudaStream_t)16, K = (cudaStream_t)32;
+static cudaStream_t U = (cudaStream_t)16;
 extern "C" {
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return call("sync"); }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return call("destroy"); }
 cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode*) { return cudaSuccess; }
-cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode) {
-    const cudaError_t e = call("begin");
-    capturing = e == cudaSuccess;
+cudaError_t cudaGraphCreate(cudaGraph_t* g, unsigned) {
     recorded = 0;
-    if (s != K) abort();
-    return e;
-}
-cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t* g) {
-    if (!capturing || s != K) abort();
-    capturing = false;
     *g = (cudaGraph_t)8;
-    return call("end");
+    return call("create");
 }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t, unsigned long long) {
     const cudaError_t e = call("instantiate");
@@ -62,7 +54,7 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* c) {
 int main(int argc, char** argv) {
     lbm::StepGraphs g;
     int shape[6] = {0, 0, 0, 0, 0, 0}, cur = 0;
-    cudaStream_t stream = U;
+    lbm::GraphRecord* record = nullptr;
     for (int i = 1; i < argc; ++i) {
         const std::string a = argv[i];
         if (a.rfind("shape:", 0) == 0) { shape[1] = atoi(a.c_str() + 6); continue; }
@@ -75,19 +67,18 @@ int main(int argc, char** argv) {
         }
         const long n = atol(argv[i]);
         ran_plain = ran_graph = 0;
-        used["begin"] = used["instantiate"] = used["replay"] = 0;
+        used["create"] = used["instantiate"] = used["replay"] = 0;
         const int start = cur;
-        const cudaError_t e = lbm::run_steps(g, shape, stream, K, cur, n, [&](long k) {
-            if (capturing != (stream == K)) abort();
-            (capturing ? recorded : ran_plain) += k;
+        const cudaError_t e = lbm::run_steps(g, shape, U, record, cur, n, [&](long k) {
+            (record ? recorded : ran_plain) += k;
             cur ^= k & 1;
-            return cudaSuccess;
+            return record ? call("node") : cudaSuccess;
         });
-        if (e != cudaSuccess || stream != U || ran_plain + ran_graph != n || cur != (start ^ (int)(n & 1))) {
+        if (e != cudaSuccess || record || ran_plain + ran_graph != n || cur != (start ^ (int)(n & 1))) {
             printf("wrong\n");
             return 1;
         }
-        printf("%ld/%ld/%d%s ", ran_graph, ran_plain, used["begin"], g.failed ? "F" : "");
+        printf("%ld/%ld/%d%s ", ran_graph, ran_plain, used["create"], g.failed ? "F" : "");
     }
     g.drop(nullptr);
     printf("\n");
@@ -110,7 +101,7 @@ def harness(tmp_path_factory):
     def run(*args):
         p = subprocess.run([str(exe), *[str(a) for a in args]], capture_output=True, text=True, timeout=60)
         assert p.returncode == 0, (args, p.stdout, p.stderr)
-        return p.stdout.split()  # per call: steps replayed / launched singly / captures begun, F once failed
+        return p.stdout.split()  # per call: steps replayed / launched singly / graphs begun, F once failed
 
     return run
 
@@ -122,15 +113,15 @@ def test_long_calls_replay_at_once_and_short_ones_never(harness):
     assert harness(*[15] * 20) == ["0/15/0"] * 20
 
 
-def test_first_short_calls_of_a_context_are_not_captured(harness):
+def test_first_short_calls_of_a_context_make_no_graph(harness):
     assert harness(16) == ["0/16/0"]
     assert harness(16, 16, 16) == ["0/16/0", "16/0/1", "16/0/0"]
     # 31 = 16 + 12 + 3, the buffers in turn
     assert harness(*[31] * 6) == ["0/31/0", "0/31/0", "28/3/2", "28/3/2", "28/3/0", "28/3/0"]
 
 
-@pytest.mark.parametrize("call", ["begin", "end", "instantiate"])
-def test_a_failed_capture_is_not_tried_again(harness, call):
+@pytest.mark.parametrize("call", ["create", "node", "instantiate"])
+def test_a_graph_that_cannot_be_made_is_not_tried_again(harness, call):
     out = harness(f"fail:{call}:-1", 64, f"ok:{call}", 64, 64)
     assert out == ["0/64/1F", "0/64/0F", "0/64/0F"]
     # the graph of 4 steps fails after that of 16 was made
