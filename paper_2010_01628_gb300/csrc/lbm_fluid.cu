@@ -612,11 +612,13 @@ static cudaError_t step_t(lbm_ctx* c, long n, bool dry) {
     const bool reg = c->grid.wall_model == LBM_WALL_REGULARIZED;
     const bool channel = (c->box.periodic & 7u) == 5u && c->box.ny >= 3;
     if (channel && (reg || c->variant == 0)) {
-        // In FP32 the interior numbered through from its first row leaves every warp off
-        // the 32-byte sectors when nx is not a multiple of 8; rows that nearly fill their
-        // warps are then faster (numbered / rows, nx x 128 x 64: 252 1.09, 250 1.06, 500
-        // 1.06, 300 1.05, 127 1.04; 100 0.97, 84 0.92; multiples of 8 0.66 .. 1.00).
-        const bool flat = step_flat(c->box, bx, sizeof(S) == 4 && c->box.nx % 8 != 0 ? 20 : 0);
+        // In FP32 the interior numbered through from node (z ny + 1) nx on leaves every
+        // warp off the 32-byte sectors when nx is not a multiple of 8 and ny is even;
+        // rows that nearly fill their warps are then faster (numbered / rows at ny 130:
+        // nx 252 1.08, 250 1.05, 500 1.09, 300 1.03, 127 1.03; 100 0.97, 84 0.92).  With
+        // odd ny every other plane is on them (ny 129: 0.96 .. 1.00 at every width).
+        const bool off = sizeof(S) == 4 && c->box.nx % 8 != 0 && c->box.ny % 2 == 0;
+        const bool flat = step_flat(c->box, bx, off ? 20 : 0);
         const unsigned inner = (unsigned)(((size_t)c->box.nx * (c->box.ny - 2) + bx - 1) / bx);
         dim3 g = step_grid(c->box, bx, c->box.ny, flat);
         if (flat) g.x = inner + (unsigned)((2 * (size_t)c->box.nx + bx - 1) / bx);
