@@ -196,9 +196,9 @@ __global__ void __launch_bounds__(256, batch_ctas(PHYS, PASS, sizeof(S)))
         fluid_node<S, C, WALLS>(src + D.off, dst + D.off, D.a, x, y, z);
 }
 
-// Diagnostic: a barrier that waits for one CTA more than the grid has, so
-// every wait runs into its (short) limit; used to check that bounded waits
-// end and report LBM_ERR_TIMEOUT.
+// Diagnostic, of use on its own: no step contains a grid barrier.  One that waits
+// for a CTA more than the grid has, so every wait runs into its (short) limit; used
+// to check that bounded waits end and report LBM_ERR_TIMEOUT.
 __global__ void barrier_selftest_kernel(BarrierState* bs, unsigned long long timeout_ns) {
     grid_barrier(bs, gridDim.x + 1, timeout_ns);
 }

@@ -13,7 +13,8 @@ namespace lbm {
 
 // Pass 1: phi and rho_r of every node from its pulled populations.  (The node
 // is found in these two lines and not by plane_node in the row form: that
-// compiled to 43 instead of 44 registers and 17.4 instead of 19.3 GLUPS.)
+// compiled to 43 instead of 44 registers and 17.4 instead of 19.1 GLUPS on the 256^3
+// droplets.)
 template <typename S, typename C, int WALLS, bool FLAT>
 __global__ void __launch_bounds__(256) cgm_phi_kernel(const S* __restrict__ src, C* __restrict__ phi,
                                                       C* __restrict__ rho_red, CgmArgs p, FastDiv div_nx) {

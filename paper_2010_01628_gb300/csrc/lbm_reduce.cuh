@@ -40,8 +40,9 @@ __device__ __forceinline__ void block_reduce_store(RedAcc& a, double* __restrict
 // multiplications (x-rows cut into 256-node chunks, 64-bit divisions per chunk and
 // idle threads past the row's end: 114 us per lbm_reduce at 100^3, now 78 us).
 // They are bound by the FP64 pipe (84 % busy): 9 fused multiply-adds, 7 additions
-// and 7 conversions a node, 16 cycles per warp instruction, 90 us of the 124 us of
-// an lbm_reduce at 128^3; the sums stay in FP64.
+// and 7 conversions a node, 16 cycles per warp instruction, 77 us of the 124 us of
+// an lbm_reduce at 128^3; the sums stay in FP64.  (lbm_reduce_state_noalloc keeps the
+// chunks of a row.)
 struct NodeDiv {
     FastDiv nx, ny;
 };
