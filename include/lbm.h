@@ -223,10 +223,9 @@ lbm_status lbm_batch_create(lbm_ctx **out, int ndomains, const lbm_grid *grids, 
                             lbm_precision precision, void *cuda_stream);
 lbm_status lbm_batch_domain(lbm_ctx *batch, int domain, lbm_ctx **view);
 lbm_status lbm_batch_step(lbm_ctx *batch, long n);
-/* Launch shape of a step: threads per CTA, CTAs, whether calls of 16 and more
- * steps may be replayed from graphs (0 once one could not be made at
- * this shape: steps are then launched one by one), number of tiles (one CTA
- * each). */
+/* Launch shape of a step: threads per CTA, CTAs, whether steps may be replayed
+ * from graphs (0 once one could not be made at this shape: steps are then
+ * launched one by one), number of tiles (one CTA each). */
 lbm_status lbm_batch_info(const lbm_ctx *batch, int *threads, int *grid, int *graph, long *tiles);
 
 /* Diagnostic of the bounded device waits: runs a grid barrier that can never

@@ -16,7 +16,7 @@ namespace lbm {
 // 22.3 us), so steps are replayed 16 at a time and the rest of a call 4 at a time.
 // More steps per graph gain nothing (the stream's gap between two graphs is
 // 0.15 us a step at 16) and make the graph, paid once per context and launch
-// shape, longer to build.  Calls of fewer than 16 steps are launched step by step.
+// shape, longer to build.
 constexpr long STEP_GRAPH[2] = {16, 4};
 // A graph is made once the steps it could have replayed, those of the present
 // call among them, reach these counts: making it costs what it
@@ -92,7 +92,7 @@ template <class Launch>
 cudaError_t run_steps(StepGraphs& g, const int (&shape)[6], cudaStream_t stream, GraphRecord*& record, int& cur,
                       long n, Launch launch) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    bool replay = n >= STEP_GRAPH[0];
+    bool replay = n >= STEP_GRAPH[1];
     if (replay && (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)) {
         cudaGetLastError();
         replay = false;

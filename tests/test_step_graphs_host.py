@@ -106,11 +106,17 @@ def harness(tmp_path_factory):
     return run
 
 
-def test_long_calls_replay_at_once_and_short_ones_never(harness):
+def test_long_calls_replay_at_once(harness):
     assert harness(32) == ["32/0/1"]
     assert harness(100, 100, 100, 100) == ["96/4/1", "96/4/0", "96/4/0", "100/0/1"]
     assert harness(47, 47) == ["32/15/1", "32/15/1"]  # the other buffer is current in the second call
-    assert harness(*[15] * 20) == ["0/15/0"] * 20
+
+
+def test_short_calls_replay_four_steps_at_a_time(harness):
+    assert harness(*[3] * 20) == ["0/3/0"] * 20
+    assert harness(*[4] * 5) == ["0/4/0"] * 3 + ["4/0/1", "4/0/0"]
+    assert harness(*[10] * 4) == ["0/10/0", "8/2/1", "8/2/0", "8/2/0"]
+    assert harness(*[15] * 6) == ["0/15/0"] * 2 + ["12/3/1"] * 2 + ["12/3/0"] * 2  # the buffers in turn
 
 
 def test_first_short_calls_of_a_context_make_no_graph(harness):
